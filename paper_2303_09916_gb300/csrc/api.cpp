@@ -243,7 +243,7 @@ void layout_results(Job* j) {
 // Estimated plan scratch of a job (rescoring arrays and tables).
 uint64_t plan_scratch_estimate(const Job* j) {
   const uint64_t C = (uint64_t)j->params.n_chains;
-  return 4096 + 3 * 8 * C + 8 * C * j->n_atoms * 3 + 64 * C + 16 * C;
+  return 4096 + 3 * 8 * C + C * std::max<uint64_t>(8 * j->n_atoms * 3, kSliceRecordBytes) + 64 * C + 16 * C;
 }
 
 // Device memory, pinned buffer and blob upload of one job on stream st, and

@@ -70,7 +70,7 @@ struct Conf {
 struct WarpScratch {
   float4* pre;     // [kMaxAtoms][2] inclusive prefix sums of (g, (r - p) x g): (gx, gy, gz, cx), (cy, cz, -, -)
   float* H;        // [6 + T][kHStride] BFGS inverse Hessian, row j owned by lane j
-  float* vec;      // [5][kHStride] + 24: g', s, u broadcast to the H rows (BFGS update);
+  float* vec;      // [5][kHStride] + kVarWords: g', s, u broadcast to the H rows (BFGS update);
                    // the chain's g and d; its ChainVars
   float* x;        // [7 + kMaxDim] local optimiser: current iterate (BFGS) / best iterate (BB)
   float* cur;      // [7 + kMaxDim] current conformation of the chain
@@ -78,6 +78,7 @@ struct WarpScratch {
 };
 
 constexpr int kConfFloats = 7 + kMaxDim;
+constexpr int kVarWords = 24;  // words of the scratch's ChainVars
 // Row stride of H (floats): >= kMaxDim rounded up to float4, and 7 float4 per row
 // so that rows j = 0..7 fall on distinct 16-byte bank groups (float4 row reads
 // by the lanes need the minimum number of shared-memory wavefronts).
@@ -88,15 +89,13 @@ __host__ __device__ constexpr int align16i(int x) { return (x + 15) & ~15; }
 struct ScratchLayout {
   int pre, H, vec, x, cur, best, bytes;
 };
-__host__ __device__ inline ScratchLayout scratch_layout(int n_atoms, int n_torsions, int n_pairs, int apl) {
-  (void)n_pairs;
-  (void)apl;
+__host__ __device__ inline ScratchLayout scratch_layout(int n_atoms, int n_torsions) {
   ScratchLayout l;
   const int D = 6 + n_torsions;
   l.pre = 0;
   l.H = l.pre + align16i(32 * n_atoms);
   l.vec = l.H + align16i(4 * kHStride * D);
-  l.x = l.vec + align16i(4 * (5 * kHStride + 24));
+  l.x = l.vec + align16i(4 * (5 * kHStride + kVarWords));
   l.cur = l.x + align16i(4 * kConfFloats);
   l.best = l.cur + align16i(4 * kConfFloats);
   l.bytes = l.best + align16i(4 * kConfFloats);
@@ -525,6 +524,23 @@ __device__ __forceinline__ float3 site_start(const DevJob& J, const ChainStream&
   return make_float3(__ldg(J.sites), __ldg(J.sites + 1), __ldg(J.sites + 2));
 }
 
+// Between two MC steps a chain is its current and best conformations, their
+// energies, the evaluation count and the step number: what a time-sliced launch
+// (dock_chains_kernel) keeps in global memory while another chain has the warp.
+// Another SM may have written it: it is read and written past L1.
+struct ChainRecord {
+  float cur[kConfFloats], best[kConfFloats];
+  float e_cur, e_best;
+  uint32_t evals;
+  uint32_t pad;
+};
+static_assert(sizeof(ChainRecord) <= kSliceRecordBytes, "the plan's scratch holds a record per chain");
+struct ChainSlice {
+  ChainRecord* rec;  // null: the call runs the whole chain
+  int* next_step;    // the step the chain stands at, 0 before its start
+  int steps;         // MC steps of a slice (the start and its optimisation count as one)
+};
+
 // Chain and optimiser variables that wait in shared memory while a
 // conformation is evaluated (read back through volatile loads, so that none of
 // them holds a register during the evaluation).
@@ -534,13 +550,14 @@ struct ChainVars {
   float e_cur, e_best;
   uint32_t evals;
   int T;
-  int bb, max_iters, n_steps;
-  float temperature;
-  float inv_gyr;
-  uint32_t seed_lo, seed_hi, chain;
-  float* trace;
+  int bb, max_iters;
+  int chain;
+  int stop;  // MC step at which this run of the chain ends (n_steps + 1: the chain's end)
+  const DevJob* job;
+  ChainRecord* rec;  // ChainSlice
+  int* next_step;
 };
-static_assert(sizeof(ChainVars) <= 4 * 24, "ChainVars must fit its 24 words of the vec area");
+static_assert(sizeof(ChainVars) <= 4 * kVarWords, "ChainVars must fit its words of the vec area");
 
 // One Monte Carlo chain (Sec. 2: one of many short independent copies; Vina's
 // mutation and Metropolis rules) with its local optimisations -- BFGS with
@@ -553,8 +570,13 @@ static_assert(sizeof(ChainVars) <= 4 * 24, "ChainVars must fit its 24 words of t
 // evaluate.  Only the conformation under evaluation stays in registers across
 // an evaluation; the optimiser's vectors g and d, the chain's scalars and the
 // iterate / current / best conformations wait in shared memory.
-template <int APL, int FMT, int IU = 2>
-__device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& W, int chain) {
+//
+// With a record in `sl`, the call runs one slice from the step the chain stands
+// at and leaves it in the record; without, the whole chain.
+// REVIEW: read the ligand's view from the staged blob at each evaluation instead of
+// holding it in registers (the 96-register kernel of mixed tiles spills otherwise).
+template <int APL, int FMT, int IU = 2, bool REVIEW = false>
+__device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& W, int chain, const ChainSlice& sl) {
   enum : int { kStart = 0, kTrial = 1, kBB = 2 };
   const int lane = threadIdx.x & 31;
   const MapView M = make_map_view(J);
@@ -564,7 +586,40 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
   volatile float* const Vd = W.vec + 4 * kHStride;  // search direction / step
   volatile ChainVars& V = *reinterpret_cast<volatile ChainVars*>(W.vec + 5 * kHStride);
   Conf xt;
+  const int first = sl.rec ? __ldcg(sl.next_step) : 0;
+  if (first > J.n_steps) return;
+  bool mutate = first > 0;  // the next evaluation starts an MC step: mutate the current conformation
   {
+    const int T = L.T;
+    // every lane writes the same values
+    V.phase = kStart;
+    V.it = V.trial = 0;
+    V.e = V.gd = V.e_opt_best = 0.f;
+    V.alpha = 1.f;
+    V.T = T;
+    V.bb = J.optimizer == DSDP_OPT_BB;
+    V.max_iters = J.n_opt_iters;
+    V.chain = chain;
+    V.job = &J;
+    V.step = first;
+    V.stop = sl.rec ? min(first + sl.steps, J.n_steps + 1) : J.n_steps + 1;
+    V.rec = sl.rec;
+    V.next_step = sl.next_step;
+    if (lane < kHStride) Vg[lane] = Vd[lane] = 0.f;
+    if (mutate) {
+      if (lane < 7 + T) {
+        W.cur[lane] = __ldcg(sl.rec->cur + lane);
+        W.best[lane] = __ldcg(sl.rec->best + lane);
+      }
+      V.e_cur = __ldcg(&sl.rec->e_cur);
+      V.e_best = __ldcg(&sl.rec->e_best);
+      V.evals = __ldcg(&sl.rec->evals);
+    } else {
+      V.e_cur = V.e_best = 0.f;
+      V.evals = 0;
+    }
+  }
+  if (!mutate) {
     const int T = L.T;
     const ChainStream rs{J.seed_lo, J.seed_hi, (uint32_t)chain};
     // initial conformation: uniform word n of step 0 is word n % 4 of block n / 4
@@ -586,23 +641,6 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       th = kPiF - kTwoPiF * ChainStream::to_uniform(pick(bk, lane & 3));
     }
     xt.th = th;
-    // every lane writes the same values
-    V.phase = kStart;
-    V.it = V.trial = V.step = 0;
-    V.e = V.gd = V.e_opt_best = V.e_cur = V.e_best = 0.f;
-    V.alpha = 1.f;
-    V.evals = 0;
-    V.T = T;
-    V.bb = J.optimizer == DSDP_OPT_BB;
-    V.max_iters = J.n_opt_iters;
-    V.n_steps = J.n_steps;
-    V.temperature = J.temperature;
-    V.inv_gyr = 1.f / L.h->gyration_radius;
-    V.seed_lo = J.seed_lo;
-    V.seed_hi = J.seed_hi;
-    V.chain = (uint32_t)chain;
-    V.trace = J.trace ? J.trace + (size_t)chain * (J.n_steps + 1) * ((size_t)7 + T + 4) : nullptr;
-    if (lane < kHStride) Vg[lane] = Vd[lane] = 0.f;
     if (J.trace && J.trace_starts) {  // row 0: the drawn start, before any optimisation
       float* t = J.trace + (size_t)chain * (J.n_steps + 1) * ((size_t)7 + T + 4);
       store_conf(t, xt, T);
@@ -613,11 +651,33 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         t[7 + T + 3] = 0.f;
       }
     }
-    __syncwarp();
   }
+  __syncwarp();
   for (;;) {
+    if (__builtin_expect(mutate, 0)) {  // once per MC step: kept out of the evaluations' way
+      // ---- mutation of the current conformation (the next local optimisation's start)
+      const int T = V.T;
+      const uint32_t step = (uint32_t)V.step;
+      const DevJob& job = *V.job;
+      const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)V.chain};
+      const uint4 w0 = rs.block(step, 0);
+      const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
+      xt = load_conf(W.cur, T);
+      if (mode == 0) {
+        const float3 b = unit_ball(rs, step);
+        xt.p = xt.p + kMutationAmplitude * b;
+      } else if (mode == 1) {
+        const float3 b = unit_ball(rs, step);
+        const float k = kMutationAmplitude * (1.f / L.h->gyration_radius);
+        xt.q = qnormalize(qmul(quat_from_rotvec(k * b.x, k * b.y, k * b.z), xt.q));
+      } else if (lane == 6 + (mode - 2)) {
+        xt.th = kPiF - kTwoPiF * ChainStream::to_uniform(w0.z);
+      }
+      mutate = false;
+    }
     float gn;
-    const float en = eval_conf<APL, FMT, IU>(M, L, R, W, xt, gn, DSDP_TERM_ALL);
+    const float en = eval_conf<APL, FMT, IU>(M, REVIEW ? view_blob(reinterpret_cast<const uint8_t*>(L.h)) : L, R, W,
+                                             xt, gn, DSDP_TERM_ALL);
     const int T = V.T, nx = 7 + T, D = 6 + T;
     const bool bb = V.bb;
     const int max_iters = V.max_iters;
@@ -688,12 +748,15 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         xt = apply_step(xt, dir, T);
       }
     }
-    if (done) {
+    if (__builtin_expect(done, 0)) {
       // ---- local optimisation finished: its result is W.x with energy eo
       const float eo = (bb && max_iters > 0) ? e_opt_best : e;
-      const ChainStream rs{V.seed_lo, V.seed_hi, V.chain};
-      float* const trace = V.trace;
+      // (the job record is read again here rather than held across the evaluations)
+      const DevJob& job = *V.job;
+      const int chain_id = V.chain;
+      const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)chain_id};
       const size_t trace_stride = (size_t)nx + 4;
+      float* const trace = job.trace ? job.trace + (size_t)chain_id * (job.n_steps + 1) * trace_stride : nullptr;
       int step = V.step;
       float e_cur = V.e_cur, e_best = V.e_best;
       __syncwarp();
@@ -703,7 +766,7 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
           W.cur[lane] = W.x[lane];
           W.best[lane] = W.x[lane];
         }
-        if (trace && !J.trace_starts) {
+        if (trace && !job.trace_starts) {
           if (lane < nx) trace[lane] = W.x[lane];
           if (lane == 0) {
             trace[nx + 0] = e_cur;
@@ -716,7 +779,7 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         const uint4 w0 = rs.block((uint32_t)step, 0);
         const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
         const float u = ChainStream::to_uniform(w0.y);
-        const bool accept = (eo < e_cur) || (u < expf(-(eo - e_cur) / V.temperature));
+        const bool accept = (eo < e_cur) || (u < expf(-(eo - e_cur) / job.temperature));
         if (accept) {
           e_cur = eo;
           if (lane < nx) W.cur[lane] = W.x[lane];
@@ -737,29 +800,32 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         }
       }
       __syncwarp();
-      if (++step > V.n_steps) {
-        if (lane < nx) J.chain_best_conf[(size_t)chain * nx + lane] = W.best[lane];
+      if (++step > job.n_steps) {
+        if (lane < nx) job.chain_best_conf[(size_t)chain_id * nx + lane] = W.best[lane];
         if (lane == 0) {
-          J.chain_best_e[chain] = e_best;
-          J.chain_evals[chain] = evals;
+          job.chain_best_e[chain_id] = e_best;
+          job.chain_evals[chain_id] = evals;
+          if (V.rec) __stcg(V.next_step, step);  // a further slice finds nothing left
         }
         __syncwarp();
         return;
       }
-      // ---- mutation of the current conformation (the next local optimisation's start)
-      const uint4 w0 = rs.block((uint32_t)step, 0);
-      const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
-      xt = load_conf(W.cur, T);
-      if (mode == 0) {
-        const float3 b = unit_ball(rs, (uint32_t)step);
-        xt.p = xt.p + kMutationAmplitude * b;
-      } else if (mode == 1) {
-        const float3 b = unit_ball(rs, (uint32_t)step);
-        const float k = kMutationAmplitude * V.inv_gyr;
-        xt.q = qnormalize(qmul(quat_from_rotvec(k * b.x, k * b.y, k * b.z), xt.q));
-      } else if (lane == 6 + (mode - 2)) {
-        xt.th = kPiF - kTwoPiF * ChainStream::to_uniform(w0.z);
+      if (step == V.stop) {  // end of this slice: the chain waits in its record
+        ChainRecord* const rec = V.rec;
+        if (lane < nx) {
+          __stcg(rec->cur + lane, W.cur[lane]);
+          __stcg(rec->best + lane, W.best[lane]);
+        }
+        if (lane == 0) {
+          __stcg(&rec->e_cur, e_cur);
+          __stcg(&rec->e_best, e_best);
+          __stcg(&rec->evals, evals);
+          __stcg(V.next_step, step);
+        }
+        __syncwarp();
+        return;
       }
+      mutate = true;
       phase = kStart;
       V.step = step;
       V.e_cur = e_cur;

@@ -42,7 +42,7 @@ struct ChainOcc<3> {
 // each): the bound changes how the compiler schedules, not the register count.
 template <int VAR, int APLS>
 __host__ __device__ constexpr int chain_min_blocks() {
-  return (VAR == 1 && APLS == 1) ? 0 : ChainOcc<VAR>::kMinBlocks;
+  return ChainOcc<VAR>::kMinBlocks;
 }
 
 // Chains: a CTA runs one tile of up to W chains of one job; W = blockDim / 32.
@@ -51,27 +51,67 @@ __host__ __device__ constexpr int chain_min_blocks() {
 // launch holds (a chain's arithmetic depends on its own job only).  APLS: the
 // tiles compiled in (1 or 2; 3 = both, for launches that mix them -- each
 // single-tile kernel keeps its register allocation to itself).
-// persistent != 0: CTAs pull tiles from *tile_counter until none are left.
+// n_items = 0: CTA b runs tile b.  Else the CTAs pull items from a work queue
+// until none are left: item i is tile i (n_blocks = 0), or, time-sliced, one
+// slice of a tile (the blocks say which).
+//
+// Why slices: a chain's length (evaluations until its last local optimisation
+// ends) varies by a factor of two around the mean and is not known before.  Run
+// to the end one after the other, the long chains that start last leave most SMs
+// idle: 6,144 typical-4k chains kept an SM busy for 72 % of the launch (37.1 ms;
+// 29.4 sliced).  In slices every chain starts early, and a slow one never waits:
+// an item of a tile that is still running is left to the CTA that runs it
+// (tickets), which goes on with the tile's next slice.  The slices come in the
+// order of the work that their chains have left, most first (plan_tiles).
+struct ChainQueue {
+  int* counter;              // the next item
+  int* tickets;              // [n_tiles] items taken and not finished
+  int* next_step;            // [n_tiles][W] the step each chain stands at
+  const SliceBlock* blocks;  // by item_begin
+  int n_blocks, n_items;
+};
+
+// The next tile for this CTA, n_tiles when none is left (one thread).  The first
+// taker of an idle tile runs it; an item of a running tile stays with its CTA.
+static __device__ __noinline__ int queue_next(const ChainQueue& q, int n_tiles) {
+  for (;;) {
+    const int item = atomicAdd(q.counter, 1);
+    if (item >= q.n_items) return n_tiles;
+    int t = item;
+    if (q.n_blocks) {
+      int lo = 0, hi = q.n_blocks;  // blocks[lo].item_begin <= item < blocks[hi].item_begin
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(&q.blocks[mid].item_begin) <= item) lo = mid;
+        else hi = mid;
+      }
+      t = __ldg(&q.blocks[lo].tile_begin) + item - __ldg(&q.blocks[lo].item_begin);
+    }
+    if (atomicAdd(q.tickets + t, 1) == 0) {
+      __threadfence();  // the records of the tile's last slice, written before its ticket was given back
+      return t;
+    }
+  }
+}
+
 template <int FMT, int VAR, int APLS>
 __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>())) dock_chains_kernel(const DevJob* __restrict__ jobs,
                                                           const Tile* __restrict__ tiles, int n_tiles,
-                                                          int* tile_counter, int persistent, int blob_smem,
-                                                          ScratchLayout lay) {
+                                                          ChainQueue queue, int blob_smem, ScratchLayout lay) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int s_tile;
   __shared__ int s_job;
   const int warp = threadIdx.x >> 5;
-  const WarpScratch W = warp_scratch_at(smem + blob_smem + warp * lay.bytes, lay);
-  if (threadIdx.x == 0) s_job = -1;
+  // the plan's next group of chains depends on nothing here: its CTAs may take
+  // the places this launch's CTAs leave (no effect without such a launch)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (threadIdx.x == 0) {
+    s_job = -1;
+    s_tile = queue.n_items ? queue_next(queue, n_tiles) : (int)blockIdx.x;
+  }
   __syncthreads();
-  int t = blockIdx.x;
   for (;;) {
-    if (persistent) {
-      __syncthreads();
-      if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1);
-      __syncthreads();
-      t = s_tile;
-    }
+    const int t = s_tile;
     if (t >= n_tiles) break;
     const Tile tile = tiles[t];
     const DevJob& J = jobs[tile.job];
@@ -82,15 +122,32 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
         reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(J.blob) + i);
       __syncthreads();
       if (threadIdx.x == 0) s_job = tile.job;
-      __syncthreads();
     }
-    const LigView L = view_blob(smem);
     if (warp < tile.count) {
-      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, APLS == 3 ? 1 : 2>(J, L, W, tile.chain0 + warp);
-      else run_chain<2, FMT>(J, L, W, tile.chain0 + warp);
+      const WarpScratch W = warp_scratch_at(smem + blob_smem + warp * lay.bytes, lay);
+      const LigView L = view_blob(smem);
+      const int chain = tile.chain0 + warp;
+      ChainSlice sl{nullptr, nullptr, 0};
+      if (queue.n_blocks) {
+        sl.rec = reinterpret_cast<ChainRecord*>(reinterpret_cast<uint8_t*>(J.chain_coords) +
+                                                (size_t)chain * kSliceRecordBytes);
+        sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
+        sl.steps = J.slice_steps;
+      }
+      constexpr bool kReview = APLS == 3 && VAR == 1;
+      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, APLS == 3 ? 1 : 2, kReview>(J, L, W, chain, sl);
+      else run_chain<2, FMT, 2, kReview>(J, L, W, chain, sl);
     }
-    if (!persistent) break;
+    if (!queue.n_items) break;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();  // this slice's records, before the ticket is given back
+      if (atomicSub(queue.tickets + s_tile, 1) == 1) s_tile = queue_next(queue, n_tiles);
+    }
+    __syncthreads();
   }
+  // what follows on the stream follows this launch: it ends after the group before it
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Score + gradient of a batch of conformations: one warp per conformation,
@@ -129,19 +186,35 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   auto k = dock_chains_kernel<FMT, VAR, APLS>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int grid = a.grid;
-  if (a.persistent) {
+  int grid = a.n_tiles;
+  ChainQueue q{a.counter, a.tickets, a.next_step, a.blocks, 0, 0};
+  if (a.queue != kNoQueue) {
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * a.warps_per_cta, smem);
     if (e != cudaSuccess) return e;
-    grid = per_sm * sms < a.n_tiles ? per_sm * sms : a.n_tiles;
-    if (grid < 1) grid = 1;
+    const int slots = per_sm * sms > 1 ? per_sm * sms : 1;
+    if (a.n_tiles > slots) {
+      grid = slots;
+      q.n_blocks = a.n_blocks;
+      q.n_items = a.n_items;
+    } else if (a.queue == kQueue) {
+      q.n_items = a.n_tiles;  // every tile has a slot of its own: nothing to slice
+    }
   }
-  k<<<grid, block, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs), reinterpret_cast<const Tile*>(a.tiles),
-                               a.n_tiles, a.tile_counter, a.persistent, a.blob_smem, a.scratch);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = a.overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, reinterpret_cast<const DevJob*>(a.jobs), reinterpret_cast<const Tile*>(a.tiles),
+                            a.n_tiles, q, a.blob_smem, a.scratch);
 }
 
 template <int FMT>

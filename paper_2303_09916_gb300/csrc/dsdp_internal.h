@@ -97,6 +97,7 @@ struct DevJob {
   const float* sites;  // adaptive search space: [n_sites][3] predicted binding-site points
   int32_t n_sites;     // 0: initial positions uniform in the box
   float site_r2;       // site radius squared (FP32)
+  int32_t slice_steps;  // MC steps of a slice in a time-sliced launch
   float* chain_best_conf;
   float* chain_best_e;
   uint32_t* chain_evals;
@@ -121,11 +122,22 @@ struct DevJob {
   float* out_coords;
 };
 
+// Bytes of a chain's record in a time-sliced launch (ChainRecord, chain_device.cuh).
+// The records share the rescoring's coordinate scratch (24 n_atoms bytes per
+// chain), which is not in use while the chains run.
+constexpr int kSliceRecordBytes = 8 * (7 + kMaxDim) + 16;
+
 struct Tile {
   int32_t job;
   int32_t chain0;
   int32_t count;
   int32_t pad;
+};
+
+// Consecutive items of a time-sliced launch's queue: one slice of each of a job's tiles.
+struct SliceBlock {
+  int32_t item_begin;
+  int32_t tile_begin;
 };
 
 // Vina constants of the kernels (the scoring function DSDP keeps, Sec. 2).

@@ -9,6 +9,8 @@
 
 #include "launch.h"
 
+constexpr int kMaxGroups = 12;  // map formats x atoms per lane
+
 struct dsdp_plan {
   dsdp_ctx* ctx = nullptr;
   int n_jobs = 0;
@@ -21,15 +23,28 @@ struct dsdp_plan {
   void* arena = nullptr;
   size_t arena_bytes = 0;
   struct Group {
-    int fmt, apl, first_tile, n_tiles, blob_smem, max_atoms, max_torsions, max_pairs, apl_mask;
+    int fmt, apl, first_tile, n_tiles, blob_smem, max_atoms, max_torsions, apl_mask;
+    int first_block, n_blocks, n_items;  // time-sliced queue (SliceBlock)
   };
   std::vector<Group> groups;
   void* d_jobs = nullptr;
   void* d_tiles = nullptr;
   void* d_rtiles = nullptr;
-  int* d_counters = nullptr;
+  // work queue: [kMaxGroups counters, one per group][tickets per tile][next step per tile and warp]; zeroed by each launch
+  int* d_queue = nullptr;
+  size_t queue_bytes = 0;
+  size_t queue_next_off = 0;  // of the next steps, in ints
+  bool auto_queue = false;    // no fixed choice: queue when a group has more tiles than fit at once
+  void* d_blocks = nullptr;
   int n_rtiles = 0;
-  std::vector<int> job_fmt, job_chains;  // to lay chain tiles out again for another warps_per_cta
+  // per job, to lay groups and tiles out again for another configuration
+  struct Shape {
+    int fmt, apl, blob, atoms, torsions, chains;
+    double cost;  // length of a chain, relative
+    int slices;   // of each of its chains
+  };
+  std::vector<Shape> shape;
+  std::vector<int> job_order;  // jobs by chain length, longest first
   int sms = 148;
 };
 
@@ -101,6 +116,12 @@ static dsdp_status check_view(const dsdp_grid_view* g) {
 
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// A job's coordinate scratch: FP64 coordinates while rescoring, the chains' records
+// (ChainRecord) while a time-sliced launch runs them.
+static size_t coord_bytes(int n_chains, int n_atoms) {
+  return (size_t)n_chains * std::max(sizeof(double) * 3 * n_atoms, (size_t)kSliceRecordBytes);
+}
+
 // Autotuner choices by plan shape: (format mask, atoms-per-lane, log2 of the
 // chain count) -> (variant, persistent).  Written by dsdp_plan_autotune, read
 // by plans created with tile_config 0.
@@ -141,27 +162,77 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
   g_tune.push_back(TuneEntry{key, variant, persistent, warps});
 }
 
-// Chain tiles of W chains of one job, grouped by map format (one launch per
-// format present); fills each group's tile range.
-static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles) {
+// Slices of the launch's longest chains when it time-slices (ChainQueue): enough
+// that the last slices are a small part of the launch, few enough that a slice
+// (a few MC steps, hundreds of evaluations) hides its record's load and store.
+constexpr int kSliceRounds = 16;
+
+static ChainQueueMode queue_mode(const dsdp_plan* P) {
+  return (P->flags & DSDP_PLAN_PERSISTENT) ? kQueue : P->auto_queue ? kQueueIfMany : kNoQueue;
+}
+
+// Chain tiles of W chains of one job in groups of one launch each, and the items
+// of a time-sliced launch.  A fixed configuration has one group per map format
+// (the kernel that holds both tiles when it mixes them).  With the queue the
+// ligands of up to and above 32 atoms are groups of their own: each runs its own
+// kernel with its own shared memory (22 KB a chain at 60 atoms, 8 KB at 30), and
+// the next group's CTAs start as the last one's leave (launch_chains_var).
+// Jobs whose chains take longest come first (what starts last decides how long
+// the launch's tail is), and of the slices those whose chains have the most work
+// left, a job's slices side by side.
+static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vector<SliceBlock>& blocks) {
   tiles.clear();
-  for (dsdp_plan::Group& g : P->groups) {
-    g.first_tile = (int)tiles.size();
-    for (int j = 0; j < P->n_jobs; ++j) {
-      if (P->job_fmt[j] != g.fmt) continue;
-      for (int c = 0; c < P->job_chains[j]; c += W)
-        tiles.push_back(Tile{j, c, std::min(W, P->job_chains[j] - c), 0});
+  blocks.clear();
+  P->groups.clear();
+  const bool split = queue_mode(P) != kNoQueue;
+  struct Item {
+    double left;
+    int tile, n;
+  };
+  std::vector<Item> items;
+  for (int f = 0; f < 6; ++f)
+    for (int apl = split ? 2 : 0; apl >= (split ? 1 : 0); --apl) {  // 0: both
+      dsdp_plan::Group g{};
+      g.fmt = f;
+      g.first_tile = (int)tiles.size();
+      items.clear();
+      for (int j : P->job_order) {
+        const dsdp_plan::Shape& s = P->shape[j];
+        if (s.fmt != f || (apl && s.apl != apl)) continue;
+        g.apl = std::max(g.apl, s.apl);
+        g.apl_mask |= s.apl;
+        g.blob_smem = std::max(g.blob_smem, s.blob);
+        g.max_atoms = std::max(g.max_atoms, s.atoms);
+        g.max_torsions = std::max(g.max_torsions, s.torsions);
+        const int first = (int)tiles.size() - g.first_tile;
+        for (int c = 0; c < s.chains; c += W) tiles.push_back(Tile{j, c, std::min(W, s.chains - c), 0});
+        const int n = (int)tiles.size() - g.first_tile - first;
+        for (int r = 0; r < s.slices; ++r) items.push_back(Item{s.cost * (s.slices - r) / s.slices, first, n});
+      }
+      g.n_tiles = (int)tiles.size() - g.first_tile;
+      if (!g.n_tiles) continue;
+      std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.left > b.left; });
+      g.first_block = (int)blocks.size();
+      for (const Item& it : items) {
+        blocks.push_back(SliceBlock{g.n_items, it.tile});
+        g.n_items += it.n;
+      }
+      g.n_blocks = (int)blocks.size() - g.first_block;
+      P->groups.push_back(g);
     }
-    g.n_tiles = (int)tiles.size() - g.first_tile;
-  }
 }
 
 static cudaError_t plan_use_warps(dsdp_plan* P, int W) {
   std::vector<Tile> tiles;
-  plan_tiles(P, W, tiles);
+  std::vector<SliceBlock> blocks;
+  plan_tiles(P, W, tiles, blocks);
   P->warps_per_cta = W;
-  return tiles.empty() ? cudaSuccess
-                       : cudaMemcpy(P->d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaSuccess;
+  if (!tiles.empty())
+    e = cudaMemcpy(P->d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !blocks.empty())
+    e = cudaMemcpy(P->d_blocks, blocks.data(), sizeof(SliceBlock) * blocks.size(), cudaMemcpyHostToDevice);
+  return e;
 }
 
 }  // namespace dsdp
@@ -190,7 +261,7 @@ extern "C" dsdp_status dsdp_score_eval_device(const dsdp_grid_view* grid, const 
   a.flags = flags;
   a.apl = n_atoms <= 32 ? 1 : 2;
   a.blob_smem = (int)((const BlobHeader*)h_blob)->stage_bytes;
-  a.scratch = scratch_layout(n_atoms, T, P, a.apl);
+  a.scratch = scratch_layout(n_atoms, T);
   return check_cuda(launch_score_dispatch(map_fmt(grid->dtype, grid->mode), a, (cudaStream_t)stream),
                     "score_eval_kernel launch");
 }
@@ -232,7 +303,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     if (!J.d_chain_best_e) scratch += up256(sizeof(float) * (size_t)p.n_chains);
     if (!J.d_chain_evals) scratch += up256(sizeof(uint32_t) * (size_t)p.n_chains);
     scratch += 3 * up256(sizeof(double) * (size_t)p.n_chains);
-    scratch += up256(sizeof(double) * (size_t)p.n_chains * atoms[j] * 3);
+    scratch += up256(coord_bytes(p.n_chains, atoms[j]));
     DevJob& d = dj[j];
     memset(&d, 0, sizeof(d));
     d.blob = (const uint8_t*)J.d_blob;
@@ -281,79 +352,94 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   P->flags = flags;
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
-  // Groups by map format (one launch per format present); a CTA runs a tile of
-  // W chains of one job (W = warps per CTA: 1, 2 or 4), staging the ligand once.
-  P->job_fmt = fmt;
-  P->job_chains.resize(n_jobs);
-  size_t total_chains = 0;
-  for (int j = 0; j < n_jobs; ++j) total_chains += (size_t)(P->job_chains[j] = dj[j].n_chains);
-  for (int f = 0; f < 6; ++f) {
-    dsdp_plan::Group g{f, 1, 0, 0, 0, 0, 0, 0, 0};
-    bool any = false;
+  size_t total_chains = 0, max_blocks = 0;
+  {
+    // Length of a job's chains, relative: evaluations (MC steps; Barzilai-Borwein
+    // runs all its iterations, BFGS about 60 of 100) times the cost of one (the
+    // intra pair steps are half of a 30-atom evaluation, the rest does not depend
+    // on the ligand much beyond its tile).
+    double longest = 1e-9;
+    P->shape.resize(n_jobs);
     for (int j = 0; j < n_jobs; ++j) {
-      if (fmt[j] != f) continue;
-      any = true;
-      g.apl = std::max(g.apl, apl[j]);  // largest tile present: part of the autotuner key
-      g.apl_mask |= apl[j];             // each job runs at its own tile (see dock_chains_kernel)
-      g.blob_smem = std::max(g.blob_smem, blob_bytes[j]);
-      g.max_atoms = std::max(g.max_atoms, atoms[j]);
-      g.max_torsions = std::max(g.max_torsions, tors[j]);
-      g.max_pairs = std::max(g.max_pairs, pairs[j]);
+      const BlobHeader* h = (const BlobHeader*)jobs[j].h_blob;
+      const double cost = (dj[j].n_steps + 1.0) * (dj[j].optimizer == DSDP_OPT_BB ? 1.6 : 1.0) *
+                          (dj[j].n_opt_iters + 1.0) * (14.0 * apl[j] + h->n_steps);
+      P->shape[j] = dsdp_plan::Shape{fmt[j], apl[j], blob_bytes[j], atoms[j], tors[j], dj[j].n_chains, cost, 0};
+      longest = std::max(longest, cost);
+      total_chains += (size_t)dj[j].n_chains;
     }
-    if (any) P->groups.push_back(g);
+    P->job_order.resize(n_jobs);
+    for (int j = 0; j < n_jobs; ++j) {
+      P->job_order[j] = j;
+      // slices of about the same length whatever the job
+      const int steps = dj[j].n_steps + 1, want = (int)ceil(kSliceRounds * P->shape[j].cost / longest);
+      dj[j].slice_steps = (steps + want - 1) / want;
+      P->shape[j].slices = (steps + dj[j].slice_steps - 1) / dj[j].slice_steps;
+      max_blocks += P->shape[j].slices;
+    }
+    std::stable_sort(P->job_order.begin(), P->job_order.end(),
+                     [&](int a, int b) { return P->shape[a].cost > P->shape[b].cost; });
   }
   int W = 1;
   {
     uint32_t fmt_mask = 0;
     int apl_max = 1;
-    for (const dsdp_plan::Group& g : P->groups) {
+    for (const dsdp_plan::Shape& g : P->shape) {
       fmt_mask |= 1u << g.fmt;
       apl_max = std::max(apl_max, g.apl);
     }
     P->tune_key = tune_key(fmt_mask, apl_max, total_chains);
     int var = 0, pers = (flags & DSDP_PLAN_PERSISTENT) ? 1 : 0;
     if (tile_config == 0) {
-      // without a recorded choice: the 96-register kernel for plans of at least
-      // two waves of 16 chains per SM, whose 20 resident warps per SM then issue
-      // more per cycle (32 typical-4k systems 69.0 against 72.4 ms per launch at
-      // 1 chain per CTA; the uneven 10-60-atom batch 307 - 309 against 317 - 319
-      // ms at 4), else the 128-register kernel, whose fewer instructions per
-      // evaluation win when the chains run latency-bound on a part-filled GPU
-      // (one typical-4k system 17.3 against 19.1 ms; 32 plain-2k systems of 64
-      // chains 1,011 against 938 systems/s).  Ligands above 32 atoms stage large
-      // blobs, which tiles of 4 chains share (measured faster on mixed
-      // batches); else 1 chain.
-      var = total_chains >= (size_t)(2 * 16 * P->sms) ? 1 : 0;
-      W = apl_max == 2 ? 4 : 1;
-      if (tune_lookup(P->tune_key, &var, &pers, &W) && pers) P->flags |= DSDP_PLAN_PERSISTENT;
+      // Without a recorded choice, by what is resident at 16 warps per SM (128
+      // registers).  Up to one such wave every chain has a place at once: no queue,
+      // and ligands above 32 atoms, whose staged blobs are large, in tiles of 4
+      // chains.  More chains: the time-sliced queue, one chain per CTA (64 ligands
+      // of 10-60 atoms x 128 chains 71 ms, in tiles of 2 and 4 72 - 77 ms; 16
+      // typical-4k systems 29.6 against 31.0 and 33 ms).  From two waves on the
+      // 96-register kernel, whose 20 resident warps per SM issue more per cycle (16
+      // typical-4k systems 29.6 against 31.0 ms), below the 128-register kernel,
+      // whose fewer instructions per evaluation win on a part-filled GPU (one
+      // typical-4k system 17.3 against 19.1 ms).
+      const size_t wave = (size_t)16 * P->sms;
+      var = total_chains >= 2 * wave ? 1 : 0;
+      const bool many = total_chains > wave;
+      W = apl_max == 2 && !many ? 4 : 1;
+      if (tune_lookup(P->tune_key, &var, &pers, &W)) {
+        if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
+      } else {
+        P->auto_queue = many;
+      }
     } else {
       var = (tile_config - 1) % 4;
       W = 1 << ((tile_config - 1) / 4);
     }
     P->variant = var;
   }
-  std::vector<Tile> tiles;
-  plan_tiles(P, W, tiles);
-  P->warps_per_cta = W;
   std::vector<Tile> rtiles;
   const int rw = rescore_tile_chains();
   for (int j = 0; j < n_jobs; ++j)
     for (int c = 0; c < dj[j].n_chains; c += rw) rtiles.push_back(Tile{j, c, std::min(rw, dj[j].n_chains - c), 0});
   P->n_rtiles = (int)rtiles.size();
   const size_t b_jobs = up256(sizeof(DevJob) * n_jobs), b_tiles = up256(sizeof(Tile) * total_chains),
-               b_rtiles = up256(sizeof(Tile) * rtiles.size()), b_cnt = up256(sizeof(int) * 8);
-  P->arena_bytes = b_jobs + b_tiles + b_rtiles + b_cnt + scratch;
+               b_rtiles = up256(sizeof(Tile) * rtiles.size()), b_blocks = up256(sizeof(SliceBlock) * max_blocks);
+  P->queue_next_off = kMaxGroups + total_chains;
+  P->queue_bytes = sizeof(int) * (kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);  // tiles of W <= 4 may be part filled
+  const size_t b_cnt = up256(P->queue_bytes);
+  P->arena_bytes = b_jobs + b_tiles + b_rtiles + b_blocks + b_cnt + scratch;
   P->arena = ctx_alloc(ctx, P->arena_bytes, nullptr);
   if (!P->arena) {
+    const size_t bytes = P->arena_bytes;
     delete P;
-    return set_error(DSDP_ERR_OUT_OF_MEMORY, "plan arena of %zu bytes", (size_t)(b_jobs + b_tiles + b_rtiles + scratch));
+    return set_error(DSDP_ERR_OUT_OF_MEMORY, "plan arena of %zu bytes", bytes);
   }
   uint8_t* a = (uint8_t*)P->arena;
   P->d_jobs = a;
   P->d_tiles = a + b_jobs;
   P->d_rtiles = a + b_jobs + b_tiles;
-  P->d_counters = (int*)(a + b_jobs + b_tiles + b_rtiles);
-  uint8_t* sc = a + b_jobs + b_tiles + b_rtiles + b_cnt;
+  P->d_blocks = a + b_jobs + b_tiles + b_rtiles;
+  P->d_queue = (int*)(a + b_jobs + b_tiles + b_rtiles + b_blocks);
+  uint8_t* sc = a + b_jobs + b_tiles + b_rtiles + b_blocks + b_cnt;
   for (int j = 0; j < n_jobs; ++j) {
     DevJob& d = dj[j];
     const int nx = 7 + tors[j];
@@ -368,11 +454,10 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     d.chain_score = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_inter = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_intra = (double*)take(sizeof(double) * (size_t)d.n_chains);
-    d.chain_coords = (double*)take(sizeof(double) * (size_t)d.n_chains * atoms[j] * 3);
+    d.chain_coords = (double*)take(coord_bytes(d.n_chains, atoms[j]));
   }
   cudaError_t e = cudaMemcpy(P->d_jobs, dj.data(), sizeof(DevJob) * n_jobs, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && !tiles.empty())
-    e = cudaMemcpy(P->d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = plan_use_warps(P, W);
   if (e == cudaSuccess && !rtiles.empty())
     e = cudaMemcpy(P->d_rtiles, rtiles.data(), sizeof(Tile) * rtiles.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -395,10 +480,10 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
   if (!P) return set_error(DSDP_ERR_INVALID_ARG, "plan is NULL");
   if (stages == 0 || (stages & ~(uint32_t)DSDP_STAGE_ALL)) return set_error(DSDP_ERR_INVALID_ARG, "bad stages");
   const cudaStream_t st = (cudaStream_t)stream;
-  const bool persistent = (P->flags & DSDP_PLAN_PERSISTENT) != 0;
-  if ((stages & DSDP_STAGE_CHAINS) && persistent) {
-    cudaError_t e = cudaMemsetAsync(P->d_counters, 0, sizeof(int) * 8, st);
-    if (e != cudaSuccess) return check_cuda(e, "plan counter reset");
+  const ChainQueueMode queue = queue_mode(P);
+  if ((stages & DSDP_STAGE_CHAINS) && queue != kNoQueue) {
+    const cudaError_t e = cudaMemsetAsync(P->d_queue, 0, P->queue_bytes, st);
+    if (e != cudaSuccess) return check_cuda(e, "plan queue reset");
   }
   for (size_t gi = 0; (stages & DSDP_STAGE_CHAINS) && gi < P->groups.size(); ++gi) {
     const dsdp_plan::Group& g = P->groups[gi];
@@ -406,15 +491,20 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.jobs = P->d_jobs;
     a.tiles = (const Tile*)P->d_tiles + g.first_tile;
     a.n_tiles = g.n_tiles;
-    a.tile_counter = P->d_counters + gi;
-    a.persistent = persistent ? 1 : 0;
+    a.queue = queue;
+    a.counter = P->d_queue + gi;
+    a.tickets = P->d_queue + kMaxGroups + g.first_tile;
+    a.next_step = P->d_queue + P->queue_next_off + (size_t)g.first_tile * P->warps_per_cta;
+    a.blocks = (const SliceBlock*)P->d_blocks + g.first_block;
+    a.n_blocks = g.n_blocks;
+    a.n_items = g.n_items;
     a.warps_per_cta = P->warps_per_cta;
     a.apl = g.apl;
     a.apl_mask = g.apl_mask;
     a.blob_smem = (g.blob_smem + 15) & ~15;
-    a.scratch = scratch_layout(g.max_atoms, g.max_torsions, g.max_pairs, g.apl);
+    a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
+    a.overlap = gi > 0 && queue != kNoQueue;
     a.variant = P->variant;
-    a.grid = g.n_tiles;  // a persistent launch sizes its grid from the occupancy
     cudaError_t e = launch_chains_dispatch(g.fmt, a, st);
     if (e != cudaSuccess) return check_cuda(e, "dock_chains_kernel launch");
   }
@@ -443,6 +533,7 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e != cudaSuccess) return check_cuda(e, "autotune events");
   const uint32_t base_flags = P->flags & ~(uint32_t)DSDP_PLAN_PERSISTENT;
+  P->auto_queue = false;  // with and without the queue are measured apart
   float best = 1e30f;
   int best_var = P->variant, best_pers = (P->flags & DSDP_PLAN_PERSISTENT) ? 1 : 0, best_w = P->warps_per_cta;
   dsdp_status s = DSDP_OK;
@@ -450,16 +541,16 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   // 96 for two and for mixed tiles (launch_chains_impl)
   int n_var = 2;
   for (const dsdp_plan::Group& g : P->groups) n_var = std::max(n_var, g.apl_mask == 1 ? 4 : 2);
-  for (int w = 1; w <= 4 && s == DSDP_OK; w *= 2) {
+  for (int w = 1; w <= 4 && s == DSDP_OK; w *= 2)
+  for (int pers = 0; pers < 2 && s == DSDP_OK; ++pers) {
+    P->flags = base_flags | (pers ? DSDP_PLAN_PERSISTENT : 0u);
     e = plan_use_warps(P, w);
     if (e != cudaSuccess) {
       s = check_cuda(e, "autotune tiles");
       break;
     }
-  for (int var = 0; var < n_var && s == DSDP_OK; ++var)
-    for (int pers = 0; pers < 2 && s == DSDP_OK; ++pers) {
+    for (int var = 0; var < n_var && s == DSDP_OK; ++var) {
       P->variant = var;
-      P->flags = base_flags | (pers ? DSDP_PLAN_PERSISTENT : 0u);
       s = dsdp_plan_launch_stage(P, DSDP_STAGE_CHAINS, stream);  // warm-up
       if (s != DSDP_OK) break;
       cudaEventRecord(a, st);

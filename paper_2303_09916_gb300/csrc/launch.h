@@ -7,13 +7,21 @@
 
 namespace dsdp {
 
+// Whether a chain launch takes its tiles from the work queue (ChainQueue): never,
+// always, or when there are more tiles than CTAs fit on the GPU at once.
+enum ChainQueueMode { kNoQueue, kQueue, kQueueIfMany };
+
 struct ChainLaunch {
   const void* jobs;   // DevJob[] (device)
   const void* tiles;  // Tile[] (device)
   int n_tiles;
-  int* tile_counter;  // device int, zeroed before a persistent launch
-  int persistent;
-  int grid;           // CTAs
+  ChainQueueMode queue;
+  int* counter;       // the queue's device arrays (ChainQueue), zeroed before the launch
+  int* tickets;
+  int* next_step;
+  const SliceBlock* blocks;  // device; the items of a time-sliced launch
+  int n_blocks, n_items;
+  bool overlap;       // independent of the launch before it on the stream: its CTAs may start as that one's leave
   int warps_per_cta;
   int apl;            // largest atoms-per-lane tile present
   int apl_mask;       // tiles present: bit 0 one atom per lane (<= 32 atoms), bit 1 two (<= 64)
