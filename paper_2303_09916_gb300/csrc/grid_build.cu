@@ -1,22 +1,48 @@
 // Receptor grid maps (Sec. 2 first modification; Appendix Eq. 1 and Eq. 4)
 // and the gather microbenchmark that bounds the score path.
 //
-// A CTA owns a brick of 8 x 8 x 4 vertices.  It streams the receptor atoms in
-// index order, keeps those within the cutoff of the brick's bounding box
+// A CTA owns a brick of 8 x 8 x 4 SB vertices.  It streams the receptor atoms in
+// index order and keeps those within the cutoff of the brick's bounding box
 // (ballot compaction into shared memory, order preserved, so the sums are
-// deterministic), then every thread sums the pair score and its gradient
-// for all 8 ligand types at its vertex.  The 8 types share 4 atomic radii:
-// the gauss / repulsion terms are summed once per radius (packed FP32x2, two
-// radii per operation), and the hydrophobic and H-bond terms, which only some
-// receptor atoms carry and only at short range, in five sums of their own;
-// each type's map is its radius sum plus its own term at the end.
+// deterministic).  A warp owns SB blocks of 4 x 4 x 2 vertices, one per lane; it tests
+// the kept atoms 32 at a time against its own box and sums, for every atom within
+// the cutoff of the box, the pair score and its gradient for all 8 ligand types.
+// The 8 types share 4 atomic radii: the gauss / repulsion terms are summed once
+// per radius (packed FP32x2, two radii per operation), and the hydrophobic and
+// H-bond terms, which only some receptor atoms carry and only at short range, in
+// five sums of their own; each type's map is its radius sum plus its own term at
+// the end.
+//
+// Bound: the FMA pipe (a packed FP32x2 instruction holds it for two cycles).  So an
+// atom takes the cheapest of three forms that its least distance to the warp's box
+// allows, chosen for the whole warp (no divergence):
+//   far  (d >= 2.4 for every radius): gauss2 alone -- there gauss1 and its slope are
+//        below half a unit in the last place of gauss2's (half the atoms in range);
+//   mid  (d >= 0): no repulsion, which is exactly 0;
+//   near: all terms.
+// The sums run in units of gauss2's weight and slope, which multiply once at the end.
+// The scan over all receptor atoms is the rest: two blocks a warp (SB = 2) halve it
+// and are taken from four waves of CTAs on; below, the smaller bricks fill the SMs
+// better.
 #include "launch.h"
 
 namespace dsdp {
 namespace {
 
 constexpr int kBX = 8, kBY = 8, kBZ = 4, kThreads = kBX * kBY * kBZ;
-constexpr int kChunk = 1536;
+constexpr int kChunk = 1536;       // kept atoms staged at once
+constexpr int kTests = 2;          // atoms a thread tests per barrier
+constexpr float kFarMid = 2.41f;  // surface distance from which gauss1 does not change an FP32 sum with gauss2
+
+// 2^(-u^2) = exp(-b^2) for u = kB2 b; b = (d - 3) / 2
+constexpr float kRootLog2E = 1.2011224087864498f;  // sqrt(1 / ln 2)
+constexpr float kU = 0.5f * kRootLog2E;            // u = kU d - 3 kU
+// units of the sums: energies of kWGauss2, slopes of -kWGauss2 / kRootLog2E (per u exp(-b^2))
+constexpr float kSlopeUnit = -kWGauss2 / kRootLog2E;
+constexpr float kE1 = kWGauss1 / kWGauss2;             // gauss1
+constexpr float kS1 = -8.f * kWGauss1 / kSlopeUnit;    //   slope -8 d exp(-4 d^2)
+constexpr float kE3 = kWRepulsion / kWGauss2;          // repulsion m^2, slope 2 m
+constexpr float kS3 = 2.f * kWRepulsion / kSlopeUnit;
 
 // hydrophobic term of surface distance d (1 below 0.5, linear to 0 at 1.5),
 // added to e and de/dd
@@ -71,123 +97,217 @@ __device__ __forceinline__ void store_node(void* maps, size_t idx, float e, floa
   }
 }
 
-template <int FMT>
-__global__ void __launch_bounds__(kThreads) grid_build_kernel(int n_rec, const float* __restrict__ xyz,
-                                                              const uint8_t* __restrict__ type, int nx, int ny,
-                                                              int nz, float ox, float oy, float oz, float h,
-                                                              void* __restrict__ maps) {
-  __shared__ float4 s_atom[kChunk];
-  __shared__ int s_count[kThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int bx0 = blockIdx.x * kBX, by0 = blockIdx.y * kBY, bz0 = blockIdx.z * kBZ;
-  const int ix = bx0 + (tid & 7), iy = by0 + ((tid >> 3) & 7), iz = bz0 + (tid >> 6);
-  const bool active = ix < nx && iy < ny && iz < nz;
-  const float mx = ox + h * (float)ix, my = oy + h * (float)iy, mz = oz + h * (float)iz;
-  const float lox = ox + h * (float)bx0, loy = oy + h * (float)by0, loz = oz + h * (float)bz0;
-  const float hix = ox + h * (float)min(bx0 + kBX - 1, nx - 1), hiy = oy + h * (float)min(by0 + kBY - 1, ny - 1),
-              hiz = oz + h * (float)min(bz0 + kBZ - 1, nz - 1);
-  const float reach2 = (kCutoff + 0.01f) * (kCutoff + 0.01f);
-  // gauss / repulsion sums per radius, packed (1.9, 1.8) and (1.7, 2.0): energy and gradient
-  float2 Ea = make_float2(0.f, 0.f), Eb = Ea, Xa = Ea, Xb = Ea, Ya = Ea, Yb = Ea, Za = Ea, Zb = Ea;
-  // hydrophobic term of C_H; H-bond terms of N_D (with receptor acceptors), N_A
-  // and O_A (with receptor donors), O_DA (with donors or acceptors): (e, gx, gy, gz)
-  float4 Hch = make_float4(0.f, 0.f, 0.f, 0.f), Hnd = Hch, Hna = Hch, Hoa = Hch, Hoda = Hch;
-  int base = 0;
-  while (base < n_rec) {
-    int count = 0;
-    while (base < n_rec && count <= kChunk - kThreads) {
-      const int j = base + tid;
-      bool keep = false;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j < n_rec) {
-        a.x = __ldg(xyz + 3 * j);
-        a.y = __ldg(xyz + 3 * j + 1);
-        a.z = __ldg(xyz + 3 * j + 2);
-        a.w = __int_as_float((int)__ldg(type + j));
-        const float dx = fmaxf(fmaxf(lox - a.x, a.x - hix), 0.f);
-        const float dy = fmaxf(fmaxf(loy - a.y, a.y - hiy), 0.f);
-        const float dz = fmaxf(fmaxf(loz - a.z, a.z - hiz), 0.f);
-        keep = dx * dx + dy * dy + dz * dz < reach2;
-      }
-      const unsigned bal = __ballot_sync(kFull, keep);
-      if (lane == 0) s_count[warp] = __popc(bal);
-      __syncthreads();
-      int off = count, total = 0;
-#pragma unroll
-      for (int w = 0; w < kThreads / 32; ++w) {
-        const int c = s_count[w];
-        if (w < warp) off += c;
-        total += c;
-      }
-      if (keep) s_atom[off + __popc(bal & ((1u << lane) - 1u))] = a;
-      count += total;
-      base += kThreads;
-      __syncthreads();
-    }
-    if (active) {
-      for (int k = 0; k < count; ++k) {
-        const float4 a = s_atom[k];
-        const float dx = mx - a.x, dy = my - a.y, dz = mz - a.z;
-        const float r2 = dx * dx + dy * dy + dz * dz;
-        if (!(r2 < kCutoff * kCutoff)) continue;
-        // a vertex on an atom (r = 0) takes no gradient from it: ir is finite there and d* = 0
-        const float ir = rsqrt_ftz(fmaxf(r2, 1e-30f));
-        const float r = r2 * ir;
-        const int tj = min(__float_as_int(a.w), 8);
-        const float Rj = c_xs_radius[tj];
-        const int bj = c_xs_bits[tj];  // the same for every thread: the branches below do not diverge on it
-        const float2 sa = make_float2(r - (1.9f + Rj), r - (1.8f + Rj));
-        const float2 sb = make_float2(r - (1.7f + Rj), r - (2.0f + Rj));
-        float2 ea, da, eb, db;
-        steric_x2(sa, ea, da);
-        steric_x2(sb, eb, db);
-        const float ux = dx * ir, uy = dy * ir, uz = dz * ir;
-        Ea = __fadd2_rn(Ea, ea);
-        Eb = __fadd2_rn(Eb, eb);
-        Xa = __ffma2_rn(da, splat2(ux), Xa);
-        Xb = __ffma2_rn(db, splat2(ux), Xb);
-        Ya = __ffma2_rn(da, splat2(uy), Ya);
-        Yb = __ffma2_rn(db, splat2(uy), Yb);
-        Za = __ffma2_rn(da, splat2(uz), Za);
-        Zb = __ffma2_rn(db, splat2(uz), Zb);
-        if ((bj & 1) && sa.x < 1.5f) {  // hydrophobic receptor atom: C_H (radius 1.9)
-          float e = 0.f, de = 0.f;
-          hydrophobic(sa.x, e, de);
-          add_term(Hch, e, de, ux, uy, uz);
-        }
-        if ((bj & 6) && sa.y < 0.f) {  // donor and/or acceptor within H-bond range (d of radius 1.8 < 0)
-          if (bj & 4) {  // receptor acceptor: N_D (1.8)
-            float e = 0.f, de = 0.f;
-            hbond(sa.y, e, de);
-            add_term(Hnd, e, de, ux, uy, uz);
-          }
-          if (bj & 2) {  // receptor donor: N_A (1.8), O_A (1.7)
-            float e = 0.f, de = 0.f;
-            hbond(sa.y, e, de);
-            add_term(Hna, e, de, ux, uy, uz);
-            e = de = 0.f;
-            hbond(sb.x, e, de);
-            add_term(Hoa, e, de, ux, uy, uz);
-          }
-          float e = 0.f, de = 0.f;  // O_DA (1.7) with either
-          hbond(sb.x, e, de);
-          add_term(Hoda, e, de, ux, uy, uz);
-        }
-      }
-    }
-    __syncthreads();
+// Sums of one vertex: gauss / repulsion per radius, packed (1.9, 1.8) and (1.7,
+// 2.0): energy and gradient (units above); hydrophobic term of C_H; H-bond terms of
+// N_D (with receptor acceptors), N_A and O_A (with receptor donors), O_DA (with
+// donors or acceptors): (e, gx, gy, gz).
+struct VertexSums {
+  float2 Ea, Eb, Xa, Xb, Ya, Yb, Za, Zb;
+  float4 Hch, Hnd, Hna, Hoa, Hoda;
+};
+
+enum { kNear, kMid, kFar };
+
+// u = kU (r - R_j - s - 3) of the far form: kU r plus this, per receptor type and radius s
+struct FarOffsets {
+  float2 a[9], b[9];  // radii (1.9, 1.8) and (1.7, 2.0)
+};
+constexpr FarOffsets make_far_offsets() {
+  constexpr float R[9] = {1.9f, 1.9f, 1.8f, 1.8f, 1.8f, 1.7f, 1.7f, 2.0f, 1.8f};
+  FarOffsets o{};
+  for (int t = 0; t < 9; ++t) {
+    o.a[t].x = -kU * (R[t] + 4.9f), o.a[t].y = -kU * (R[t] + 4.8f);
+    o.b[t].x = -kU * (R[t] + 4.7f), o.b[t].y = -kU * (R[t] + 5.0f);
   }
-  if (!active) return;
-  const size_t nxyz = (size_t)nx * ny * nz;
-  const size_t v = ((size_t)iz * ny + iy) * nx + ix;
-  store_node<FMT>(maps, 0 * nxyz + v, Ea.x + Hch.x, Xa.x + Hch.y, Ya.x + Hch.z, Za.x + Hch.w);     // C_H
-  store_node<FMT>(maps, 1 * nxyz + v, Ea.x, Xa.x, Ya.x, Za.x);                                     // C_P
-  store_node<FMT>(maps, 2 * nxyz + v, Ea.y, Xa.y, Ya.y, Za.y);                                     // N_P
-  store_node<FMT>(maps, 3 * nxyz + v, Ea.y + Hnd.x, Xa.y + Hnd.y, Ya.y + Hnd.z, Za.y + Hnd.w);     // N_D
-  store_node<FMT>(maps, 4 * nxyz + v, Ea.y + Hna.x, Xa.y + Hna.y, Ya.y + Hna.z, Za.y + Hna.w);     // N_A
-  store_node<FMT>(maps, 5 * nxyz + v, Eb.x + Hoa.x, Xb.x + Hoa.y, Yb.x + Hoa.z, Zb.x + Hoa.w);     // O_A
-  store_node<FMT>(maps, 6 * nxyz + v, Eb.x + Hoda.x, Xb.x + Hoda.y, Yb.x + Hoda.z, Zb.x + Hoda.w); // O_DA
-  store_node<FMT>(maps, 7 * nxyz + v, Eb.y, Xb.y, Yb.y, Zb.y);                                     // S_P
+  return o;
+}
+__constant__ FarOffsets c_far = make_far_offsets();
+
+// gauss2 at u, and with KIND != kFar gauss1 (and repulsion) at the surface distance d, of two radii
+template <int KIND>
+__device__ __forceinline__ void add_radii(float2 d, float2 u, float2 ux, float2 uy, float2 uz, float2& E, float2& X,
+                                          float2& Y, float2& Z) {
+  const float2 uu = __fmul2_rn(u, u);
+  const float2 g2 = make_float2(ex2_approx(-uu.x), ex2_approx(-uu.y));
+  float2 p = __fmul2_rn(u, g2);
+  E = __fadd2_rn(E, g2);
+  if (KIND != kFar) {
+    const float2 dd = __fmul2_rn(d, __fmul2_rn(d, splat2(-4.f * kLog2E)));
+    const float2 g1 = make_float2(ex2_approx(dd.x), ex2_approx(dd.y));
+    E = __ffma2_rn(g1, splat2(kE1), E);
+    p = __ffma2_rn(__fmul2_rn(g1, d), splat2(kS1), p);
+  }
+  if (KIND == kNear) {
+    const float2 m = make_float2(fminf(d.x, 0.f), fminf(d.y, 0.f));
+    E = __ffma2_rn(__fmul2_rn(m, m), splat2(kE3), E);
+    p = __ffma2_rn(m, splat2(kS3), p);
+  }
+  X = __ffma2_rn(p, ux, X);
+  Y = __ffma2_rn(p, uy, Y);
+  Z = __ffma2_rn(p, uz, Z);
+}
+
+// One receptor atom at the vertex (mx, my, mz).  The distance, the cutoff and the
+// surface distances of the hydrophobic and H-bond branches are one fixed sequence
+// of FP32 operations in every form; beyond the cutoff the distance is set so far
+// out that every term is exactly 0.
+template <int KIND>
+__device__ __forceinline__ void add_atom(VertexSums& S, const float4 a, float mx, float my, float mz) {
+  const float dx = mx - a.x, dy = my - a.y, dz = mz - a.z;
+  const float r2 = dx * dx + dy * dy + dz * dz;
+  const int tj = __float_as_int(a.w);
+  const float Rj = c_xs_radius[tj];
+  // a vertex on an atom (r = 0) takes no gradient from it: ir is finite there and d* = 0
+  const float ir = rsqrt_ftz(fmaxf(r2, 1e-30f));
+  const float r = r2 < kCutoff * kCutoff ? r2 * ir : 2.f * kFarD;
+  const float2 ux = splat2(dx * ir), uy = splat2(dy * ir), uz = splat2(dz * ir);
+  if (KIND == kFar) {
+    const float2 ur = splat2(kU * r), none = make_float2(0.f, 0.f);
+    add_radii<kFar>(none, __fadd2_rn(ur, c_far.a[tj]), ux, uy, uz, S.Ea, S.Xa, S.Ya, S.Za);
+    add_radii<kFar>(none, __fadd2_rn(ur, c_far.b[tj]), ux, uy, uz, S.Eb, S.Xb, S.Yb, S.Zb);
+    return;
+  }
+  const float2 sa = make_float2(r - (1.9f + Rj), r - (1.8f + Rj));
+  const float2 sb = make_float2(r - (1.7f + Rj), r - (2.0f + Rj));
+  const float2 ku = splat2(kU), k3 = splat2(-3.f * kU);
+  add_radii<KIND>(sa, __ffma2_rn(sa, ku, k3), ux, uy, uz, S.Ea, S.Xa, S.Ya, S.Za);
+  add_radii<KIND>(sb, __ffma2_rn(sb, ku, k3), ux, uy, uz, S.Eb, S.Xb, S.Yb, S.Zb);
+  const int bj = c_xs_bits[tj];  // the same for every lane: the branches below do not diverge on it
+  if ((bj & 1) && sa.x < 1.5f) {  // hydrophobic receptor atom: C_H (radius 1.9)
+    float e = 0.f, de = 0.f;
+    hydrophobic(sa.x, e, de);
+    add_term(S.Hch, e, de, ux.x, uy.x, uz.x);
+  }
+  if (KIND == kNear && (bj & 6) && sa.y < 0.f) {  // donor and/or acceptor within H-bond range (d of radius 1.8 < 0)
+    if (bj & 4) {  // receptor acceptor: N_D (1.8)
+      float e = 0.f, de = 0.f;
+      hbond(sa.y, e, de);
+      add_term(S.Hnd, e, de, ux.x, uy.x, uz.x);
+    }
+    if (bj & 2) {  // receptor donor: N_A (1.8), O_A (1.7)
+      float e = 0.f, de = 0.f;
+      hbond(sa.y, e, de);
+      add_term(S.Hna, e, de, ux.x, uy.x, uz.x);
+      e = de = 0.f;
+      hbond(sb.x, e, de);
+      add_term(S.Hoa, e, de, ux.x, uy.x, uz.x);
+    }
+    float e = 0.f, de = 0.f;  // O_DA (1.7) with either
+    hbond(sb.x, e, de);
+    add_term(S.Hoda, e, de, ux.x, uy.x, uz.x);
+  }
+}
+
+// squared distance from a point to the box of half sides (ex, ey, ez) around (cx, cy, cz)
+__device__ __forceinline__ float box_dist2(float4 a, float cx, float cy, float cz, float ex, float ey, float ez) {
+  const float dx = fmaxf(fabsf(a.x - cx) - ex, 0.f), dy = fmaxf(fabsf(a.y - cy) - ey, 0.f),
+              dz = fmaxf(fabsf(a.z - cz) - ez, 0.f);
+  return dx * dx + dy * dy + dz * dz;
+}
+
+template <int FMT, int SB>
+__global__ void __launch_bounds__(kThreads, 3) grid_build_kernel(int n_rec, const float* __restrict__ xyz,
+                                                                 const uint8_t* __restrict__ type, int nx, int ny,
+                                                                 int nz, float ox, float oy, float oz, float h,
+                                                                 void* __restrict__ maps) {
+  constexpr int kWarps = kThreads / 32;
+  __shared__ float4 s_atom[kChunk];
+  __shared__ int s_count[kTests * kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bx0 = blockIdx.x * kBX, by0 = blockIdx.y * kBY, bz0 = blockIdx.z * kBZ * SB;
+  const float bcx = ox + h * ((float)bx0 + 0.5f * (kBX - 1)), bcy = oy + h * ((float)by0 + 0.5f * (kBY - 1)),
+              bcz = oz + h * ((float)bz0 + 0.5f * (kBZ * SB - 1));
+  // the boxes' tests allow 0.01 A for rounding
+  const float reach2 = (kCutoff + 0.01f) * (kCutoff + 0.01f);
+  int count = 0;
+  bool staged = false;  // the kept atoms of the whole receptor are in s_atom
+#pragma unroll 1
+  for (int sb = 0; sb < SB; ++sb) {
+    // the warp's 4 x 4 x 2 vertices
+    const int wx0 = bx0 + 4 * (warp & 1), wy0 = by0 + 4 * ((warp >> 1) & 1), wz0 = bz0 + 2 * (warp >> 2) + kBZ * sb;
+    const int ix = wx0 + (lane & 3), iy = wy0 + ((lane >> 2) & 3), iz = wz0 + (lane >> 4);
+    const bool warp_active = wx0 < nx && wy0 < ny && wz0 < nz;
+    const float mx = ox + h * (float)ix, my = oy + h * (float)iy, mz = oz + h * (float)iz;
+    const float wcx = ox + h * ((float)wx0 + 1.5f), wcy = oy + h * ((float)wy0 + 1.5f),
+                wcz = oz + h * ((float)wz0 + 0.5f);
+    VertexSums S;
+    S.Ea = S.Eb = S.Xa = S.Xb = S.Ya = S.Yb = S.Za = S.Zb = make_float2(0.f, 0.f);
+    S.Hch = S.Hnd = S.Hna = S.Hoa = S.Hoda = make_float4(0.f, 0.f, 0.f, 0.f);
+    int base = staged ? n_rec : 0;
+    do {
+      const bool first = base == 0;
+      if (!staged) count = 0;
+      while (base < n_rec && count <= kChunk - kTests * kThreads) {
+        float4 a[kTests];
+        unsigned bal[kTests];
+#pragma unroll
+        for (int k = 0; k < kTests; ++k) {
+          const int j = base + k * kThreads + tid;
+          bool keep = false;
+          a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (j < n_rec) {
+            a[k].x = __ldg(xyz + 3 * j);
+            a[k].y = __ldg(xyz + 3 * j + 1);
+            a[k].z = __ldg(xyz + 3 * j + 2);
+            a[k].w = __int_as_float(min((int)__ldg(type + j), 8));
+            // an atom that is not at a finite place is in no vertex's range
+            keep = box_dist2(a[k], bcx, bcy, bcz, 0.5f * (kBX - 1) * h, 0.5f * (kBY - 1) * h,
+                             0.5f * (kBZ * SB - 1) * h) < reach2 && isfinite(a[k].x + a[k].y + a[k].z);
+          }
+          bal[k] = __ballot_sync(kFull, keep);
+          if (lane == 0) s_count[k * kWarps + warp] = __popc(bal[k]);
+        }
+        __syncthreads();
+        int total = 0;
+#pragma unroll
+        for (int k = 0; k < kTests; ++k) {
+          int off = count + total;
+#pragma unroll
+          for (int w = 0; w < kWarps; ++w) {
+            const int c = s_count[k * kWarps + w];
+            if (w < warp) off += c;
+            total += c;
+          }
+          if ((bal[k] >> lane) & 1) s_atom[off + __popc(bal[k] & ((1u << lane) - 1u))] = a[k];
+        }
+        count += total;
+        base += kTests * kThreads;
+        __syncthreads();
+      }
+      if (first && base >= n_rec) staged = true;  // the same in every thread
+      if (warp_active) {
+        for (int k0 = 0; k0 < count; k0 += 32) {
+          const bool have = k0 + lane < count;
+          const float4 a = have ? s_atom[k0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float d2 = have ? box_dist2(a, wcx, wcy, wcz, 1.5f * h, 1.5f * h, 0.5f * h) : reach2;
+          const float far = 2.0f + kFarMid + c_xs_radius[__float_as_int(a.w)], mid = far - kFarMid + 0.01f;
+          unsigned m_far = __ballot_sync(kFull, d2 < reach2 && d2 >= far * far);
+          unsigned m_mid = __ballot_sync(kFull, d2 < far * far && d2 >= mid * mid);
+          unsigned m_near = __ballot_sync(kFull, d2 < mid * mid);
+          for (; m_far; m_far &= m_far - 1) add_atom<kFar>(S, s_atom[k0 + __ffs(m_far) - 1], mx, my, mz);
+          for (; m_mid; m_mid &= m_mid - 1) add_atom<kMid>(S, s_atom[k0 + __ffs(m_mid) - 1], mx, my, mz);
+          for (; m_near; m_near &= m_near - 1) add_atom<kNear>(S, s_atom[k0 + __ffs(m_near) - 1], mx, my, mz);
+        }
+      }
+      if (!staged) __syncthreads();  // the next atoms replace these
+    } while (base < n_rec);
+    if (ix >= nx || iy >= ny || iz >= nz) continue;
+    const size_t nxyz = (size_t)nx * ny * nz;
+    const size_t v = ((size_t)iz * ny + iy) * nx + ix;
+    auto store = [&](int t, float e, float x, float y, float z, const float4& H) {
+      store_node<FMT>(maps, t * nxyz + v, fmaf(e, kWGauss2, H.x), fmaf(x, kSlopeUnit, H.y), fmaf(y, kSlopeUnit, H.z),
+                      fmaf(z, kSlopeUnit, H.w));
+    };
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    store(0, S.Ea.x, S.Xa.x, S.Ya.x, S.Za.x, S.Hch);   // C_H
+    store(1, S.Ea.x, S.Xa.x, S.Ya.x, S.Za.x, none);    // C_P
+    store(2, S.Ea.y, S.Xa.y, S.Ya.y, S.Za.y, none);    // N_P
+    store(3, S.Ea.y, S.Xa.y, S.Ya.y, S.Za.y, S.Hnd);   // N_D
+    store(4, S.Ea.y, S.Xa.y, S.Ya.y, S.Za.y, S.Hna);   // N_A
+    store(5, S.Eb.x, S.Xb.x, S.Yb.x, S.Zb.x, S.Hoa);   // O_A
+    store(6, S.Eb.x, S.Xb.x, S.Yb.x, S.Zb.x, S.Hoda);  // O_DA
+    store(7, S.Eb.y, S.Xb.y, S.Yb.y, S.Zb.y, none);    // S_P
+  }
 }
 
 // 32-bit mixing hash (multiply-xorshift; the finaliser of MurmurHash3) for the
@@ -233,8 +353,14 @@ __global__ void __launch_bounds__(256) gather_bench_kernel(MapView M, const floa
 template <int FMT>
 cudaError_t launch_grid(const dsdp_receptor* rec, int nx, int ny, int nz, float ox, float oy, float oz, float h,
                         void* maps, cudaStream_t st) {
-  const dim3 grid((nx + kBX - 1) / kBX, (ny + kBY - 1) / kBY, (nz + kBZ - 1) / kBZ);
-  grid_build_kernel<FMT><<<grid, kThreads, 0, st>>>(rec->n, rec->xyz, rec->xs_type, nx, ny, nz, ox, oy, oz, h, maps);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  dim3 grid((nx + kBX - 1) / kBX, (ny + kBY - 1) / kBY, (nz + 2 * kBZ - 1) / (2 * kBZ));
+  const bool two = (long long)grid.x * grid.y * grid.z >= 4ll * 3 * sms;  // 3 CTAs per SM
+  if (!two) grid.z = (nz + kBZ - 1) / kBZ;
+  auto k = two ? grid_build_kernel<FMT, 2> : grid_build_kernel<FMT, 1>;
+  k<<<grid, kThreads, 0, st>>>(rec->n, rec->xyz, rec->xs_type, nx, ny, nz, ox, oy, oz, h, maps);
   return cudaGetLastError();
 }
 
