@@ -18,11 +18,18 @@
 //     and accumulated as 64-bit integers; a channel is the sum times 2^-24
 //     rounded to FP32.
 //
-// One warp per atom: lanes hold the atom's 98 test points (four per lane); the
-// warp scans the receptor 32 atoms at a time, keeps those whose sphere can
-// reach the atom's (a conservative FP32 pre-test), and each lane checks its
-// points against them, broadcast by shuffle.  No shared memory, no scratch
-// beyond the caller's accumulator.
+// Three launches.  voxel_bin_kernel sorts the atoms into cells of 4 voxels (one
+// CTA, counting sort in shared memory; the others clear the accumulator).
+// voxel_atoms_kernel gives an atom a warp, whose lanes hold its 98 test points
+// (four per lane): it scans the cells in reach 32 atoms at a time, keeps those
+// whose sphere can reach the atom's (a conservative FP32 pre-test), and each lane
+// checks its points against them, broadcast by shuffle, until all are buried.
+// voxel_finish_kernel writes the channels.
+//
+// Bound: latency (launches, L2 loads).  Scanning every atom for every atom, as
+// receptors of more atoms than the output holds cell lists for still do, took
+// 52 us of the call's 59 at 4,000 atoms.  The lists wait in the output array, which
+// is written last.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -80,23 +87,133 @@ __device__ __forceinline__ float3 sas_direction(int m) {
   return make_float3(__fdiv_rn((float)a, len), __fdiv_rn((float)b, len), __fdiv_rn((float)c, len));
 }
 
+// Cells of 4 voxels: 9 per axis in the cube and one on either side for all that
+// lies beyond it.
+constexpr int kCells = kVoxN / 4 + 2;
+constexpr int kCellCount = kCells * kCells * kCells;
+constexpr float kCellInv = 36.0f / 70.0f / 4.0f;
+
+// The sorted atoms' lists in the output array (4-byte aligned).
+struct CellLists {
+  int* start;         // [kCellCount + 1]
+  float* max_radius;  // largest |r_i + 1.4|
+  int* index;         // [n] the caller's index of each sorted atom
+  float *x, *y, *z, *R;
+};
+constexpr int kListWords = kCellCount + 2;
+constexpr int kMaxListed = (kVoxN * kVoxN * kVoxN * kVoxC - kListWords) / 5;
+__host__ __device__ inline CellLists cell_lists(float* out, int n) {
+  CellLists L;
+  L.start = reinterpret_cast<int*>(out);
+  L.max_radius = out + kCellCount + 1;
+  float* p = out + kListWords;
+  L.index = reinterpret_cast<int*>(p);
+  L.x = p + n;
+  L.y = p + 2 * n;
+  L.z = p + 3 * n;
+  L.R = p + 4 * n;
+  return L;
+}
+
+// Cell of a coordinate along one axis (0: below the cube, kCells - 1: above);
+// monotonic in x, so atoms closer than k cells are at most k cells apart.
+__device__ __forceinline__ int cell_of(float x, float lo) {
+  return (int)fminf(fmaxf(floorf((x - lo) * kCellInv) + 1.f, 0.f), (float)(kCells - 1));
+}
+
+__global__ void __launch_bounds__(1024) voxel_bin_kernel(int n, const float* __restrict__ xyz,
+                                                         const float* __restrict__ radius, float lox, float loy,
+                                                         float loz, CellLists L, unsigned long long* __restrict__ acc) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x > 0) {
+    const int total = kVoxN * kVoxN * kVoxN * kVoxC, stride = (gridDim.x - 1) * blockDim.x;
+    const int q0 = (blockIdx.x - 1) * blockDim.x + tid;
+    if ((reinterpret_cast<uintptr_t>(acc) & 15) == 0) {
+      for (int q = q0; q < total / 2; q += stride) reinterpret_cast<ulonglong2*>(acc)[q] = make_ulonglong2(0ull, 0ull);
+    } else {
+      for (int q = q0; q < total; q += stride) acc[q] = 0ull;
+    }
+    return;
+  }
+  __shared__ int s_at[kCellCount];  // counts, then the next free place of each cell
+  __shared__ int s_warp[32];
+  __shared__ unsigned s_max;
+  for (int c = tid; c < kCellCount; c += 1024) s_at[c] = 0;
+  if (tid == 0) s_max = 0u;
+  __syncthreads();
+  // an atom that is not at a finite place is in no voxel and near no atom
+  auto cell = [&](int i, float& x, float& y, float& z) {
+    x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
+    if (!isfinite(x) || !isfinite(y) || !isfinite(z)) return -1;
+    return (cell_of(z, loz) * kCells + cell_of(y, loy)) * kCells + cell_of(x, lox);
+  };
+  float x, y, z, most = 0.f;
+#pragma unroll 4
+  for (int i = tid; i < n; i += 1024) {
+    const int c = cell(i, x, y, z);
+    if (c >= 0) atomicAdd(s_at + c, 1);
+    most = fmaxf(most, fabsf(__fadd_rn(radius[i], kProbe)));  // NaN reaches nothing
+  }
+  atomicMax(&s_max, __float_as_uint(most));  // of non-negative floats
+  __syncthreads();
+  // exclusive prefix sums over the cells, two per thread
+  const int c0 = 2 * tid, v0 = c0 < kCellCount ? s_at[c0] : 0, v1 = c0 + 1 < kCellCount ? s_at[c0 + 1] : 0;
+  int inc = v0 + v1;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  int before = inc - v0 - v1 + __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0);
+  if (c0 < kCellCount) s_at[c0] = L.start[c0] = before;
+  if (c0 + 1 < kCellCount) s_at[c0 + 1] = L.start[c0 + 1] = before + v0;
+  if (c0 <= kCellCount - 1 && c0 + 2 > kCellCount - 1) L.start[kCellCount] = before + v0 + v1;
+  if (tid == 0) *L.max_radius = __uint_as_float(s_max);
+  __syncthreads();
+#pragma unroll 4
+  for (int i = tid; i < n; i += 1024) {
+    const int c = cell(i, x, y, z);
+    if (c < 0) continue;
+    const int p = atomicAdd(s_at + c, 1);  // any order within a cell: what follows does not depend on it
+    L.index[p] = i;
+    L.x[p] = x, L.y[p] = y, L.z[p] = z;
+    L.R[p] = __fadd_rn(radius[i], kProbe);
+  }
+}
+
+// LISTED: atoms and neighbours from the cell lists; else every atom is scanned.
+template <bool LISTED>
 __global__ void __launch_bounds__(256) voxel_atoms_kernel(int n, const float* __restrict__ xyz,
                                                           const float* __restrict__ radius,
                                                           const float* __restrict__ feat, float lox, float loy,
-                                                          float loz, unsigned long long* __restrict__ acc) {
+                                                          float loz, CellLists L,
+                                                          unsigned long long* __restrict__ acc) {
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5);
+  // one direction per thread, shared by the CTA's warps: per lane and warp the
+  // divergent reads of the constant table and the divisions were a third of the kernel
+  __shared__ float3 s_dir[32 * kPointsPerLane];
+  if (threadIdx.x < 32 * kPointsPerLane)
+    s_dir[threadIdx.x] = threadIdx.x < 98 ? sas_direction(threadIdx.x) : make_float3(0.f, 0.f, 0.f);
+  __syncthreads();
   float3 u[kPointsPerLane];
   bool used[kPointsPerLane];
 #pragma unroll
   for (int s = 0; s < kPointsPerLane; ++s) {
-    const int m = lane + 32 * s;
-    used[s] = m < 98;
-    u[s] = used[s] ? sas_direction(m) : make_float3(0.f, 0.f, 0.f);
+    used[s] = lane + 32 * s < 98;
+    u[s] = s_dir[lane + 32 * s];
   }
   const float inv = 36.0f / 70.0f;
-  for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {  // warp-uniform
-    const float xi = xyz[3 * i], yi = xyz[3 * i + 1], zi = xyz[3 * i + 2];
+  const int count = LISTED ? L.start[kCellCount] : n;
+  // cells in reach on either side: no sphere reaches farther than the two largest;
+  // a little more against the rounding of the cells
+  const int reach_cells =
+      LISTED ? (int)fminf(floorf((2.f * *L.max_radius + 0.02f) * kCellInv + 1e-3f) + 1.f, (float)kCells) : 0;
+  for (int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < count; p += warps) {  // warp-uniform
+    const int i = LISTED ? L.index[p] : p;
+    const float xi = LISTED ? L.x[p] : xyz[3 * i], yi = LISTED ? L.y[p] : xyz[3 * i + 1],
+                zi = LISTED ? L.z[p] : xyz[3 * i + 2];
     const float ux = __fmul_rn(__fsub_rn(xi, lox), inv), uy = __fmul_rn(__fsub_rn(yi, loy), inv),
                 uz = __fmul_rn(__fsub_rn(zi, loz), inv);
     // floor(u) in [0, 36) exactly when u in [0, 36) (false for NaN): tested before any conversion
@@ -104,10 +221,12 @@ __global__ void __launch_bounds__(256) voxel_atoms_kernel(int n, const float* __
       continue;
     const int kx = (int)ux, ky = (int)uy, kz = (int)uz;
     unsigned long long* v = acc + (((size_t)kz * kVoxN + ky) * kVoxN + kx) * kVoxC;
-    if (lane < kVoxF)
-      atomicAdd(v + lane, (unsigned long long)__float2ll_rn(__fmul_rn(feat[(size_t)kVoxF * i + lane], kFix)));
+    if (lane < kVoxF) {
+      const long long q = __float2ll_rn(__fmul_rn(feat[(size_t)kVoxF * i + lane], kFix));
+      if (q) atomicAdd(v + lane, (unsigned long long)q);
+    }
     // ---- surface test
-    const float Ri = __fadd_rn(radius[i], kProbe);
+    const float Ri = LISTED ? L.R[p] : __fadd_rn(radius[i], kProbe);
     float px[kPointsPerLane], py[kPointsPerLane], pz[kPointsPerLane];
     bool buried[kPointsPerLane];
 #pragma unroll
@@ -117,45 +236,76 @@ __global__ void __launch_bounds__(256) voxel_atoms_kernel(int n, const float* __
       pz[s] = __fadd_rn(zi, __fmul_rn(Ri, u[s].z));
       buried[s] = !used[s];
     }
-    for (int j0 = 0; j0 < n; j0 += 32) {
-      const int j = j0 + lane;
-      float xj = 0.f, yj = 0.f, zj = 0.f, Rj = 0.f;
-      bool near = false;
-      if (j < n && j != i) {
-        xj = xyz[3 * j];
-        yj = xyz[3 * j + 1];
-        zj = xyz[3 * j + 2];
-        Rj = __fadd_rn(radius[j], kProbe);
-        // a sphere farther than Ri + Rj cannot cover a point of atom i's sphere;
-        // 0.01 A of slack keeps the pre-test conservative under FP32 rounding
-        const float dx = xj - xi, dy = yj - yi, dz = zj - zi, reach = Ri + Rj + 0.01f;
-        near = dx * dx + dy * dy + dz * dz < reach * reach;
-      }
-      unsigned m = __ballot_sync(0xffffffffu, near);
-      while (m) {  // warp-uniform
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        const float bx = __shfl_sync(0xffffffffu, xj, src), by = __shfl_sync(0xffffffffu, yj, src),
-                    bz = __shfl_sync(0xffffffffu, zj, src), bR = __shfl_sync(0xffffffffu, Rj, src);
-        const float R2 = __fmul_rn(bR, bR);
-#pragma unroll
-        for (int s = 0; s < kPointsPerLane; ++s) {
-          const float dx = __fsub_rn(px[s], bx), dy = __fsub_rn(py[s], by), dz = __fsub_rn(pz[s], bz);
-          const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-          buried[s] = buried[s] || d2 < R2;
+    // atoms [j0, j1) of the list (or of the receptor) against the points, until all are buried
+    bool hidden = false;
+    auto scan = [&](int j0, int j1) {
+      for (; j0 < j1 && !hidden; j0 += 32) {
+        const int j = j0 + lane;
+        float xj = 0.f, yj = 0.f, zj = 0.f, Rj = 0.f;
+        bool near = false;
+        if (j < j1 && j != p) {
+          xj = LISTED ? L.x[j] : xyz[3 * j];
+          yj = LISTED ? L.y[j] : xyz[3 * j + 1];
+          zj = LISTED ? L.z[j] : xyz[3 * j + 2];
+          Rj = LISTED ? L.R[j] : __fadd_rn(radius[j], kProbe);
+          // a sphere farther than Ri + Rj cannot cover a point of atom i's sphere;
+          // 0.01 A of slack keeps the pre-test conservative under FP32 rounding
+          const float dx = xj - xi, dy = yj - yi, dz = zj - zi, reach = Ri + Rj + 0.01f;
+          near = dx * dx + dy * dy + dz * dz < reach * reach;
         }
-      }
-    }
-    bool exposed = false;
+        unsigned m = __ballot_sync(0xffffffffu, near);
+        if (!m) continue;
+        while (m) {  // warp-uniform
+          const int src = __ffs(m) - 1;
+          m &= m - 1;
+          const float bx = __shfl_sync(0xffffffffu, xj, src), by = __shfl_sync(0xffffffffu, yj, src),
+                      bz = __shfl_sync(0xffffffffu, zj, src), bR = __shfl_sync(0xffffffffu, Rj, src);
+          const float R2 = __fmul_rn(bR, bR);
 #pragma unroll
-    for (int s = 0; s < kPointsPerLane; ++s) exposed = exposed || !buried[s];
-    if (__any_sync(0xffffffffu, exposed) && lane == 0) atomicAdd(v + kVoxF, (unsigned long long)(1ll << 24));
+          for (int s = 0; s < kPointsPerLane; ++s) {
+            const float dx = __fsub_rn(px[s], bx), dy = __fsub_rn(py[s], by), dz = __fsub_rn(pz[s], bz);
+            const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+            buried[s] = buried[s] || d2 < R2;
+          }
+        }
+        bool all = true;
+#pragma unroll
+        for (int s = 0; s < kPointsPerLane; ++s) all = all && buried[s];
+        hidden = __all_sync(0xffffffffu, all);
+      }
+    };
+    if (LISTED) {
+      const int cx = cell_of(xi, lox), cy = cell_of(yi, loy), cz = cell_of(zi, loz);
+      const int x0 = max(cx - reach_cells, 0), x1 = min(cx + reach_cells, kCells - 1), m = 2 * reach_cells + 1;
+      // rows of cells along x are contiguous in the list; the atom's own row first
+      for (int q = 0; q < m * m && !hidden; ++q) {
+        const int r = (q + (m * m) / 2) % (m * m), rz = cz + r / m - reach_cells, ry = cy + r % m - reach_cells;
+        if (rz < 0 || rz >= kCells || ry < 0 || ry >= kCells) continue;
+        const int row = (rz * kCells + ry) * kCells;
+        scan(L.start[row + x0], L.start[row + x1 + 1]);
+      }
+    } else {
+      scan(0, n);
+    }
+    if (!hidden && lane == 0) atomicAdd(v + kVoxF, (unsigned long long)(1ll << 24));
   }
 }
 
-__global__ void voxel_finish_kernel(const unsigned long long* __restrict__ acc, float* __restrict__ out, int n) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
-    out[q] = __double2float_rn(__ll2double_rn((long long)acc[q]) * (1.0 / 16777216.0));
+// Each sum times 2^-24, rounded to FP32 once.  Most voxels are empty and most sums
+// whole numbers; the others go through FP64, of which an SM does two a cycle.
+__global__ void __launch_bounds__(256) voxel_finish_kernel(const unsigned long long* __restrict__ acc,
+                                                           float* __restrict__ out, int n) {
+  const int stride = gridDim.x * blockDim.x;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) {
+    const long long v = (long long)acc[q];
+    float f = 0.f;
+    if (v != 0) {
+      const long long whole = v >> 24;
+      f = (v & 0xffffffll) == 0 && whole == (int)whole ? (float)(int)whole
+                                                       : __double2float_rn(__ll2double_rn(v) * (1.0 / 16777216.0));
+    }
+    out[q] = f;
+  }
 }
 
 }  // namespace
@@ -182,20 +332,30 @@ extern "C" dsdp_status dsdp_voxelize_device(int32_t n_atoms, const float* d_xyz,
     if (!isfinite(center[a])) return set_error(DSDP_ERR_INVALID_ARG, "voxelize: center not finite");
   const cudaStream_t st = (cudaStream_t)stream;
   unsigned long long* acc = (unsigned long long*)d_work;
-  cudaError_t e = cudaMemsetAsync(acc, 0, dsdp_voxel_work_bytes(), st);
-  if (e == cudaSuccess && n_atoms > 0) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int want = (n_atoms + 7) / 8, cap = sms * 8;  // 8 warps (atoms) per CTA
-    voxel_atoms_kernel<<<want < cap ? want : cap, 256, 0, st>>>(
-        n_atoms, d_xyz, d_radius, d_features, (float)(center[0] - 35.0), (float)(center[1] - 35.0),
-        (float)(center[2] - 35.0), acc);
+  const int total = kVoxN * kVoxN * kVoxN * kVoxC;
+  const float lox = (float)(center[0] - 35.0), loy = (float)(center[1] - 35.0), loz = (float)(center[2] - 35.0);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int want = (n_atoms + 7) / 8, cap = sms * 8;  // 8 warps (atoms) per CTA
+  const int grid = want < cap ? want : cap;
+  const CellLists lists = cell_lists(d_out, n_atoms);
+  cudaError_t e = cudaSuccess;
+  if (n_atoms > 0 && n_atoms <= kMaxListed) {
+    voxel_bin_kernel<<<1 + sms, 1024, 0, st>>>(n_atoms, d_xyz, d_radius, lox, loy, loz, lists, acc);
+    voxel_atoms_kernel<true>
+        <<<grid, 256, 0, st>>>(n_atoms, d_xyz, d_radius, d_features, lox, loy, loz, lists, acc);
     e = cudaGetLastError();
+  } else {
+    e = cudaMemsetAsync(acc, 0, dsdp_voxel_work_bytes(), st);
+    if (e == cudaSuccess && n_atoms > 0) {
+      voxel_atoms_kernel<false>
+          <<<grid, 256, 0, st>>>(n_atoms, d_xyz, d_radius, d_features, lox, loy, loz, lists, acc);
+      e = cudaGetLastError();
+    }
   }
   if (e == cudaSuccess) {
-    const int total = kVoxN * kVoxN * kVoxN * kVoxC;
-    voxel_finish_kernel<<<(total + 255) / 256, 256, 0, st>>>(acc, d_out, total);
+    voxel_finish_kernel<<<sms * 8, 256, 0, st>>>(acc, d_out, total);
     e = cudaGetLastError();
   }
   return check_cuda(e, "voxelize launch");
