@@ -252,23 +252,6 @@ __device__ __forceinline__ int pair_bits(int ti, int tj) {
   return bits;
 }
 
-// FP64 version for the rescoring (same terms; exp in double).
-__device__ __forceinline__ double vina_pair_f64(double d, int bits) {
-  const double a = 2.0 * d;
-  const double b = 0.5 * (d - 3.0);
-  double e = kWGauss1D * exp(-a * a) + kWGauss2D * exp(-b * b);
-  if (d < 0.0) e += kWRepulsionD * d * d;
-  if (bits & 1) {
-    if (d < 0.5) e += kWHydrophobicD;
-    else if (d < 1.5) e += kWHydrophobicD * (1.5 - d);
-  }
-  if (bits & 2) {
-    if (d < -0.7) e += kWHBondD;
-    else if (d < 0.0) e += kWHBondD * (-d / 0.7);
-  }
-  return e;
-}
-
 // ------------------------------------------------------------------ map formats
 // FMT encodes (dtype, mode): 0 F32 EQ4, 1 BF16 EQ4, 2 F16 EQ4, 3 F32 EQ3,
 // 4 BF16 EQ3, 5 F16 EQ3.

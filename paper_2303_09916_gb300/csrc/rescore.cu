@@ -14,8 +14,13 @@
 namespace dsdp {
 namespace {
 
-constexpr int kRescoreWarps = 8;
-constexpr int kRecTile = 1024;
+constexpr int kRescoreWarps = 8;  // poses of a tile
+// CTAs a tile is split into, each of kCtaWarps poses.  The FP64 pipe bounds the
+// kernel, so what counts is that every SM gets as many poses: 3,072 poses in CTAs of
+// 8 leave SMs with 16 and SMs with 24 of them, in CTAs of 2 with 20 and 22.
+constexpr int kSplit = 4, kCtaWarps = kRescoreWarps / kSplit;
+constexpr int kRecTile = 512;
+constexpr int kExpTable = 256;
 
 struct DQuat {
   double w, x, y, z;
@@ -32,19 +37,91 @@ __device__ __forceinline__ double3 dqrot(const DQuat& q, double3 v) {
 }
 __device__ __forceinline__ double shd(double v, int src) { return __shfl_sync(kFull, v, src); }
 
-// One warp per chain: FP64 pose, exact inter (receptor staged through shared
-// memory in tiles, FP32 pre-filter then FP64 distance) and intra.
-__global__ void __launch_bounds__(32 * kRescoreWarps) rescore_kernel(const DevJob* __restrict__ jobs,
-                                                                     const Tile* __restrict__ tiles) {
+// exp(-t), 0 <= t < 700, by table-driven argument reduction (P. T. P. Tang, ACM TOMS
+// 15, 144 (1989)): exp(-t) = 2^m T[j] exp(r) with 256 m + j the integer nearest
+// -256 t / ln 2, T[j] = 2^(j / 256) and |r| <= ln 2 / 512, where the Taylor
+// polynomial of degree 4 is off by less than 4e-17.  Nine FP64 operations.
+__device__ __forceinline__ double exp_neg(double t, const double* table) {
+  constexpr double kPerLn2 = 256.0 / 0.69314718055994530942;
+  constexpr double kStepHi = 0.69314718055994530942 / 256.0;
+  constexpr double kStepLo = 2.3190468138462996e-17 / 256.0;  // ln 2 minus its FP64 value, over 256
+  constexpr double kRound = 6755399441055744.0;               // 1.5 2^52: adding it leaves the nearest integer
+  const double n = fma(t, -kPerLn2, kRound);
+  const int k = __double2loint(n);
+  const double kd = n - kRound;
+  const double r = fma(-kd, kStepLo, fma(-kd, kStepHi, -t));
+  const double q = fma(r, fma(r, fma(r, 1.0 / 24.0, 1.0 / 6.0), 0.5), 1.0);
+  const double T = table[k & (kExpTable - 1)];
+  const double e = fma(T, r * q, T);
+  return __hiloint2double(__double2hiint(e) + ((k >> 8) << 20), __double2loint(e));
+}
+
+// Square root of r2 >= 0 from the FP32 reciprocal square root by two Newton steps
+// on the root (the first leaves 2^-43 relative, the second FP64 rounding).
+__device__ __forceinline__ double sqrt_d(double r2) {
+  const float y = rsqrt_ftz(fmaxf((float)r2, 1e-30f));
+  const double yd = (double)y, h = (double)(0.5f * y);
+  double r = r2 * yd;
+  r = fma(fma(-r, r, r2), h, r);
+  return fma(fma(-r, r, r2), h, r);
+}
+
+// Tables of the pair terms, in shared memory: 2^(j / 256); per pair of types
+// 9 ti + tj the sum of the radii and the terms it carries (pair_bits).  (Read from
+// the constant bank, the per-lane indices would take up to nine reads each.)
+struct PairTables {
+  double exp2[kExpTable];
+  double radii[81];
+  int bits[81];
+};
+__device__ __forceinline__ void fill_pair_tables(PairTables& P) {
+  for (int k = threadIdx.x; k < kExpTable; k += blockDim.x) P.exp2[k] = ::exp2(k * (1.0 / kExpTable));
+  for (int k = threadIdx.x; k < 81; k += blockDim.x) {
+    P.radii[k] = c_xs_radius_d[k / 9] + c_xs_radius_d[k % 9];
+    P.bits[k] = pair_bits(k / 9, k % 9);
+  }
+}
+
+// Vina-form pair energy at squared distance r2 < 64 (the terms of vina_pair_x2).
+__device__ __forceinline__ double pair_energy(double r2, int types, const PairTables& P) {
+  const double r = sqrt_d(r2);
+  if (!(r < kCutoffD)) return 0.0;
+  const double d = r - P.radii[types], c = d - 3.0;
+  double e = kWGauss1D * exp_neg(4.0 * (d * d), P.exp2);
+  e = fma(kWGauss2D, exp_neg(0.25 * (c * c), P.exp2), e);
+  if (d < 1.5) {  // the short-range terms
+    const int bits = P.bits[types];
+    if (d < 0.0) e = fma(kWRepulsionD * d, d, e);
+    if (bits & 1) e += d < 0.5 ? kWHydrophobicD : kWHydrophobicD * (1.5 - d);
+    if ((bits & 2) && d < 0.0) e += d < -0.7 ? kWHBondD : kWHBondD * (-d / 0.7);
+  }
+  return e;
+}
+
+// One warp per chain: FP64 pose, exact inter and intra.  For each receptor tile
+// staged in shared memory the warp keeps the atoms near the pose's bounding box (a
+// fifth of a 4,000-atom receptor), scans (ligand atom, kept atom) pairs with an
+// FP32 pre-filter (cutoff + 0.05 A), compacts the survivors into a per-warp list by
+// ballot, and evaluates them in FP64 32 at a time with every lane busy.
+//
+// Bound: the FP64 pipe (two results a cycle and SM), so the pair terms are written
+// for few FP64 operations: about 40 a pair where the library's exp and square root
+// took about 70.
+__global__ void __launch_bounds__(32 * kCtaWarps) rescore_kernel(const DevJob* __restrict__ jobs,
+                                                                 const Tile* __restrict__ tiles) {
   __shared__ float4 s_rec[kRecTile];
-  __shared__ double s_xyz[kRescoreWarps][kMaxAtoms * 3];
-  __shared__ int s_type[kRescoreWarps][kMaxAtoms];
-  __shared__ uint32_t s_list[kRescoreWarps][64];
-  const Tile tile = tiles[blockIdx.x];
+  __shared__ PairTables s_pair;
+  __shared__ double s_xyz[kCtaWarps][kMaxAtoms * 3];
+  __shared__ int s_type[kCtaWarps][kMaxAtoms];
+  __shared__ uint32_t s_list[kCtaWarps][64];
+  __shared__ uint16_t s_kept[kCtaWarps][kRecTile];
+  fill_pair_tables(s_pair);  // read after the first barrier below
+  const Tile tile = tiles[blockIdx.x / kSplit];
   const DevJob& J = jobs[tile.job];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool has_chain = warp < tile.count;
-  const int chain = tile.chain0 + warp;
+  const int in_tile = (blockIdx.x % kSplit) * kCtaWarps + warp;
+  const bool has_chain = in_tile < tile.count;
+  const int chain = tile.chain0 + in_tile;
   const LigView L = view_blob(J.blob);  // read through the cache; small
   const double* atom64 = reinterpret_cast<const double*>(J.blob + L.h->off_atom64);
   const double* body64 = reinterpret_cast<const double*>(J.blob + L.h->off_body64);
@@ -113,10 +190,21 @@ __global__ void __launch_bounds__(32 * kRescoreWarps) rescore_kernel(const DevJo
     type[0] = type[1] = 0;
     pos[0] = pos[1] = make_double3(0.0, 0.0, 0.0);
   }
-  // Inter, exact: for each receptor tile staged in shared memory, the warp scans
-  // (ligand atom, receptor atom) pairs with an FP32 pre-filter (cutoff + 0.05 A),
-  // compacts the survivors into a per-warp list by ballot, and evaluates them in
-  // FP64 32 at a time with every lane busy.
+  __syncthreads();  // the pair tables; each warp's coordinates
+  // the pose's bounding box, FP32
+  float3 lo = make_float3(3e38f, 3e38f, 3e38f), hi = make_float3(-3e38f, -3e38f, -3e38f);
+  for (int s = 0; s < 2; ++s)
+    if (valid[s]) {
+      const float x = (float)pos[s].x, y = (float)pos[s].y, z = (float)pos[s].z;
+      lo = make_float3(fminf(lo.x, x), fminf(lo.y, y), fminf(lo.z, z));
+      hi = make_float3(fmaxf(hi.x, x), fmaxf(hi.y, y), fmaxf(hi.z, z));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo.x = fminf(lo.x, __shfl_xor_sync(kFull, lo.x, o)), hi.x = fmaxf(hi.x, __shfl_xor_sync(kFull, hi.x, o));
+    lo.y = fminf(lo.y, __shfl_xor_sync(kFull, lo.y, o)), hi.y = fmaxf(hi.y, __shfl_xor_sync(kFull, hi.y, o));
+    lo.z = fminf(lo.z, __shfl_xor_sync(kFull, lo.z, o)), hi.z = fmaxf(hi.z, __shfl_xor_sync(kFull, hi.z, o));
+  }
   const float pre2 = (kCutoff + 0.05f) * (kCutoff + 0.05f);
   uint32_t* list = s_list[warp];
   int n_list = 0;
@@ -128,30 +216,43 @@ __global__ void __launch_bounds__(32 * kRescoreWarps) rescore_kernel(const DevJo
       const float4 a = s_rec[k];
       const double dx = s_xyz[warp][3 * i] - (double)a.x, dy = s_xyz[warp][3 * i + 1] - (double)a.y,
                    dz = s_xyz[warp][3 * i + 2] - (double)a.z;
-      const double r = sqrt(dx * dx + dy * dy + dz * dz);
-      if (r < kCutoffD) {
-        const int ti = s_type[warp][i], tj = min(__float_as_int(a.w), 8);
-        e_inter += vina_pair_f64(r - (c_xs_radius_d[ti] + c_xs_radius_d[tj]), pair_bits(ti, tj));
-      }
+      e_inter += pair_energy(fma(dx, dx, fma(dy, dy, dz * dz)), 9 * s_type[warp][i] + __float_as_int(a.w), s_pair);
     }
   };
   for (int r0 = 0; r0 < J.n_rec; r0 += kRecTile) {
     const int cnt = min(kRecTile, J.n_rec - r0);
     __syncthreads();
+#pragma unroll 4
     for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
       const int j = r0 + k;
       s_rec[k] = make_float4(J.rec_xyz[3 * j], J.rec_xyz[3 * j + 1], J.rec_xyz[3 * j + 2],
-                             __int_as_float((int)J.rec_type[j]));
+                             __int_as_float(min((int)J.rec_type[j], 8)));
     }
     __syncthreads();
     if (!has_chain) continue;
-    for (int i = 0; i < N; ++i) {
+    int n_kept = 0;
+    for (int k0 = 0; k0 < cnt; k0 += 32) {
+      const int k = k0 + lane;
+      bool keep = false;
+      if (k < cnt) {
+        const float4 a = s_rec[k];
+        const float fx = fmaxf(fmaxf(lo.x - a.x, a.x - hi.x), 0.f), fy = fmaxf(fmaxf(lo.y - a.y, a.y - hi.y), 0.f),
+                    fz = fmaxf(fmaxf(lo.z - a.z, a.z - hi.z), 0.f);
+        keep = fx * fx + fy * fy + fz * fz < pre2;
+      }
+      const unsigned bal = __ballot_sync(kFull, keep);
+      if (keep) s_kept[warp][n_kept + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)k;
+      n_kept += __popc(bal);
+    }
+    __syncwarp();
+    for (int i = 0; n_kept > 0 && i < N; ++i) {
       const float px = (float)s_xyz[warp][3 * i], py = (float)s_xyz[warp][3 * i + 1],
                   pz = (float)s_xyz[warp][3 * i + 2];
-      for (int k0 = 0; k0 < cnt; k0 += 32) {
-        const int k = k0 + lane;
+      for (int k0 = 0; k0 < n_kept; k0 += 32) {
         bool pass = false;
-        if (k < cnt) {
+        int k = 0;
+        if (k0 + lane < n_kept) {
+          k = s_kept[warp][k0 + lane];
           const float4 a = s_rec[k];
           const float fx = px - a.x, fy = py - a.y, fz = pz - a.z;
           pass = fx * fx + fy * fy + fz * fz < pre2;
@@ -183,10 +284,8 @@ __global__ void __launch_bounds__(32 * kRescoreWarps) rescore_kernel(const DevJo
     const int i = (pr & 0xffff) >> 4, j = pr >> 20;
     const double dx = s_xyz[warp][3 * i] - s_xyz[warp][3 * j], dy = s_xyz[warp][3 * i + 1] - s_xyz[warp][3 * j + 1],
                  dz = s_xyz[warp][3 * i + 2] - s_xyz[warp][3 * j + 2];
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    if (!(r < kCutoffD)) continue;
-    const int ti = __float_as_int(L.atom[i].w) & 0xff, tj = __float_as_int(L.atom[j].w) & 0xff;
-    e_intra += vina_pair_f64(r - (c_xs_radius_d[ti] + c_xs_radius_d[tj]), pair_bits(ti, tj));
+    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+    if (r2 < 65.0) e_intra += pair_energy(r2, 9 * s_type[warp][i] + s_type[warp][j], s_pair);
   }
   e_inter = warp_sum_d(e_inter);
   e_intra = warp_sum_d(e_intra);
@@ -300,7 +399,7 @@ __global__ void __launch_bounds__(512) topk_kernel(const DevJob* __restrict__ jo
 
 cudaError_t launch_rescore(const void* jobs, const void* tiles, int n_tiles, cudaStream_t st) {
   if (n_tiles <= 0) return cudaSuccess;
-  rescore_kernel<<<n_tiles, 32 * kRescoreWarps, 0, st>>>(reinterpret_cast<const DevJob*>(jobs),
+  rescore_kernel<<<n_tiles * kSplit, 32 * kCtaWarps, 0, st>>>(reinterpret_cast<const DevJob*>(jobs),
                                                          reinterpret_cast<const Tile*>(tiles));
   return cudaGetLastError();
 }
