@@ -50,6 +50,14 @@ struct LaneLig {
   int n_atoms, nb, T, tbody;
 };
 
+// Steps [0, n) may hold hydrophobic or H-bond pairs, [n, n_steps) hold none; n is
+// even.  (The steps with such pairs come first; bits 14 / 15 are the same in every lane.)
+__device__ __forceinline__ int ramp_steps(const LigView& L) {
+  int n = 0;
+  while (n < L.n_steps && ((L.steps[32 * n].x | L.steps[32 * n + 32].x) & 0xc000u)) n += 2;
+  return n;
+}
+
 template <int APL>
 __device__ __forceinline__ void load_lane_lig(const LigView& L, LaneLig<APL>& R) {
   const int lane = threadIdx.x & 31;
@@ -153,33 +161,96 @@ __device__ __forceinline__ void body_frames(const LigView& L, const Conf& c, Qua
   }
 }
 
-// Score and gradient of one conformation (all lanes return the same E;
-// lane j < 6 + T returns gradient component j, other lanes 0).  IU: how many
-// step pairs of the one-atom-per-lane intra loop are unrolled.
-template <int APL, int FMT, int IU = 2>
-__device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, const LaneLig<APL>& R,
-                                           const WarpScratch& W, const Conf& c, float& grad, uint32_t flags) {
-  const int lane = threadIdx.x & 31;
-  const int N = L.n_atoms, nb = L.n_bodies;
+// A conformation's atoms and body frames: lane b < n_bodies holds body b's frame,
+// every lane the atoms of its slots.
+template <int APL>
+struct Placed {
   Quat Q;
   float3 O;
-  body_frames(L, c, Q, O);
-  // ---- atom positions
   float3 pos[APL];
   int type[APL];
   int atom[APL];  // the slot's atom, -1 when empty
+};
+
+template <int APL>
+__device__ __forceinline__ void place_atoms(const LigView& L, const Conf& c, Placed<APL>& P) {
+  const int lane = threadIdx.x & 31;
+  body_frames(L, c, P.Q, P.O);
 #pragma unroll
   for (int s = 0; s < APL; ++s) {
-    atom[s] = APL == 1 ? (lane < N ? lane : -1) : (int)L.lane_map[2 * lane + s];
-    const int i = atom[s];
+    P.atom[s] = APL == 1 ? (lane < L.n_atoms ? lane : -1) : (int)L.lane_map[2 * lane + s];
+    const int i = P.atom[s];
     const float4 a = L.atom[i >= 0 ? i : 0];
     const int packed = __float_as_int(a.w);
-    type[s] = packed & 0xff;
+    P.type[s] = packed & 0xff;
     const int b = i >= 0 ? (packed >> 8) & 0xff : 0;
-    const Quat Qb = shflq(Q, b);
-    const float3 Ob = shfl3(O, b);
-    pos[s] = Ob + qrot(Qb, make_float3(a.x, a.y, a.z));
+    const Quat Qb = shflq(P.Q, b);
+    const float3 Ob = shfl3(P.O, b);
+    P.pos[s] = Ob + qrot(Qb, make_float3(a.x, a.y, a.z));
   }
+}
+
+// Energy of a placed conformation (all lanes return the same), without its
+// gradient: a BFGS line search rejects three of four trial points and needs
+// nothing else of those.  The operations that make up the energy, and their
+// order, are score_placed's: both return the same bits.
+template <int APL, int FMT, int IU = 2>
+__device__ __forceinline__ float energy_placed(const MapView& M, const LigView& L, int n_ramp, const Placed<APL>& P) {
+  const int lane = threadIdx.x & 31;
+  const uint2* tab = L.steps + lane;
+  float2 e_pair = make_float2(0.f, 0.f);
+  const float2 px = splat2(P.pos[0].x), py = splat2(P.pos[0].y), pz = splat2(P.pos[0].z);
+  auto pass = [&](int st, bool ramp) {
+    const uint2 t0 = tab[st * 32], t1 = tab[st * 32 + 32];
+    float2 dx, dy, dz;
+    if (APL == 1) {
+      const float3 b0 = shfl3(P.pos[0], (int)t0.x), b1 = shfl3(P.pos[0], (int)t1.x);
+      dx = __ffma2_rn(make_float2(b0.x, b1.x), splat2(-1.f), px);
+      dy = __ffma2_rn(make_float2(b0.y, b1.y), splat2(-1.f), py);
+      dz = __ffma2_rn(make_float2(b0.z, b1.z), splat2(-1.f), pz);
+    } else {
+      const float3 a0 = t0.x & (1u << 10) ? P.pos[APL - 1] : P.pos[0], a1 = t1.x & (1u << 10) ? P.pos[APL - 1] : P.pos[0];
+      const float3 s0 = t0.x & (1u << 11) ? P.pos[APL - 1] : P.pos[0], s1 = t1.x & (1u << 11) ? P.pos[APL - 1] : P.pos[0];
+      const float3 b0 = shfl3(s0, (int)t0.x), b1 = shfl3(s1, (int)t1.x);
+      dx = make_float2(a0.x - b0.x, a1.x - b1.x);
+      dy = make_float2(a0.y - b0.y, a1.y - b1.y);
+      dz = make_float2(a0.z - b0.z, a1.z - b1.z);
+    }
+    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+    const uint32_t both = t0.x | t1.x;
+    e_pair = __fadd2_rn(e_pair, vina_energy_x2(r2, make_float2(__uint_as_float(t0.y), __uint_as_float(t1.y)),
+                                               t0.x >> 12, t1.x >> 12, ramp && ((both >> 14) & 1),
+                                               ramp && ((both >> 15) & 1)));
+  };
+  int st = 0;
+#pragma unroll 1
+  for (; st < n_ramp; st += 2) pass(st, true);
+#pragma unroll (APL == 1 ? IU : 1)
+  for (; st < L.n_steps; st += 2) pass(st, false);
+  float e_lane = 0.f;
+  e_lane += e_pair.x + e_pair.y;
+#pragma unroll
+  for (int s = 0; s < APL; ++s)
+    if (P.atom[s] >= 0) e_lane += map_energy<FMT>(M, P.type[s], map_cell(M, P.pos[s]));
+  return warp_sum(e_lane);
+}
+
+// Score and gradient of a placed conformation c (all lanes return the same E;
+// lane j < 6 + T returns gradient component j, other lanes 0).  IU: how many
+// step pairs of the one-atom-per-lane intra loop are unrolled.
+template <int APL, int FMT, int IU = 2>
+__device__ __forceinline__ float score_placed(const MapView& M, const LigView& L, const LaneLig<APL>& R,
+                                              int n_ramp, const WarpScratch& W, const Conf& c, const Placed<APL>& P,
+                                              float& grad, uint32_t flags) {
+  const int lane = threadIdx.x & 31;
+  const int N = L.n_atoms, nb = L.n_bodies;
+  const Quat Q = P.Q;
+  const float3 O = P.O;
+  float3 pos[APL];
+  int type[APL];
+  int atom[APL];
+#pragma unroll
+  for (int s = 0; s < APL; ++s) pos[s] = P.pos[s], type[s] = P.type[s], atom[s] = P.atom[s];
   float e_lane = 0.f;
   float3 g[APL];
 #pragma unroll
@@ -195,11 +266,10 @@ __device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, c
       // packed accumulators: component .x collects the even steps, .y the odd ones
       const float2 px = splat2(pos[0].x), py = splat2(pos[0].y), pz = splat2(pos[0].z);
       float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
-      // unrolled (IU = 2): the shuffles of one step pair overlap the arithmetic of
-      // the next; four measured slower, and the kernel that holds both tiles
-      // (more live registers) runs faster without unrolling
-#pragma unroll IU
-      for (int st = 0; st < L.n_steps; st += 2) {
+      // A pass takes two steps.  The passes with hydrophobic or H-bond pairs come
+      // first; the others have no branch, so that unrolled (IU passes) the shuffles of
+      // one overlap the arithmetic of the next.
+      auto pass = [&](int st, bool ramp) {
         const uint2 t0 = tab[st * 32], t1 = tab[st * 32 + 32];
         // shfl.idx reads the source lane from bits 0-4 only: the entry's partner field
         const float3 b0 = shfl3(pos[0], (int)t0.x), b1 = shfl3(pos[0], (int)t1.x);
@@ -210,7 +280,7 @@ __device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, c
         const uint32_t both = t0.x | t1.x;  // bits 14 / 15: warp-uniform
         float2 e, sp;
         vina_pair_x2(r2, make_float2(__uint_as_float(t0.y), __uint_as_float(t1.y)), t0.x >> 12, t1.x >> 12,
-                     (both >> 14) & 1, (both >> 15) & 1, e, sp);
+                     ramp && ((both >> 14) & 1), ramp && ((both >> 15) & 1), e, sp);
         e_pair = __fadd2_rn(e_pair, e);
         const float2 fx = __fmul2_rn(sp, dx), fy = __fmul2_rn(sp, dy), fz = __fmul2_rn(sp, dz);
         // reaction forces of the pairs this lane is passive in (source lane: bits 5-9)
@@ -219,13 +289,17 @@ __device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, c
         ax = __ffma2_rn(make_float2(c0.x, c1.x), splat2(-1.f), __fadd2_rn(ax, fx));
         ay = __ffma2_rn(make_float2(c0.y, c1.y), splat2(-1.f), __fadd2_rn(ay, fy));
         az = __ffma2_rn(make_float2(c0.z, c1.z), splat2(-1.f), __fadd2_rn(az, fz));
-      }
+      };
+      int st = 0;
+#pragma unroll 1
+      for (; st < n_ramp; st += 2) pass(st, true);
+#pragma unroll IU
+      for (; st < L.n_steps; st += 2) pass(st, false);
       g[0].x += ax.x + ax.y;
       g[0].y += ay.x + ay.y;
       g[0].z += az.x + az.y;
     } else {
-#pragma unroll 1
-      for (int st = 0; st < L.n_steps; st += 2) {
+      auto pass = [&](int st, bool ramp) {
         const uint2 t0 = tab[st * 32], t1 = tab[st * 32 + 32];
         const bool ac0 = t0.x & (1u << 10), ac1 = t1.x & (1u << 10);
         const bool pc0 = t0.x & (1u << 11), pc1 = t1.x & (1u << 11);
@@ -239,7 +313,7 @@ __device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, c
         const uint32_t both = t0.x | t1.x;
         float2 e, sp;
         vina_pair_x2(r2, make_float2(__uint_as_float(t0.y), __uint_as_float(t1.y)), t0.x >> 12, t1.x >> 12,
-                     (both >> 14) & 1, (both >> 15) & 1, e, sp);
+                     ramp && ((both >> 14) & 1), ramp && ((both >> 15) & 1), e, sp);
         e_pair = __fadd2_rn(e_pair, e);
         const float2 fx = __fmul2_rn(sp, dx), fy = __fmul2_rn(sp, dy), fz = __fmul2_rn(sp, dz);
         const float3 c0 = shfl3(make_float3(fx.x, fy.x, fz.x), (int)(t0.x >> 5));
@@ -253,7 +327,12 @@ __device__ __forceinline__ float eval_conf(const MapView& M, const LigView& L, c
         else g[0].x -= c0.x, g[0].y -= c0.y, g[0].z -= c0.z;
         if (pc1) g[APL - 1].x -= c1.x, g[APL - 1].y -= c1.y, g[APL - 1].z -= c1.z;
         else g[0].x -= c1.x, g[0].y -= c1.y, g[0].z -= c1.z;
-      }
+      };
+      int st = 0;
+#pragma unroll 1
+      for (; st < n_ramp; st += 2) pass(st, true);
+#pragma unroll 1
+      for (; st < L.n_steps; st += 2) pass(st, false);
     }
     e_lane += e_pair.x + e_pair.y;
   }
@@ -551,6 +630,7 @@ struct ChainVars {
   uint32_t evals;
   int T;
   int bb, max_iters;
+  int n_ramp;
   int chain;
   int stop;  // MC step at which this run of the chain ends (n_steps + 1: the chain's end)
   const DevJob* job;
@@ -599,6 +679,7 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
     V.T = T;
     V.bb = J.optimizer == DSDP_OPT_BB;
     V.max_iters = J.n_opt_iters;
+    V.n_ramp = ramp_steps(L);
     V.chain = chain;
     V.job = &J;
     V.step = first;
@@ -675,41 +756,66 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       }
       mutate = false;
     }
-    float gn;
-    const float en = eval_conf<APL, FMT, IU>(M, REVIEW ? view_blob(reinterpret_cast<const uint8_t*>(L.h)) : L, R, W,
-                                             xt, gn, DSDP_TERM_ALL);
-    const int T = V.T, nx = 7 + T, D = 6 + T;
-    const bool bb = V.bb;
-    const int max_iters = V.max_iters;
-    int phase = V.phase, it = V.it, trial = V.trial;
-    float e = V.e, gd = V.gd, alpha = V.alpha, e_opt_best = V.e_opt_best;
-    float g = lane < kHStride ? Vg[lane] : 0.f, dir = lane < kHStride ? Vd[lane] : 0.f;
-    const uint32_t evals = V.evals + 1;
-    bool done = false;
-    if (phase == kStart) {  // first evaluation of a local optimisation
-      e = en;
-      g = gn;
-      store_conf(W.x, xt, T);
-      if (max_iters == 0) {
-        done = true;
-      } else if (!bb) {
-        bfgs_reset(W, D);
-        dir = -g;  // H0 = I
-        gd = -warp_sum(g * g);
-        it = trial = 0;
-        alpha = 1.f;
-        xt = apply_step(xt, dir, T);
-        phase = kTrial;
-      } else {
-        e_opt_best = e;
-        alpha = kBBAlpha0;
-        it = 0;
-        dir = -alpha * g;
-        xt = apply_step(xt, dir, T);
-        phase = kBB;
+    bool done = false;  // the local optimisation ends with this evaluation
+    Placed<APL> P;
+    const LigView Lv = REVIEW ? view_blob(reinterpret_cast<const uint8_t*>(L.h)) : L;
+    place_atoms<APL>(Lv, xt, P);
+    int phase = V.phase;
+    if (phase == kTrial) {
+      // BFGS: Armijo test of the trial point x + alpha d on its energy alone; its
+      // gradient is evaluated when it is accepted (27 % of first trials, 23 % of all)
+      const float en = energy_placed<APL, FMT, IU>(M, Lv, V.n_ramp, P);
+      const float e = V.e, gd = V.gd;
+      float alpha = V.alpha;
+      if (!(en <= e + kArmijoC1 * alpha * gd)) {
+        const int T = V.T, trial = V.trial + 1;
+        V.evals = V.evals + 1;
+        if (trial < kMaxTrials) {
+          alpha *= kShrink;
+          V.alpha = alpha;
+          V.trial = trial;
+          const float dir = lane < kHStride ? Vd[lane] : 0.f;
+          xt = apply_step(load_conf(W.x, T), alpha * dir, T);
+          __syncwarp();
+          continue;
+        }
+        done = true;  // no acceptable step: the optimisation ends at the current iterate
       }
-    } else if (phase == kTrial) {  // BFGS: Armijo test of the trial point x + alpha d
-      if (en <= e + kArmijoC1 * alpha * gd) {
+    }
+    if (!done) {
+      float gn;
+      const float en = score_placed<APL, FMT, IU>(M, Lv, R, V.n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
+      const int T = V.T, D = 6 + T;
+      const int max_iters = V.max_iters;
+      phase = V.phase;
+      int it = V.it;
+      float e_opt_best = V.e_opt_best;
+      float e = V.e, gd = V.gd, alpha = V.alpha;
+      float g = lane < kHStride ? Vg[lane] : 0.f, dir = lane < kHStride ? Vd[lane] : 0.f;
+      if (phase == kStart) {  // first evaluation of a local optimisation
+        e = en;
+        g = gn;
+        store_conf(W.x, xt, T);
+        if (max_iters == 0) {
+          done = true;
+        } else if (!V.bb) {
+          bfgs_reset(W, D);
+          dir = -g;  // H0 = I
+          gd = -warp_sum(g * g);
+          it = 0;
+          alpha = 1.f;
+          V.trial = 0;
+          xt = apply_step(xt, dir, T);
+          phase = kTrial;
+        } else {
+          e_opt_best = e;
+          alpha = kBBAlpha0;
+          it = 0;
+          dir = -alpha * g;
+          xt = apply_step(xt, dir, T);
+          phase = kBB;
+        }
+      } else if (phase == kTrial) {  // BFGS: an accepted trial point
         const float s = alpha * dir, y = gn - g;
         g = gn;
         e = en;
@@ -720,37 +826,44 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
           dir = bfgs_update(W, D, s, y, gn, dir);
           gd = warp_sum(g * dir);  // computed directly: the sufficient-decrease test must see the true slope
           alpha = 1.f;
-          trial = 0;
+          V.trial = 0;
           xt = apply_step(xt, dir, T);
         }
-      } else {
-        alpha *= kShrink;
-        if (++trial == kMaxTrials) {
-          done = true;  // no acceptable step: the optimisation ends at the current iterate
+      } else {  // BB: x_{k+1} = x_k + s_k evaluated; next step length from s.s / s.y
+        const float sy = warp_sum(dir * (gn - g));
+        const float ss = warp_sum(dir * dir);
+        alpha = sy > 0.f ? fminf(fmaxf(ss / sy, kBBAlphaMin), kBBAlphaMax) : kBBAlphaMax;
+        g = gn;
+        if (en < e_opt_best) {
+          e_opt_best = en;
+          store_conf(W.x, xt, T);
+        }
+        if (++it == max_iters) {
+          done = true;
         } else {
-          __syncwarp();
-          xt = apply_step(load_conf(W.x, T), alpha * dir, T);
+          dir = -alpha * g;
+          xt = apply_step(xt, dir, T);
         }
       }
-    } else {  // BB: x_{k+1} = x_k + s_k evaluated; next step length from s.s / s.y
-      const float sy = warp_sum(dir * (gn - g));
-      const float ss = warp_sum(dir * dir);
-      alpha = sy > 0.f ? fminf(fmaxf(ss / sy, kBBAlphaMin), kBBAlphaMax) : kBBAlphaMax;
-      g = gn;
-      if (en < e_opt_best) {
-        e_opt_best = en;
-        store_conf(W.x, xt, T);
+      V.evals = V.evals + 1;
+      V.phase = phase;
+      V.it = it;
+      V.e = e;
+      V.gd = gd;
+      V.alpha = alpha;
+      V.e_opt_best = e_opt_best;
+      if (lane < kHStride) {
+        Vg[lane] = g;
+        Vd[lane] = dir;
       }
-      if (++it == max_iters) {
-        done = true;
-      } else {
-        dir = -alpha * g;
-        xt = apply_step(xt, dir, T);
-      }
+      __syncwarp();
     }
     if (__builtin_expect(done, 0)) {
       // ---- local optimisation finished: its result is W.x with energy eo
-      const float eo = (bb && max_iters > 0) ? e_opt_best : e;
+      __syncwarp();
+      const int T = V.T, nx = 7 + T;
+      const uint32_t evals = V.evals;
+      const float eo = (V.bb && V.max_iters > 0) ? V.e_opt_best : V.e;
       // (the job record is read again here rather than held across the evaluations)
       const DevJob& job = *V.job;
       const int chain_id = V.chain;
@@ -826,24 +939,12 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         return;
       }
       mutate = true;
-      phase = kStart;
+      V.phase = kStart;
       V.step = step;
       V.e_cur = e_cur;
       V.e_best = e_best;
+      __syncwarp();
     }
-    V.phase = phase;
-    V.it = it;
-    V.trial = trial;
-    V.e = e;
-    V.gd = gd;
-    V.alpha = alpha;
-    V.e_opt_best = e_opt_best;
-    V.evals = evals;
-    if (lane < kHStride) {
-      Vg[lane] = g;
-      Vd[lane] = dir;
-    }
-    __syncwarp();
   }
 }
 

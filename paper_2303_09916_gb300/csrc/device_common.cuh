@@ -245,6 +245,35 @@ __device__ __forceinline__ void vina_pair_x2(float2 r2, float2 nrs, uint32_t cls
   s = __fmul2_rn(de, ir);
 }
 
+// The energy of vina_pair_x2 alone, by the same operations.
+__device__ __forceinline__ float2 vina_energy_x2(float2 r2, float2 nrs, uint32_t cls0, uint32_t cls1, bool use_hyd,
+                                                 bool use_hb) {
+  const float2 rp = __fadd2_rn(r2, splat2(1e-30f));
+  const float2 ir = make_float2(rsqrt_ftz(rp.x), rsqrt_ftz(rp.y));
+  float2 d = __ffma2_rn(r2, ir, nrs);
+  d.x = r2.x < kCutoff * kCutoff ? d.x : kFarD;
+  d.y = r2.y < kCutoff * kCutoff ? d.y : kFarD;
+  const float2 u1 = __fmul2_rn(__fmul2_rn(d, d), splat2(-4.f * kLog2E));
+  const float2 b = __ffma2_rn(d, splat2(0.5f), splat2(-1.5f));
+  const float2 u2 = __fmul2_rn(__fmul2_rn(b, b), splat2(-kLog2E));
+  const float2 g1 = make_float2(ex2_approx(u1.x), ex2_approx(u1.y));
+  const float2 g2 = make_float2(ex2_approx(u2.x), ex2_approx(u2.y));
+  const float2 m = make_float2(fminf(d.x, 0.f), fminf(d.y, 0.f));
+  float2 e = __ffma2_rn(g2, splat2(kWGauss2), __fmul2_rn(g1, splat2(kWGauss1)));
+  e = __ffma2_rn(__fmul2_rn(m, m), splat2(kWRepulsion), e);
+  if (use_hyd) {
+    const float2 wh = make_float2((cls0 & 1u) ? kWHydrophobic : 0.f, (cls1 & 1u) ? kWHydrophobic : 0.f);
+    const float2 t = __ffma2_rn(d, splat2(-1.f), splat2(1.5f));
+    e = __ffma2_rn(wh, make_float2(__saturatef(t.x), __saturatef(t.y)), e);
+  }
+  if (use_hb) {
+    const float2 wb = make_float2((cls0 & 2u) ? kWHBond : 0.f, (cls1 & 2u) ? kWHBond : 0.f);
+    const float2 t = __fmul2_rn(d, splat2(-1.f / 0.7f));
+    e = __ffma2_rn(wb, make_float2(__saturatef(t.x), __saturatef(t.y)), e);
+  }
+  return e;
+}
+
 __device__ __forceinline__ int pair_bits(int ti, int tj) {
   const int a = c_xs_bits[ti], b = c_xs_bits[tj];
   int bits = (a & b & 1);
@@ -285,6 +314,15 @@ __device__ __forceinline__ float4 load_node(const void* maps, unsigned idx) {
     else v = __half2float(__ushort_as_half(raw));
     return make_float4(v, 0.f, 0.f, 0.f);
   }
+}
+
+// The score of a node alone.
+template <int FMT>
+__device__ __forceinline__ float load_score(const void* maps, unsigned idx) {
+  if (FMT == 0) return __ldg(reinterpret_cast<const float*>(maps) + 4 * (size_t)idx);
+  if (FMT == 1) return __bfloat162float(__ushort_as_bfloat16(__ldg(reinterpret_cast<const unsigned short*>(maps) + 4 * (size_t)idx)));
+  if (FMT == 2) return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(maps) + 4 * (size_t)idx)));
+  return load_node<FMT>(maps, idx).x;
 }
 
 struct MapView {
@@ -375,6 +413,27 @@ __device__ __forceinline__ float map_interp(const MapView& M, int t, const MapCe
     e += kWallSlope * fabsf(c.ez);
     g.z = c.ez > 0.f ? kWallSlope : -kWallSlope;
   }
+  return e;
+}
+
+// The score of map_interp alone, by the same operations.
+template <int FMT>
+__device__ __forceinline__ float map_energy(const MapView& M, int t, const MapCell& c) {
+  const unsigned sxy = (unsigned)M.nx * (unsigned)M.ny;
+  const unsigned base = (unsigned)t * sxy * (unsigned)M.nz + c.base;
+  const float v000 = load_score<FMT>(M.maps, base), v100 = load_score<FMT>(M.maps, base + 1);
+  const float v010 = load_score<FMT>(M.maps, base + M.nx), v110 = load_score<FMT>(M.maps, base + M.nx + 1);
+  const float v001 = load_score<FMT>(M.maps, base + sxy), v101 = load_score<FMT>(M.maps, base + sxy + 1);
+  const float v011 = load_score<FMT>(M.maps, base + sxy + M.nx), v111 = load_score<FMT>(M.maps, base + sxy + M.nx + 1);
+  const float fx = c.fx, fy = c.fy, fz = c.fz;
+  const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
+  const float w000 = gx0 * gy0 * gz0, w100 = fx * gy0 * gz0, w010 = gx0 * fy * gz0, w110 = fx * fy * gz0;
+  const float w001 = gx0 * gy0 * fz, w101 = fx * gy0 * fz, w011 = gx0 * fy * fz, w111 = fx * fy * fz;
+  float e = w000 * v000 + w100 * v100 + w010 * v010 + w110 * v110 + w001 * v001 + w101 * v101 + w011 * v011 +
+            w111 * v111;
+  if (c.ex != 0.f) e += kWallSlope * fabsf(c.ex);
+  if (c.ey != 0.f) e += kWallSlope * fabsf(c.ey);
+  if (c.ez != 0.f) e += kWallSlope * fabsf(c.ez);
   return e;
 }
 

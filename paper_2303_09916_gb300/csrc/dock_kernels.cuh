@@ -94,10 +94,9 @@ static __device__ __noinline__ int queue_next(const ChainQueue& q, int n_tiles) 
   }
 }
 
-template <int FMT, int VAR, int APLS>
-__global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>())) dock_chains_kernel(const DevJob* __restrict__ jobs,
-                                                          const Tile* __restrict__ tiles, int n_tiles,
-                                                          ChainQueue queue, int blob_smem, ScratchLayout lay) {
+template <int FMT, int APLS, int IU, bool REVIEW>
+__device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles,
+                                          const ChainQueue& queue, int blob_smem, const ScratchLayout& lay) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int s_tile;
   __shared__ int s_job;
@@ -134,9 +133,8 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
         sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
         sl.steps = J.slice_steps;
       }
-      constexpr bool kReview = APLS == 3 && VAR == 1;
-      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, APLS == 3 ? 1 : 2, kReview>(J, L, W, chain, sl);
-      else run_chain<2, FMT, 2, kReview>(J, L, W, chain, sl);
+      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, IU, REVIEW>(J, L, W, chain, sl);
+      else run_chain<2, FMT, IU, REVIEW>(J, L, W, chain, sl);
     }
     if (!queue.n_items) break;
     __syncthreads();
@@ -148,6 +146,13 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
   }
   // what follows on the stream follows this launch: it ends after the group before it
   if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <int FMT, int VAR, int APLS>
+__global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>()))
+    dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
+                       int blob_smem, ScratchLayout lay) {
+  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
 // Score + gradient of a batch of conformations: one warp per conformation,
@@ -168,12 +173,15 @@ __global__ void __launch_bounds__(256) score_eval_kernel(MapView M, const uint8_
   LaneLig<APL> R;
   load_lane_lig<APL>(L, R);
   const int T = L.T;
+  const int n_ramp = ramp_steps(L);
   const int warps = gridDim.x * (blockDim.x >> 5);
   for (int c = blockIdx.x * (blockDim.x >> 5) + warp; c < n_conf; c += warps) {  // warp-uniform loop
     Conf x = load_conf(conf + (size_t)c * (7 + T), T);
     x.q = qnormalize(x.q);
     float g;
-    const float e = eval_conf<APL, FMT>(M, L, R, W, x, g, flags);
+    Placed<APL> P;
+    place_atoms<APL>(L, x, P);
+    const float e = score_placed<APL, FMT>(M, L, R, n_ramp, W, x, P, g, flags);
     if (lane == 0 && energy) energy[c] = e;
     if (grad && lane < 6 + T) grad[(size_t)c * (6 + T) + lane] = g;
   }
