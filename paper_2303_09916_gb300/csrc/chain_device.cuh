@@ -237,8 +237,11 @@ __device__ __forceinline__ float energy_placed(const MapView& M, const LigView& 
 
 // Score and gradient of a placed conformation c (all lanes return the same E;
 // lane j < 6 + T returns gradient component j, other lanes 0).  IU: how many
-// step pairs of the one-atom-per-lane intra loop are unrolled.
-template <int APL, int FMT, int IU = 2>
+// step pairs of the one-atom-per-lane intra loop are unrolled.  FLAT: the passes that
+// may hold hydrophobic or H-bond pairs compute both terms for all (with weight 0
+// where a pair has none: the same bits) instead of branching, and are unrolled too --
+// more instructions, a shorter way through them.
+template <int APL, int FMT, int IU = 2, bool FLAT = false>
 __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L, const LaneLig<APL>& R,
                                               int n_ramp, const WarpScratch& W, const Conf& c, const Placed<APL>& P,
                                               float& grad, uint32_t flags) {
@@ -280,7 +283,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         const uint32_t both = t0.x | t1.x;  // bits 14 / 15: warp-uniform
         float2 e, sp;
         vina_pair_x2(r2, make_float2(__uint_as_float(t0.y), __uint_as_float(t1.y)), t0.x >> 12, t1.x >> 12,
-                     ramp && ((both >> 14) & 1), ramp && ((both >> 15) & 1), e, sp);
+                     ramp && (FLAT || ((both >> 14) & 1)), ramp && (FLAT || ((both >> 15) & 1)), e, sp);
         e_pair = __fadd2_rn(e_pair, e);
         const float2 fx = __fmul2_rn(sp, dx), fy = __fmul2_rn(sp, dy), fz = __fmul2_rn(sp, dz);
         // reaction forces of the pairs this lane is passive in (source lane: bits 5-9)
@@ -291,7 +294,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         az = __ffma2_rn(make_float2(c0.z, c1.z), splat2(-1.f), __fadd2_rn(az, fz));
       };
       int st = 0;
-#pragma unroll 1
+#pragma unroll (FLAT ? 2 : 1)
       for (; st < n_ramp; st += 2) pass(st, true);
 #pragma unroll IU
       for (; st < L.n_steps; st += 2) pass(st, false);
@@ -313,7 +316,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         const uint32_t both = t0.x | t1.x;
         float2 e, sp;
         vina_pair_x2(r2, make_float2(__uint_as_float(t0.y), __uint_as_float(t1.y)), t0.x >> 12, t1.x >> 12,
-                     ramp && ((both >> 14) & 1), ramp && ((both >> 15) & 1), e, sp);
+                     ramp && (FLAT || ((both >> 14) & 1)), ramp && (FLAT || ((both >> 15) & 1)), e, sp);
         e_pair = __fadd2_rn(e_pair, e);
         const float2 fx = __fmul2_rn(sp, dx), fy = __fmul2_rn(sp, dy), fz = __fmul2_rn(sp, dz);
         const float3 c0 = shfl3(make_float3(fx.x, fy.x, fz.x), (int)(t0.x >> 5));
@@ -329,9 +332,9 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         else g[0].x -= c1.x, g[0].y -= c1.y, g[0].z -= c1.z;
       };
       int st = 0;
-#pragma unroll 1
+#pragma unroll (FLAT ? 2 : 1)
       for (; st < n_ramp; st += 2) pass(st, true);
-#pragma unroll 1
+#pragma unroll (FLAT ? 2 : 1)
       for (; st < L.n_steps; st += 2) pass(st, false);
     }
     e_lane += e_pair.x + e_pair.y;
@@ -639,6 +642,119 @@ struct ChainVars {
 };
 static_assert(sizeof(ChainVars) <= 4 * kVarWords, "ChainVars must fit its words of the vec area");
 
+// The drawn start of a chain.
+__device__ __forceinline__ Conf draw_start(const DevJob& J, int T, int chain) {
+  const int lane = threadIdx.x & 31;
+  const ChainStream rs{J.seed_lo, J.seed_hi, (uint32_t)chain};
+  Conf xt;
+  // initial conformation: uniform word n of step 0 is word n % 4 of block n / 4
+  const uint4 b0 = rs.block(0, 0), b1 = rs.block(0, 1);
+  xt.p = make_float3(__fmaf_rn(J.box_size[0], ChainStream::to_uniform(b0.x), J.box_lo[0]),
+                     __fmaf_rn(J.box_size[1], ChainStream::to_uniform(b0.y), J.box_lo[1]),
+                     __fmaf_rn(J.box_size[2], ChainStream::to_uniform(b0.z), J.box_lo[2]));
+  if (J.n_sites > 0) xt.p = site_start(J, rs, xt.p);
+  const float u1 = ChainStream::to_uniform(b0.w), u2 = ChainStream::to_uniform(b1.x),
+              u3 = ChainStream::to_uniform(b1.y);
+  float s2, c2, s3, c3;
+  sincosf(kTwoPiF * u2, &s2, &c2);
+  sincosf(kTwoPiF * u3, &s3, &c3);
+  const float a = sqrtf(1.f - u1), b = sqrtf(u1);
+  xt.q = Quat{b * c3, a * s2, a * c2, b * s3};
+  float th = 0.f;
+  if (lane >= 6 && lane < 6 + T) {
+    const uint4 bk = rs.block(0, (uint32_t)(lane >> 2));
+    th = kPiF - kTwoPiF * ChainStream::to_uniform(pick(bk, lane & 3));
+  }
+  xt.th = th;
+  return xt;
+}
+
+// The chain's current conformation (W.cur) mutated for MC step `step`: the start of
+// its local optimisation.
+__device__ __forceinline__ Conf mutated_conf(const DevJob& job, const LigView& L, const WarpScratch& W, int chain,
+                                             uint32_t step, int T) {
+  const int lane = threadIdx.x & 31;
+  const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)chain};
+  const uint4 w0 = rs.block(step, 0);
+  const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
+  Conf xt = load_conf(W.cur, T);
+  if (mode == 0) {
+    const float3 b = unit_ball(rs, step);
+    xt.p = xt.p + kMutationAmplitude * b;
+  } else if (mode == 1) {
+    const float3 b = unit_ball(rs, step);
+    const float k = kMutationAmplitude * (1.f / L.h->gyration_radius);
+    xt.q = qnormalize(qmul(quat_from_rotvec(k * b.x, k * b.y, k * b.z), xt.q));
+  } else if (lane == 6 + (mode - 2)) {
+    xt.th = kPiF - kTwoPiF * ChainStream::to_uniform(w0.z);
+  }
+  return xt;
+}
+
+// End of MC step `step`: Metropolis test of the optimised conformation W.x with
+// energy eo, the chain's current and best conformations, and the trace (by one
+// warp of the chain, `writer`).
+__device__ __forceinline__ void metropolis_step(const DevJob& job, const WarpScratch& W, int chain, int step, int T,
+                                                float eo, float& e_cur, float& e_best, bool writer) {
+  const int lane = threadIdx.x & 31;
+  const int nx = 7 + T;
+  const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)chain};
+  const size_t trace_stride = (size_t)nx + 4;
+  float* const trace =
+      job.trace && writer ? job.trace + (size_t)chain * (job.n_steps + 1) * trace_stride : nullptr;
+  if (step == 0) {
+    e_cur = e_best = eo;
+    if (lane < nx) {
+      W.cur[lane] = W.x[lane];
+      W.best[lane] = W.x[lane];
+    }
+    if (trace && !job.trace_starts) {
+      if (lane < nx) trace[lane] = W.x[lane];
+      if (lane == 0) {
+        trace[nx + 0] = e_cur;
+        trace[nx + 1] = e_cur;
+        trace[nx + 2] = -1.f;
+        trace[nx + 3] = 1.f;
+      }
+    }
+  } else {
+    const uint4 w0 = rs.block((uint32_t)step, 0);
+    const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
+    const float u = ChainStream::to_uniform(w0.y);
+    const bool accept = (eo < e_cur) || (u < expf(-(eo - e_cur) / job.temperature));
+    if (accept) {
+      e_cur = eo;
+      if (lane < nx) W.cur[lane] = W.x[lane];
+      if (eo < e_best) {
+        e_best = eo;
+        if (lane < nx) W.best[lane] = W.x[lane];
+      }
+    }
+    if (trace) {
+      float* t = trace + (size_t)step * trace_stride;
+      if (lane < nx) t[lane] = W.cur[lane];
+      if (lane == 0) {
+        t[nx + 0] = eo;
+        t[nx + 1] = e_cur;
+        t[nx + 2] = (float)mode;
+        t[nx + 3] = accept ? 1.f : 0.f;
+      }
+    }
+  }
+}
+
+// Row 0 of a trace that records starts: the drawn one, before any optimisation.
+__device__ __forceinline__ void trace_start(const DevJob& J, int chain, const Conf& c, int T) {
+  float* t = J.trace + (size_t)chain * (J.n_steps + 1) * ((size_t)7 + T + 4);
+  store_conf(t, c, T);
+  if ((threadIdx.x & 31) == 0) {
+    t[7 + T + 0] = 0.f;
+    t[7 + T + 1] = 0.f;
+    t[7 + T + 2] = -2.f;
+    t[7 + T + 3] = 0.f;
+  }
+}
+
 // One Monte Carlo chain (Sec. 2: one of many short independent copies; Vina's
 // mutation and Metropolis rules) with its local optimisations -- BFGS with
 // Armijo backtracking (Vina's optimiser; Nocedal & Wright Alg. 6.1) or
@@ -702,58 +818,13 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
   }
   if (!mutate) {
     const int T = L.T;
-    const ChainStream rs{J.seed_lo, J.seed_hi, (uint32_t)chain};
-    // initial conformation: uniform word n of step 0 is word n % 4 of block n / 4
-    const uint4 b0 = rs.block(0, 0), b1 = rs.block(0, 1);
-    xt.p = make_float3(__fmaf_rn(J.box_size[0], ChainStream::to_uniform(b0.x), J.box_lo[0]),
-                       __fmaf_rn(J.box_size[1], ChainStream::to_uniform(b0.y), J.box_lo[1]),
-                       __fmaf_rn(J.box_size[2], ChainStream::to_uniform(b0.z), J.box_lo[2]));
-    if (J.n_sites > 0) xt.p = site_start(J, rs, xt.p);
-    const float u1 = ChainStream::to_uniform(b0.w), u2 = ChainStream::to_uniform(b1.x),
-                u3 = ChainStream::to_uniform(b1.y);
-    float s2, c2, s3, c3;
-    sincosf(kTwoPiF * u2, &s2, &c2);
-    sincosf(kTwoPiF * u3, &s3, &c3);
-    const float a = sqrtf(1.f - u1), b = sqrtf(u1);
-    xt.q = Quat{b * c3, a * s2, a * c2, b * s3};
-    float th = 0.f;
-    if (lane >= 6 && lane < 6 + T) {
-      const uint4 bk = rs.block(0, (uint32_t)(lane >> 2));
-      th = kPiF - kTwoPiF * ChainStream::to_uniform(pick(bk, lane & 3));
-    }
-    xt.th = th;
-    if (J.trace && J.trace_starts) {  // row 0: the drawn start, before any optimisation
-      float* t = J.trace + (size_t)chain * (J.n_steps + 1) * ((size_t)7 + T + 4);
-      store_conf(t, xt, T);
-      if (lane == 0) {
-        t[7 + T + 0] = 0.f;
-        t[7 + T + 1] = 0.f;
-        t[7 + T + 2] = -2.f;
-        t[7 + T + 3] = 0.f;
-      }
-    }
+    xt = draw_start(J, T, chain);
+    if (J.trace && J.trace_starts) trace_start(J, chain, xt, T);
   }
   __syncwarp();
   for (;;) {
     if (__builtin_expect(mutate, 0)) {  // once per MC step: kept out of the evaluations' way
-      // ---- mutation of the current conformation (the next local optimisation's start)
-      const int T = V.T;
-      const uint32_t step = (uint32_t)V.step;
-      const DevJob& job = *V.job;
-      const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)V.chain};
-      const uint4 w0 = rs.block(step, 0);
-      const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
-      xt = load_conf(W.cur, T);
-      if (mode == 0) {
-        const float3 b = unit_ball(rs, step);
-        xt.p = xt.p + kMutationAmplitude * b;
-      } else if (mode == 1) {
-        const float3 b = unit_ball(rs, step);
-        const float k = kMutationAmplitude * (1.f / L.h->gyration_radius);
-        xt.q = qnormalize(qmul(quat_from_rotvec(k * b.x, k * b.y, k * b.z), xt.q));
-      } else if (lane == 6 + (mode - 2)) {
-        xt.th = kPiF - kTwoPiF * ChainStream::to_uniform(w0.z);
-      }
+      xt = mutated_conf(*V.job, L, W, V.chain, (uint32_t)V.step, V.T);
       mutate = false;
     }
     bool done = false;  // the local optimisation ends with this evaluation
@@ -867,51 +938,10 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       // (the job record is read again here rather than held across the evaluations)
       const DevJob& job = *V.job;
       const int chain_id = V.chain;
-      const ChainStream rs{job.seed_lo, job.seed_hi, (uint32_t)chain_id};
-      const size_t trace_stride = (size_t)nx + 4;
-      float* const trace = job.trace ? job.trace + (size_t)chain_id * (job.n_steps + 1) * trace_stride : nullptr;
       int step = V.step;
       float e_cur = V.e_cur, e_best = V.e_best;
       __syncwarp();
-      if (step == 0) {
-        e_cur = e_best = eo;
-        if (lane < nx) {
-          W.cur[lane] = W.x[lane];
-          W.best[lane] = W.x[lane];
-        }
-        if (trace && !job.trace_starts) {
-          if (lane < nx) trace[lane] = W.x[lane];
-          if (lane == 0) {
-            trace[nx + 0] = e_cur;
-            trace[nx + 1] = e_cur;
-            trace[nx + 2] = -1.f;
-            trace[nx + 3] = 1.f;
-          }
-        }
-      } else {
-        const uint4 w0 = rs.block((uint32_t)step, 0);
-        const int mode = (int)(((unsigned long long)(w0.x >> 8) * (unsigned long long)(2 + T)) >> 24);
-        const float u = ChainStream::to_uniform(w0.y);
-        const bool accept = (eo < e_cur) || (u < expf(-(eo - e_cur) / job.temperature));
-        if (accept) {
-          e_cur = eo;
-          if (lane < nx) W.cur[lane] = W.x[lane];
-          if (eo < e_best) {
-            e_best = eo;
-            if (lane < nx) W.best[lane] = W.x[lane];
-          }
-        }
-        if (trace) {
-          float* t = trace + (size_t)step * trace_stride;
-          if (lane < nx) t[lane] = W.cur[lane];
-          if (lane == 0) {
-            t[nx + 0] = eo;
-            t[nx + 1] = e_cur;
-            t[nx + 2] = (float)mode;
-            t[nx + 3] = accept ? 1.f : 0.f;
-          }
-        }
-      }
+      metropolis_step(job, W, chain_id, step, T, eo, e_cur, e_best, true);
       __syncwarp();
       if (++step > job.n_steps) {
         if (lane < nx) job.chain_best_conf[(size_t)chain_id * nx + lane] = W.best[lane];
@@ -944,6 +974,120 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       V.e_cur = e_cur;
       V.e_best = e_best;
       __syncwarp();
+    }
+  }
+}
+
+// What a team's warps tell each other of one round: each warp's trial point and its
+// score and gradient.  Two of them, used in turn: a warp writes a round's only after
+// the barrier that all pass when they have read the one before the last.
+struct TeamSlot {
+  float e;
+  float x[kConfFloats];
+  float g[kHStride];
+};
+
+// run_chain's BFGS chain by a team of the CTA's warps, for launches whose chains leave
+// most of the GPU idle.  A line search halves its step until the energy falls
+// enough: three of four trial points are rejected, and run_chain evaluates them one
+// after the other.  Here warp w evaluates trial t0 + w, all at once, and the first
+// acceptable one in the search's order is taken: the decisions, and so the chain,
+// are run_chain's bit for bit.  Everything between evaluations every warp does for
+// itself, in scratch of its own; one barrier per round.
+//
+// Bound: latency (a round is one evaluation and one update, 3.2 us).  One typical-4k
+// system (384 chains, 2.6 evaluations a round with teams of 4) takes 6.1 ms of chain
+// stage against 12.0, one plain-2k system (64 chains, teams of 8) 6.3 against 14.4.
+template <int APL, int FMT>
+__device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W, TeamSlot* ex, int chain) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = blockDim.x >> 5;
+  const MapView M = make_map_view(J);
+  LaneLig<APL> R;
+  load_lane_lig<APL>(L, R);
+  const int n_ramp = ramp_steps(L);
+  const int T = L.T, nx = 7 + T, D = 6 + T, max_iters = J.n_opt_iters;
+  Conf xt = draw_start(J, T, chain);
+  if (J.trace && J.trace_starts && warp == 0) trace_start(J, chain, xt, T);
+  float e_cur = 0.f, e_best = 0.f;
+  uint32_t evals = 0;
+  int round = 0;
+  for (int step = 0;; ++step) {
+    if (step > 0) xt = mutated_conf(J, L, W, chain, (uint32_t)step, T);
+    // ---- the start, evaluated by warp 0
+    float e = 0.f, g = 0.f;
+    {
+      TeamSlot* const s = ex + (round++ & 1) * team;
+      if (warp == 0) {
+        Placed<APL> P;
+        place_atoms<APL>(L, xt, P);
+        float gn;
+        const float en = score_placed<APL, FMT, 2, true>(M, L, R, n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
+        if (lane == 0) s->e = en;
+        if (lane < kHStride) s->g[lane] = gn;
+      }
+      store_conf(W.x, xt, T);
+      __syncthreads();
+      e = s->e;
+      if (lane < kHStride) g = s->g[lane];
+      ++evals;
+    }
+    if (max_iters > 0) {
+      bfgs_reset(W, D);
+      float dir = -g;  // H0 = I
+      float gd = -warp_sum(g * g);
+      int it = 0, t0 = 0;
+      for (;;) {
+        TeamSlot* const slots = ex + (round++ & 1) * team;
+        const int trial = t0 + warp;
+        const float alpha = __int_as_float((127 - trial) << 23);  // kShrink^trial
+        if (trial < kMaxTrials) {
+          xt = apply_step(load_conf(W.x, T), alpha * dir, T);
+          Placed<APL> P;
+          place_atoms<APL>(L, xt, P);
+          float gn;
+          const float en = score_placed<APL, FMT, 2, true>(M, L, R, n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
+          TeamSlot* const s = slots + warp;
+          store_conf(s->x, xt, T);
+          if (lane == 0) s->e = en;
+          if (lane < kHStride) s->g[lane] = gn;
+        }
+        __syncthreads();
+        const int tried = min(team, kMaxTrials - t0);
+        const float e_l = lane < tried ? slots[lane].e : 0.f, a_l = __int_as_float((127 - t0 - lane) << 23);
+        const unsigned ok = __ballot_sync(kFull, lane < tried && e_l <= e + kArmijoC1 * a_l * gd);
+        if (!ok) {
+          evals += tried;
+          t0 += team;
+          if (t0 >= kMaxTrials) break;  // no acceptable step: the optimisation ends at the current iterate
+          continue;
+        }
+        const int k = __ffs(ok) - 1;
+        evals += k + 1;
+        const TeamSlot& won = slots[k];
+        const float ak = __int_as_float((127 - t0 - k) << 23);
+        const float gn = lane < kHStride ? won.g[lane] : 0.f;
+        const float s = ak * dir, y = gn - g;
+        g = gn;
+        e = won.e;
+        if (lane < nx) W.x[lane] = won.x[lane];
+        __syncwarp();
+        if (++it == max_iters) break;
+        dir = bfgs_update(W, D, s, y, gn, dir);
+        gd = warp_sum(g * dir);
+        t0 = 0;
+      }
+    }
+    // ---- local optimisation finished: its result is W.x with energy e
+    __syncwarp();
+    metropolis_step(J, W, chain, step, T, e, e_cur, e_best, warp == 0);
+    __syncwarp();
+    if (step == J.n_steps) break;
+  }
+  if (warp == 0) {
+    if (lane < nx) J.chain_best_conf[(size_t)chain * nx + lane] = W.best[lane];
+    if (lane == 0) {
+      J.chain_best_e[chain] = e_best;
+      J.chain_evals[chain] = evals;
     }
   }
 }

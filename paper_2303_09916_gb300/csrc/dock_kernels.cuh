@@ -155,6 +155,26 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
   chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
+// Teams (run_team): CTA b runs tile b, a single chain, with all its warps.
+template <int FMT>
+__global__ void __launch_bounds__(32 * kMaxTeam)
+    dock_team_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int blob_smem,
+                     ScratchLayout lay) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const Tile tile = tiles[blockIdx.x];
+  const DevJob& J = jobs[tile.job];
+  const int words = reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes / 16;
+  for (int i = threadIdx.x; i < words; i += blockDim.x)
+    reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(J.blob) + i);
+  __syncthreads();
+  const LigView L = view_blob(smem);
+  uint8_t* const scratch = smem + blob_smem;
+  const WarpScratch W = warp_scratch_at(scratch + (threadIdx.x >> 5) * lay.bytes, lay);
+  TeamSlot* const ex = reinterpret_cast<TeamSlot*>(scratch + (blockDim.x >> 5) * lay.bytes);
+  if (L.n_atoms <= 32) run_team<1, FMT>(J, L, W, ex, tile.chain0);
+  else run_team<2, FMT>(J, L, W, ex, tile.chain0);
+}
+
 // Score + gradient of a batch of conformations: one warp per conformation,
 // warps striding over the batch (the ligand is staged once per CTA).
 template <int APL, int FMT>
@@ -226,7 +246,19 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
 }
 
 template <int FMT>
+cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
+  const size_t smem = (size_t)a.blob_smem + (size_t)a.team * (a.scratch.bytes + 2 * sizeof(TeamSlot));
+  auto k = dock_team_kernel<FMT>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),
+                                          reinterpret_cast<const Tile*>(a.tiles), a.blob_smem, a.scratch);
+  return cudaGetLastError();
+}
+
+template <int FMT>
 cudaError_t launch_chains_impl(const ChainLaunch& a, cudaStream_t st) {
+  if (a.team > 1) return launch_team<FMT>(a, st);
   if (a.warps_per_cta != 1 && a.warps_per_cta != 2 && a.warps_per_cta != kMaxChainWarps) return cudaErrorInvalidValue;
   if (a.apl_mask == 1) {
     switch (a.variant) {

@@ -35,6 +35,7 @@ struct dsdp_plan {
   size_t queue_bytes = 0;
   size_t queue_next_off = 0;  // of the next steps, in ints
   bool auto_queue = false;    // no fixed choice: queue when a group has more tiles than fit at once
+  int team = 1;               // no fixed choice, few chains: warps of each (dock_team_kernel)
   void* d_blocks = nullptr;
   int n_rtiles = 0;
   // per job, to lay groups and tiles out again for another configuration
@@ -222,6 +223,18 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
     }
 }
 
+// Warps of a chain (dock_team_kernel) when the plan's chains leave most of the GPU
+// idle; 1 when they do not.  Up to one chain per SM a team of 8 (64 plain-2k chains
+// 6.3 ms against 6.7 in teams of 4; 200 typical-4k chains 2.8 against 2.6), up to 8
+// per SM teams of 4 (1,200 chains 6.9 ms, one warp each 8.1; 1,536 chains 9.7 against
+// 8.3): beyond, the trial points that a line search does not come to cost more than
+// the shorter way saves.  Teams are a warp per SM sub-partition or two: 5 and 6 warps
+// measured slower than 4.
+static int team_warps(size_t chains, int sms) {
+  if (chains <= (size_t)sms) return kMaxTeam;
+  return chains <= (size_t)(8 * sms) ? 4 : 1;
+}
+
 static cudaError_t plan_use_warps(dsdp_plan* P, int W) {
   std::vector<Tile> tiles;
   std::vector<SliceBlock> blocks;
@@ -353,6 +366,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
   size_t total_chains = 0, max_blocks = 0;
+  bool all_bfgs = true;
   {
     // Length of a job's chains, relative: evaluations (MC steps; Barzilai-Borwein
     // runs all its iterations, BFGS about 60 of 100) times the cost of one (the
@@ -368,6 +382,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
       longest = std::max(longest, cost);
       total_chains += (size_t)dj[j].n_chains;
     }
+    for (int j = 0; j < n_jobs; ++j) all_bfgs = all_bfgs && dj[j].optimizer == DSDP_OPT_BFGS;
     P->job_order.resize(n_jobs);
     for (int j = 0; j < n_jobs; ++j) {
       P->job_order[j] = j;
@@ -409,6 +424,8 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
         if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
       } else {
         P->auto_queue = many;
+        P->team = all_bfgs && !pers ? team_warps(total_chains, P->sms) : 1;
+        if (P->team > 1) W = 1;
       }
     } else {
       var = (tile_config - 1) % 4;
@@ -505,6 +522,7 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
     a.overlap = gi > 0 && queue != kNoQueue;
     a.variant = P->variant;
+    a.team = P->team;
     cudaError_t e = launch_chains_dispatch(g.fmt, a, st);
     if (e != cudaSuccess) return check_cuda(e, "dock_chains_kernel launch");
   }
@@ -533,36 +551,45 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e != cudaSuccess) return check_cuda(e, "autotune events");
   const uint32_t base_flags = P->flags & ~(uint32_t)DSDP_PLAN_PERSISTENT;
-  P->auto_queue = false;  // with and without the queue are measured apart
+  // the automatic arrangement (queue when needed, teams) first: kept if nothing beats it
+  const bool auto_queue = P->auto_queue;
+  const int team = P->team, auto_var = P->variant, auto_w = P->warps_per_cta;
+  const uint32_t auto_flags = P->flags;
+  float auto_ms = 1e30f;
   float best = 1e30f;
   int best_var = P->variant, best_pers = (P->flags & DSDP_PLAN_PERSISTENT) ? 1 : 0, best_w = P->warps_per_cta;
   dsdp_status s = DSDP_OK;
-  // register budgets compiled: 128, 96, 80, 72 for one atom per lane, 128 and
-  // 96 for two and for mixed tiles (launch_chains_impl)
-  int n_var = 2;
-  for (const dsdp_plan::Group& g : P->groups) n_var = std::max(n_var, g.apl_mask == 1 ? 4 : 2);
-  for (int w = 1; w <= 4 && s == DSDP_OK; w *= 2)
-  for (int pers = 0; pers < 2 && s == DSDP_OK; ++pers) {
+  auto measure = [&](float* ms) {
+    dsdp_status r = dsdp_plan_launch_stage(P, DSDP_STAGE_CHAINS, stream);  // warm-up
+    if (r != DSDP_OK) return r;
+    cudaEventRecord(a, st);
+    for (int k = 0; k < repeats && r == DSDP_OK; ++k) r = dsdp_plan_launch_stage(P, DSDP_STAGE_CHAINS, stream);
+    cudaEventRecord(b, st);
+    const cudaError_t ee = cudaEventSynchronize(b);
+    if (ee != cudaSuccess) return check_cuda(ee, "autotune run");
+    cudaEventElapsedTime(ms, a, b);
+    return r;
+  };
+  if (auto_queue || team > 1) s = measure(&auto_ms);
+  P->auto_queue = false;  // with and without the queue are measured apart
+  P->team = 1;
+  for (int c = 0; c < 6 && s == DSDP_OK; ++c) {
+    const int w = 1 << (c / 2), pers = c % 2;
     P->flags = base_flags | (pers ? DSDP_PLAN_PERSISTENT : 0u);
     e = plan_use_warps(P, w);
     if (e != cudaSuccess) {
       s = check_cuda(e, "autotune tiles");
       break;
     }
+    // register budgets compiled: 128, 96, 80, 72 for one atom per lane, 128 and
+    // 96 for two and for mixed tiles (launch_chains_impl)
+    int n_var = 2;
+    for (const dsdp_plan::Group& g : P->groups) n_var = std::max(n_var, g.apl_mask == 1 ? 4 : 2);
     for (int var = 0; var < n_var && s == DSDP_OK; ++var) {
       P->variant = var;
-      s = dsdp_plan_launch_stage(P, DSDP_STAGE_CHAINS, stream);  // warm-up
-      if (s != DSDP_OK) break;
-      cudaEventRecord(a, st);
-      for (int r = 0; r < repeats && s == DSDP_OK; ++r) s = dsdp_plan_launch_stage(P, DSDP_STAGE_CHAINS, stream);
-      cudaEventRecord(b, st);
-      e = cudaEventSynchronize(b);
-      if (e != cudaSuccess) {
-        s = check_cuda(e, "autotune run");
-        break;
-      }
       float ms = 0.f;
-      cudaEventElapsedTime(&ms, a, b);
+      s = measure(&ms);
+      if (s != DSDP_OK) break;
       if (ms_by_config) ms_by_config[var + 4 * (w == 4 ? 2 : w - 1) + 12 * pers] = ms / repeats;
       if (ms < best) {
         best = ms;
@@ -574,12 +601,19 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
+  if (chosen) *chosen = 1 + best_var + 4 * (best_w == 4 ? 2 : best_w - 1) + 12 * best_pers;
+  if (s == DSDP_OK && auto_ms <= best) {  // later plans of this shape find it by themselves
+    P->variant = auto_var;
+    P->flags = auto_flags;
+    P->auto_queue = auto_queue;
+    P->team = team;
+    return check_cuda(plan_use_warps(P, auto_w), "plan tiles");
+  }
   P->variant = best_var;
   P->flags = base_flags | (best_pers ? DSDP_PLAN_PERSISTENT : 0u);
   if (s == DSDP_OK) s = check_cuda(plan_use_warps(P, best_w), "plan tiles");
   if (s != DSDP_OK) return s;
   tune_store(P->tune_key, best_var, best_pers, best_w);
-  if (chosen) *chosen = 1 + best_var + 4 * (best_w == 4 ? 2 : best_w - 1) + 12 * best_pers;
   return DSDP_OK;
 }
 

@@ -11,6 +11,8 @@ namespace dsdp {
 // always, or when there are more tiles than CTAs fit on the GPU at once.
 enum ChainQueueMode { kNoQueue, kQueue, kQueueIfMany };
 
+constexpr int kMaxTeam = 8;  // warps of a chain (dock_team_kernel)
+
 struct ChainLaunch {
   const void* jobs;   // DevJob[] (device)
   const void* tiles;  // Tile[] (device)
@@ -23,6 +25,7 @@ struct ChainLaunch {
   int n_blocks, n_items;
   bool overlap;       // independent of the launch before it on the stream: its CTAs may start as that one's leave
   int warps_per_cta;
+  int team;           // warps of a chain (dock_team_kernel); 1: none of it
   int apl;            // largest atoms-per-lane tile present
   int apl_mask;       // tiles present: bit 0 one atom per lane (<= 32 atoms), bit 1 two (<= 64)
   int blob_smem;      // bytes reserved for the largest staged blob prefix
