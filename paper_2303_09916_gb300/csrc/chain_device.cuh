@@ -995,7 +995,9 @@ struct TeamSlot {
 // are run_chain's bit for bit.  Everything between evaluations every warp does for
 // itself, in scratch of its own; one barrier per round.
 //
-// Bound: latency (a round is one evaluation and one update, 3.2 us).  One typical-4k
+// Bound: latency (a round is one evaluation and one update, 3.2 us; energies first and
+// the winner's gradient after a second barrier: 8 % slower alone and no faster with
+// eight launches at once).  One typical-4k
 // system (384 chains, 2.6 evaluations a round with teams of 4) takes 6.1 ms of chain
 // stage against 12.0, one plain-2k system (64 chains, teams of 8) 6.3 against 14.4.
 template <int APL, int FMT>

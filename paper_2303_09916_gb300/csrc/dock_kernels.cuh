@@ -155,9 +155,12 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
   chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
-// Teams (run_team): CTA b runs tile b, a single chain, with all its warps.
-template <int FMT>
-__global__ void __launch_bounds__(32 * kMaxTeam)
+// Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
+// of kMaxTeam warps the registers must allow per SM; with one chain per SM at most,
+// one (64 plain-2k chains 5.9 ms against 6.2), else two, which is 128 registers and
+// four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5).
+template <int FMT, int MB>
+__global__ void __launch_bounds__(32 * kMaxTeam, MB)
     dock_team_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int blob_smem,
                      ScratchLayout lay) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -248,7 +251,7 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
 template <int FMT>
 cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
   const size_t smem = (size_t)a.blob_smem + (size_t)a.team * (a.scratch.bytes + 2 * sizeof(TeamSlot));
-  auto k = dock_team_kernel<FMT>;
+  auto k = a.team == kMaxTeam ? dock_team_kernel<FMT, 1> : dock_team_kernel<FMT, 2>;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),

@@ -127,6 +127,9 @@ struct DevJob {
 // chain), which is not in use while the chains run.
 constexpr int kSliceRecordBytes = 8 * (7 + kMaxDim) + 16;
 
+// Internal plan flag: other launches share the GPU with this plan's (no teams).
+constexpr uint32_t kPlanShared = 1u << 30;
+
 struct Tile {
   int32_t job;
   int32_t chain0;

@@ -227,7 +227,8 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
 // idle; 1 when they do not.  Up to one chain per SM a team of 8 (64 plain-2k chains
 // 6.3 ms against 6.7 in teams of 4; 200 typical-4k chains 2.8 against 2.6), up to 8
 // per SM teams of 4 (1,200 chains 6.9 ms, one warp each 8.1; 1,536 chains 9.7 against
-// 8.3): beyond, the trial points that a line search does not come to cost more than
+// 8.3; four such launches of 384 chains at once 7.3 against 9.3, eight 13.5 against
+// 11.9 -- the job queue, which knows, does without teams then): beyond, the trial points that a line search does not come to cost more than
 // the shorter way saves.  Teams are a warp per SM sub-partition or two: 5 and 6 warps
 // measured slower than 4.
 static int team_warps(size_t chains, int sms) {
@@ -362,7 +363,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   dsdp_plan* P = new dsdp_plan();
   P->ctx = ctx;
   P->n_jobs = n_jobs;
-  P->flags = flags;
+  P->flags = flags & ~kPlanShared;
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
   size_t total_chains = 0, max_blocks = 0;
@@ -424,7 +425,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
         if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
       } else {
         P->auto_queue = many;
-        P->team = all_bfgs && !pers ? team_warps(total_chains, P->sms) : 1;
+        P->team = all_bfgs && !pers && !(flags & kPlanShared) ? team_warps(total_chains, P->sms) : 1;
         if (P->team > 1) W = 1;
       }
     } else {
