@@ -771,7 +771,7 @@ __device__ __forceinline__ void trace_start(const DevJob& J, int chain, const Co
 // at and leaves it in the record; without, the whole chain.
 // REVIEW: read the ligand's view from the staged blob at each evaluation instead of
 // holding it in registers (the 96-register kernel of mixed tiles spills otherwise).
-template <int APL, int FMT, int IU = 2, bool REVIEW = false>
+template <int APL, int FMT, int IU = 2, bool REVIEW = false, bool FLAT = false>
 __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& W, int chain, const ChainSlice& sl) {
   enum : int { kStart = 0, kTrial = 1, kBB = 2 };
   const int lane = threadIdx.x & 31;
@@ -855,7 +855,7 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
     }
     if (!done) {
       float gn;
-      const float en = score_placed<APL, FMT, IU>(M, Lv, R, V.n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
+      const float en = score_placed<APL, FMT, IU, FLAT>(M, Lv, R, V.n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
       const int T = V.T, D = 6 + T;
       const int max_iters = V.max_iters;
       phase = V.phase;

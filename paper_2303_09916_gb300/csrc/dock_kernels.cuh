@@ -94,7 +94,7 @@ static __device__ __noinline__ int queue_next(const ChainQueue& q, int n_tiles) 
   }
 }
 
-template <int FMT, int APLS, int IU, bool REVIEW>
+template <int FMT, int APLS, int IU, bool REVIEW, bool FLAT>
 __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles,
                                           const ChainQueue& queue, int blob_smem, const ScratchLayout& lay) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -133,8 +133,8 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
         sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
         sl.steps = J.slice_steps;
       }
-      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, IU, REVIEW>(J, L, W, chain, sl);
-      else run_chain<2, FMT, IU, REVIEW>(J, L, W, chain, sl);
+      if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_chain<1, FMT, IU, REVIEW, FLAT>(J, L, W, chain, sl);
+      else run_chain<2, FMT, IU, REVIEW, FLAT>(J, L, W, chain, sl);
     }
     if (!queue.n_items) break;
     __syncthreads();
@@ -152,7 +152,7 @@ template <int FMT, int VAR, int APLS>
 __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>()))
     dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
                        int blob_smem, ScratchLayout lay) {
-  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
+  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && APLS != 3>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
 // Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
