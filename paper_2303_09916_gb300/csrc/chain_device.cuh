@@ -42,6 +42,20 @@ __device__ __forceinline__ LigView view_blob(const uint8_t* b) {
   return v;
 }
 
+// Stages a ligand's blob into shared memory (all threads of the CTA; no barrier before,
+// one after) and notes at each body the lane of its parent's first atom, which one
+// atom per lane is that atom's index.
+__device__ __forceinline__ void stage_blob(uint8_t* smem, const uint8_t* blob, int bytes) {
+  for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x)
+    reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(blob) + i);
+  __syncthreads();
+  const BlobHeader* h = reinterpret_cast<const BlobHeader*>(smem);
+  BodyRec* body = reinterpret_cast<BodyRec*>(smem + h->off_body);
+  if (threadIdx.x < h->n_bodies)
+    body[threadIdx.x].parent_lane = body[threadIdx.x].parent >= 0 ? body[body[threadIdx.x].parent].atom_begin : -1;
+  __syncthreads();
+}
+
 // Per-lane ligand data: the atoms of the lane's slots (atom lane with one atom
 // per lane; the blob's lane map with two) and, on lane b < n_bodies, body b's
 // record; re-read from the staged blob (shared memory) where used.
@@ -64,7 +78,8 @@ __device__ __forceinline__ void load_lane_lig(const LigView& L, LaneLig<APL>& R)
   R.n_atoms = L.n_atoms;
   R.nb = L.n_bodies;
   R.T = L.T;
-  R.tbody = (lane >= 6 && lane < 6 + L.T) ? L.torsion_body[lane - 6] : 0;
+  R.tbody = (lane >= 6 && lane < 6 + L.T) ? L.torsion_body[lane - 6] : 0;  // the lane with that body's gradient
+  if (APL == 1) R.tbody = L.body[R.tbody].atom_begin;
 }
 
 // Conformation held by a warp: p and q replicated in every lane, torsion k in lane 6 + k.
@@ -76,7 +91,7 @@ struct Conf {
 
 // Per-warp shared scratch (layout in scratch_layout).
 struct WarpScratch {
-  float4* pre;     // [kMaxAtoms][2] inclusive prefix sums of (g, (r - p) x g): (gx, gy, gz, cx), (cy, cz, -, -)
+  float4* pre;     // inclusive prefix sums of (g, (r - p) x g): [n_atoms] (gx, gy, gz, cx), then [n_atoms] (cy, cz)
   float* H;        // [6 + T][kHStride] BFGS inverse Hessian, row j owned by lane j
   float* vec;      // [5][kHStride] + kVarWords: g', s, u broadcast to the H rows (BFGS update);
                    // the chain's g and d; its ChainVars
@@ -101,7 +116,7 @@ __host__ __device__ inline ScratchLayout scratch_layout(int n_atoms, int n_torsi
   ScratchLayout l;
   const int D = 6 + n_torsions;
   l.pre = 0;
-  l.H = l.pre + align16i(32 * n_atoms);
+  l.H = l.pre + align16i(24 * n_atoms);
   l.vec = l.H + align16i(4 * kHStride * D);
   l.x = l.vec + align16i(4 * (5 * kHStride + kVarWords));
   l.cur = l.x + align16i(4 * kConfFloats);
@@ -120,30 +135,34 @@ __device__ __forceinline__ WarpScratch warp_scratch_at(uint8_t* base, const Scra
   return W;
 }
 
-// Body frames for a conformation: lane b < n_bodies returns body b's world
-// rotation Q and origin O, composed from the local transforms by pointer
-// jumping (ceil(log2(depth + 1)) rounds of shuffles).
-__device__ __forceinline__ void body_frames(const LigView& L, const Conf& c, Quat& Q, float3& O) {
+// Body frames for a conformation: the lane returns the world rotation Q and origin O
+// of body `body`, composed from the local transforms by pointer jumping
+// (ceil(log2(depth + 1)) rounds of shuffles).  OF_ATOM: the body of the lane's atom
+// (the parent's frame is at the parent's first atom, stage_blob); else body = lane,
+// nothing beyond n_bodies.
+template <bool OF_ATOM>
+__device__ __forceinline__ void body_frames(const LigView& L, const Conf& c, int body, Quat& Q, float3& O) {
   const int lane = threadIdx.x & 31;
-  const int nb = L.n_bodies;
-  const bool child = lane > 0 && lane < nb;
+  const bool child = body > 0 && (OF_ATOM || lane < L.n_bodies);
   float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
+  int parent_lane = -1;
   if (child) {
-    const float4* rec = reinterpret_cast<const float4*>(L.body + lane);
+    const float4* rec = reinterpret_cast<const float4*>(L.body + body);
     b0 = rec[0];  // off xyz, parent
     b1 = rec[1];  // axis xyz, torsion
+    parent_lane = OF_ATOM ? L.body[body].parent_lane : __float_as_int(b0.w);
   }
   const int tors = __float_as_int(b1.w);
   const float tb = __shfl_sync(kFull, c.th, child ? 6 + tors : 0);
   int ptr = -1;
-  if (lane == 0) {
-    Q = c.q;
-    O = c.p;
-  } else if (child) {
+  if (child) {
     const float s = sin_ftz(0.5f * tb), co = cos_ftz(0.5f * tb);  // |theta / 2| <= pi / 2: absolute error < 4e-7
     Q = Quat{co, s * b1.x, s * b1.y, s * b1.z};
     O = make_float3(b0.x, b0.y, b0.z);
-    ptr = __float_as_int(b0.w);
+    ptr = parent_lane;
+  } else if (OF_ATOM || lane == 0) {
+    Q = c.q;
+    O = c.p;
   } else {
     Q = Quat{1.f, 0.f, 0.f, 0.f};
     O = make_float3(0.f, 0.f, 0.f);
@@ -161,29 +180,39 @@ __device__ __forceinline__ void body_frames(const LigView& L, const Conf& c, Qua
   }
 }
 
-// A conformation's atoms and body frames: lane b < n_bodies holds body b's frame,
-// every lane the atoms of its slots.
+// A conformation's atoms and body frames.  Two atoms per lane: lane b < n_bodies holds
+// body b's frame.  One: every lane holds the frame of its own atom's body, which
+// saves fetching it for the atom (seven shuffles); what is done once per body is
+// done on the lane of its first atom.
 template <int APL>
 struct Placed {
   Quat Q;
   float3 O;
   float3 pos[APL];
-  int type[APL];
+  int type[APL];  // map type | body << 8
   int atom[APL];  // the slot's atom, -1 when empty
 };
 
 template <int APL>
 __device__ __forceinline__ void place_atoms(const LigView& L, const Conf& c, Placed<APL>& P) {
   const int lane = threadIdx.x & 31;
-  body_frames(L, c, P.Q, P.O);
+  if (APL == 1) {
+    P.atom[0] = lane < L.n_atoms ? lane : -1;
+    const float4 a = L.atom[lane < L.n_atoms ? lane : 0];
+    P.type[0] = __float_as_int(a.w);
+    const int b = P.type[0] >> 8;
+    body_frames<true>(L, c, b, P.Q, P.O);
+    P.pos[0] = P.O + qrot(P.Q, make_float3(a.x, a.y, a.z));
+    return;
+  }
+  body_frames<false>(L, c, lane, P.Q, P.O);
 #pragma unroll
   for (int s = 0; s < APL; ++s) {
-    P.atom[s] = APL == 1 ? (lane < L.n_atoms ? lane : -1) : (int)L.lane_map[2 * lane + s];
+    P.atom[s] = (int)L.lane_map[2 * lane + s];
     const int i = P.atom[s];
     const float4 a = L.atom[i >= 0 ? i : 0];
-    const int packed = __float_as_int(a.w);
-    P.type[s] = packed & 0xff;
-    const int b = i >= 0 ? (packed >> 8) & 0xff : 0;
+    P.type[s] = __float_as_int(a.w);
+    const int b = i >= 0 ? (P.type[s] >> 8) & 0xff : 0;
     const Quat Qb = shflq(P.Q, b);
     const float3 Ob = shfl3(P.O, b);
     P.pos[s] = Ob + qrot(Qb, make_float3(a.x, a.y, a.z));
@@ -231,7 +260,7 @@ __device__ __forceinline__ float energy_placed(const MapView& M, const LigView& 
   e_lane += e_pair.x + e_pair.y;
 #pragma unroll
   for (int s = 0; s < APL; ++s)
-    if (P.atom[s] >= 0) e_lane += map_energy<FMT>(M, P.type[s], map_cell(M, P.pos[s]));
+    if (P.atom[s] >= 0) e_lane += map_energy<FMT>(M, P.type[s] & 0xff, map_cell(M, P.pos[s]));
   return warp_sum(e_lane);
 }
 
@@ -346,7 +375,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
       float3 gi;
       // the cell is located here, where it is used: holding it across the intra
       // block miscompiled the two-atoms-per-lane kernels (gradient x channel lost)
-      e_lane += map_interp<FMT>(M, type[s], map_cell(M, pos[s]), gi);
+      e_lane += map_interp<FMT>(M, type[s] & 0xff, map_cell(M, pos[s]), gi);
       g[s] = g[s] + gi;
     }
   }
@@ -356,13 +385,14 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
   //      With two atoms per lane the lane map is not in atom order: each slot
   //      first parks its raw terms at its atom's place, and lane l then scans
   //      atoms 2l and 2l + 1 of the atom order.
+  float2* const pre2 = reinterpret_cast<float2*>(W.pre + N);
   if (APL == 2) {
 #pragma unroll
     for (int s = 0; s < APL; ++s) {
       if (atom[s] < 0) continue;
       const float3 t = cross3(pos[s] - c.p, g[s]);
-      W.pre[2 * atom[s]] = make_float4(g[s].x, g[s].y, g[s].z, t.x);
-      W.pre[2 * atom[s] + 1] = make_float4(t.y, t.z, 0.f, 0.f);
+      W.pre[atom[s]] = make_float4(g[s].x, g[s].y, g[s].z, t.x);
+      pre2[atom[s]] = make_float2(t.y, t.z);
     }
     __syncwarp();
   }
@@ -379,7 +409,8 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
       raw[s][0] = g[s].x, raw[s][1] = g[s].y, raw[s][2] = g[s].z;
       raw[s][3] = t.x, raw[s][4] = t.y, raw[s][5] = t.z;
     } else {
-      const float4 h0 = W.pre[2 * i], h1 = W.pre[2 * i + 1];
+      const float4 h0 = W.pre[i];
+      const float2 h1 = pre2[i];
       raw[s][0] = h0.x, raw[s][1] = h0.y, raw[s][2] = h0.z;
       raw[s][3] = h0.w, raw[s][4] = h1.x, raw[s][5] = h1.y;
     }
@@ -409,18 +440,19 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
       if (i >= N) continue;
 #pragma unroll
       for (int k = 0; k < 6; ++k) run[k] += raw[s][k];
-      W.pre[2 * i] = make_float4(run[0], run[1], run[2], run[3]);
-      W.pre[2 * i + 1] = make_float4(run[4], run[5], 0.f, 0.f);
+      W.pre[i] = make_float4(run[0], run[1], run[2], run[3]);
+      pre2[i] = make_float2(run[4], run[5]);
     }
   }
   __syncwarp();
   float tor = 0.f;
-  if (lane > 0 && lane < nb) {
-    const float4* rec = reinterpret_cast<const float4*>(L.body + lane);
+  const int body = APL == 1 ? type[0] >> 8 : lane;
+  if (body > 0 && (APL == 1 || lane < nb)) {
+    const float4* rec = reinterpret_cast<const float4*>(L.body + body);
     const float4 b1 = rec[1];
-    const int4 b2 = *reinterpret_cast<const int4*>(rec + 2);  // atom_begin, atom_end, depth, pad
-    const float4 h0 = W.pre[2 * (b2.y - 1)], h1 = W.pre[2 * (b2.y - 1) + 1];
-    const float4 l0 = W.pre[2 * (b2.x - 1)], l1 = W.pre[2 * (b2.x - 1) + 1];
+    const int4 b2 = *reinterpret_cast<const int4*>(rec + 2);  // atom_begin, atom_end, depth, parent_lane
+    const float4 h0 = W.pre[b2.y - 1], l0 = W.pre[b2.x - 1];
+    const float2 h1 = pre2[b2.y - 1], l1 = pre2[b2.x - 1];
     const float3 G = make_float3(h0.x - l0.x, h0.y - l0.y, h0.z - l0.z);
     const float3 C = make_float3(h0.w - l0.w, h1.x - l1.x, h1.y - l1.y);
     const float3 axis = qrot(Q, make_float3(b1.x, b1.y, b1.z));
@@ -429,8 +461,8 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
   const float tv = __shfl_sync(kFull, tor, R.tbody);
   float gl = 0.f;
   if (lane < 6) {
-    const float* tot = reinterpret_cast<const float*>(W.pre + 2 * (N - 1));
-    gl = tot[lane];
+    gl = lane < 4 ? reinterpret_cast<const float*>(W.pre + N - 1)[lane]
+                  : reinterpret_cast<const float*>(pre2 + N - 1)[lane - 4];
   } else if (lane < 6 + L.T) {
     gl = tv;
   }
@@ -626,20 +658,36 @@ struct ChainSlice {
 // Chain and optimiser variables that wait in shared memory while a
 // conformation is evaluated (read back through volatile loads, so that none of
 // them holds a register during the evaluation).
-struct ChainVars {
-  int phase, it, trial, step;
-  float e, gd, alpha, e_opt_best;
-  float e_cur, e_best;
+struct alignas(16) ChainVars {
+  // what each evaluation reads and writes, in groups of one 16-byte access
+  int phase, trial;
+  float alpha;
   uint32_t evals;
-  int T;
-  int bb, max_iters;
-  int n_ramp;
-  int chain;
+  float e, gd, e_opt_best;
+  int it;
+  int T, bb, max_iters, n_ramp;
+  // once per local optimisation
+  float e_cur, e_best;
+  int step, chain;
   int stop;  // MC step at which this run of the chain ends (n_steps + 1: the chain's end)
+  int pad;
   const DevJob* job;
   ChainRecord* rec;  // ChainSlice
   int* next_step;
 };
+// Volatile 16-byte accesses of a group (its first member).
+__device__ __forceinline__ uint4 load_group(const volatile void* p) {
+  uint4 v;
+  asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"((uint32_t)__cvta_generic_to_shared(const_cast<const void*>(p))));
+  return v;
+}
+__device__ __forceinline__ void store_group(volatile void* p, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.volatile.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(const_cast<void*>(p))),
+               "r"(x), "r"(y), "r"(z), "r"(w));
+}
 static_assert(sizeof(ChainVars) <= 4 * kVarWords, "ChainVars must fit its words of the vec area");
 
 // The drawn start of a chain.
@@ -836,16 +884,17 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       // BFGS: Armijo test of the trial point x + alpha d on its energy alone; its
       // gradient is evaluated when it is accepted (27 % of first trials, 23 % of all)
       const float en = energy_placed<APL, FMT, IU>(M, Lv, V.n_ramp, P);
-      const float e = V.e, gd = V.gd;
-      float alpha = V.alpha;
+      const uint4 v0 = load_group(&V.phase), v1 = load_group(&V.e);
+      const float e = __uint_as_float(v1.x), gd = __uint_as_float(v1.y);
+      float alpha = __uint_as_float(v0.z);
       if (!(en <= e + kArmijoC1 * alpha * gd)) {
-        const int T = V.T, trial = V.trial + 1;
-        V.evals = V.evals + 1;
+        const int trial = (int)v0.y + 1;
+        alpha *= kShrink;
+        __syncwarp();
+        if (lane == 0) store_group(&V.phase, v0.x, (uint32_t)trial, __float_as_uint(alpha), v0.w + 1u);
         if (trial < kMaxTrials) {
-          alpha *= kShrink;
-          V.alpha = alpha;
-          V.trial = trial;
           const float dir = lane < kHStride ? Vd[lane] : 0.f;
+          const int T = Lv.T;
           xt = apply_step(load_conf(W.x, T), alpha * dir, T);
           __syncwarp();
           continue;
@@ -856,12 +905,13 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
     if (!done) {
       float gn;
       const float en = score_placed<APL, FMT, IU, FLAT>(M, Lv, R, V.n_ramp, W, xt, P, gn, DSDP_TERM_ALL);
-      const int T = V.T, D = 6 + T;
-      const int max_iters = V.max_iters;
-      phase = V.phase;
-      int it = V.it;
-      float e_opt_best = V.e_opt_best;
-      float e = V.e, gd = V.gd, alpha = V.alpha;
+      const uint4 v0 = load_group(&V.phase), v1 = load_group(&V.e), v2 = load_group(&V.T);
+      const int T = (int)v2.x, D = 6 + T, max_iters = (int)v2.z;
+      const bool bb = v2.y != 0;
+      phase = (int)v0.x;
+      int it = (int)v1.w;
+      float e_opt_best = __uint_as_float(v1.z);
+      float e = __uint_as_float(v1.x), gd = __uint_as_float(v1.y), alpha = __uint_as_float(v0.z);
       float g = lane < kHStride ? Vg[lane] : 0.f, dir = lane < kHStride ? Vd[lane] : 0.f;
       if (phase == kStart) {  // first evaluation of a local optimisation
         e = en;
@@ -869,13 +919,12 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
         store_conf(W.x, xt, T);
         if (max_iters == 0) {
           done = true;
-        } else if (!V.bb) {
+        } else if (!bb) {
           bfgs_reset(W, D);
           dir = -g;  // H0 = I
           gd = -warp_sum(g * g);
           it = 0;
           alpha = 1.f;
-          V.trial = 0;
           xt = apply_step(xt, dir, T);
           phase = kTrial;
         } else {
@@ -897,7 +946,6 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
           dir = bfgs_update(W, D, s, y, gn, dir);
           gd = warp_sum(g * dir);  // computed directly: the sufficient-decrease test must see the true slope
           alpha = 1.f;
-          V.trial = 0;
           xt = apply_step(xt, dir, T);
         }
       } else {  // BB: x_{k+1} = x_k + s_k evaluated; next step length from s.s / s.y
@@ -916,13 +964,11 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
           xt = apply_step(xt, dir, T);
         }
       }
-      V.evals = V.evals + 1;
-      V.phase = phase;
-      V.it = it;
-      V.e = e;
-      V.gd = gd;
-      V.alpha = alpha;
-      V.e_opt_best = e_opt_best;
+      __syncwarp();  // the groups are read by every lane
+      if (lane == 0) {
+        store_group(&V.phase, (uint32_t)phase, 0u, __float_as_uint(alpha), v0.w + 1u);  // the next trial is the first
+        store_group(&V.e, __float_as_uint(e), __float_as_uint(gd), __float_as_uint(e_opt_best), (uint32_t)it);
+      }
       if (lane < kHStride) {
         Vg[lane] = g;
         Vd[lane] = dir;

@@ -73,7 +73,7 @@ struct ChainQueue {
 
 // The next tile for this CTA, n_tiles when none is left (one thread).  The first
 // taker of an idle tile runs it; an item of a running tile stays with its CTA.
-static __device__ __noinline__ int queue_next(const ChainQueue& q, int n_tiles) {
+__device__ __forceinline__ int queue_next(const ChainQueue& q, int n_tiles) {
   for (;;) {
     const int item = atomicAdd(q.counter, 1);
     if (item >= q.n_items) return n_tiles;
@@ -116,10 +116,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
     const DevJob& J = jobs[tile.job];
     if (s_job != tile.job) {  // uniform: s_job only changes between barriers
       __syncthreads();
-      const int words = reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes / 16;
-      for (int i = threadIdx.x; i < words; i += blockDim.x)
-        reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(J.blob) + i);
-      __syncthreads();
+      stage_blob(smem, J.blob, reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes);
       if (threadIdx.x == 0) s_job = tile.job;
     }
     if (warp < tile.count) {
@@ -152,7 +149,7 @@ template <int FMT, int VAR, int APLS>
 __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>()))
     dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
                        int blob_smem, ScratchLayout lay) {
-  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && APLS != 3>(jobs, tiles, n_tiles, queue, blob_smem, lay);
+  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && (APLS == 1 || (APLS == 2 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
 // Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
@@ -166,10 +163,7 @@ __global__ void __launch_bounds__(32 * kMaxTeam, MB)
   extern __shared__ __align__(16) uint8_t smem[];
   const Tile tile = tiles[blockIdx.x];
   const DevJob& J = jobs[tile.job];
-  const int words = reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes / 16;
-  for (int i = threadIdx.x; i < words; i += blockDim.x)
-    reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(J.blob) + i);
-  __syncthreads();
+  stage_blob(smem, J.blob, reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes);
   const LigView L = view_blob(smem);
   uint8_t* const scratch = smem + blob_smem;
   const WarpScratch W = warp_scratch_at(scratch + (threadIdx.x >> 5) * lay.bytes, lay);
@@ -179,34 +173,35 @@ __global__ void __launch_bounds__(32 * kMaxTeam, MB)
 }
 
 // Score + gradient of a batch of conformations: one warp per conformation,
-// warps striding over the batch (the ligand is staged once per CTA).
-template <int APL, int FMT>
-__global__ void __launch_bounds__(256) score_eval_kernel(MapView M, const uint8_t* __restrict__ blob,
-                                                         const float* __restrict__ conf, int n_conf,
-                                                         float* __restrict__ energy, float* __restrict__ grad,
-                                                         uint32_t flags, int blob_smem, ScratchLayout lay) {
+// warps striding over the batch (the ligand is staged once per CTA, while the first
+// conformation is on its way).  FLAT (score_placed): a batch of at most one warp
+// per scheduler, which takes as long as one evaluation does.
+template <int APL, int FMT, bool FLAT>
+__global__ void __launch_bounds__(128, 6) score_eval_kernel(MapView M, const uint8_t* __restrict__ blob,
+                                                            const float* __restrict__ conf, int n_conf, int T,
+                                                            float* __restrict__ energy, float* __restrict__ grad,
+                                                            uint32_t flags, int blob_smem, ScratchLayout lay) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const int words = reinterpret_cast<const BlobHeader*>(blob)->stage_bytes / 16;
-  for (int i = threadIdx.x; i < words; i += blockDim.x)
-    reinterpret_cast<int4*>(smem)[i] = __ldg(reinterpret_cast<const int4*>(blob) + i);
-  __syncthreads();
-  const LigView L = view_blob(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  int c = blockIdx.x * (blockDim.x >> 5) + warp;
+  Conf x = load_conf(conf + (size_t)(c < n_conf ? c : 0) * (7 + T), T);
+  stage_blob(smem, blob, blob_smem);
+  const LigView L = view_blob(smem);
   const WarpScratch W = warp_scratch_at(smem + blob_smem + warp * lay.bytes, lay);
   LaneLig<APL> R;
   load_lane_lig<APL>(L, R);
-  const int T = L.T;
   const int n_ramp = ramp_steps(L);
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  for (int c = blockIdx.x * (blockDim.x >> 5) + warp; c < n_conf; c += warps) {  // warp-uniform loop
-    Conf x = load_conf(conf + (size_t)c * (7 + T), T);
+  while (c < n_conf) {  // warp-uniform loop
     x.q = qnormalize(x.q);
     float g;
     Placed<APL> P;
     place_atoms<APL>(L, x, P);
-    const float e = score_placed<APL, FMT>(M, L, R, n_ramp, W, x, P, g, flags);
+    const float e = score_placed<APL, FMT, 2, FLAT>(M, L, R, n_ramp, W, x, P, g, flags);
     if (lane == 0 && energy) energy[c] = e;
     if (grad && lane < 6 + T) grad[(size_t)c * (6 + T) + lane] = g;
+    c += warps;
+    if (c < n_conf) x = load_conf(conf + (size_t)c * (7 + T), T);
   }
 }
 
@@ -215,14 +210,13 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   const dim3 block(32 * a.warps_per_cta);
   const size_t smem = (size_t)a.blob_smem + (size_t)a.warps_per_cta * a.scratch.bytes;
   auto k = dock_chains_kernel<FMT, VAR, APLS>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   int grid = a.n_tiles;
   ChainQueue q{a.counter, a.tickets, a.next_step, a.blocks, 0, 0};
   if (a.queue != kNoQueue) {
-    int per_sm = 0, dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per_sm = 0;
+    const int sms = device_sms();
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * a.warps_per_cta, smem);
     if (e != cudaSuccess) return e;
     const int slots = per_sm * sms > 1 ? per_sm * sms : 1;
@@ -252,7 +246,7 @@ template <int FMT>
 cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
   const size_t smem = (size_t)a.blob_smem + (size_t)a.team * (a.scratch.bytes + 2 * sizeof(TeamSlot));
   auto k = a.team == kMaxTeam ? dock_team_kernel<FMT, 1> : dock_team_kernel<FMT, 2>;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),
                                           reinterpret_cast<const Tile*>(a.tiles), a.blob_smem, a.scratch);
@@ -279,24 +273,17 @@ cudaError_t launch_chains_impl(const ChainLaunch& a, cudaStream_t st) {
 template <int FMT>
 cudaError_t launch_score_impl(const ScoreLaunch& a, cudaStream_t st) {
   const int wpc = 4;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int want = (a.n_conf + wpc - 1) / wpc, cap = sms * 8;  // warps stride over the conformations
   const dim3 block(32 * wpc), grid(want < cap ? want : cap);
   const size_t smem = (size_t)a.blob_smem + (size_t)wpc * a.scratch.bytes;
-  const MapView M = a.map;
-  if (a.apl == 1) {
-    auto k = score_eval_kernel<1, FMT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k<<<grid, block, smem, st>>>(M, a.blob, a.conf, a.n_conf, a.energy, a.grad, a.flags, a.blob_smem, a.scratch);
-  } else {
-    auto k = score_eval_kernel<2, FMT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k<<<grid, block, smem, st>>>(M, a.blob, a.conf, a.n_conf, a.energy, a.grad, a.flags, a.blob_smem, a.scratch);
-  }
+  const bool flat = a.n_conf <= 4 * sms;
+  auto k = a.apl == 1 ? (flat ? score_eval_kernel<1, FMT, true> : score_eval_kernel<1, FMT, false>)
+                      : (flat ? score_eval_kernel<2, FMT, true> : score_eval_kernel<2, FMT, false>);
+  const cudaError_t e = allow_smem((const void*)k, smem);
+  if (e != cudaSuccess) return e;
+  k<<<grid, block, smem, st>>>(a.map, a.blob, a.conf, a.n_conf, a.n_torsions, a.energy, a.grad, a.flags, a.blob_smem,
+                               a.scratch);
   return cudaGetLastError();
 }
 

@@ -72,7 +72,7 @@ struct BodyRec {
   int32_t atom_begin; // subtree atoms [atom_begin, atom_end)
   int32_t atom_end;
   int32_t depth;
-  int32_t pad;
+  int32_t parent_lane;  // written when the blob is staged (stage_blob); 0 in the blob
 };
 static_assert(sizeof(BodyRec) == 48, "body record size");
 

@@ -353,9 +353,7 @@ __global__ void __launch_bounds__(256) gather_bench_kernel(MapView M, const floa
 template <int FMT>
 cudaError_t launch_grid(const dsdp_receptor* rec, int nx, int ny, int nz, float ox, float oy, float oz, float h,
                         void* maps, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   dim3 grid((nx + kBX - 1) / kBX, (ny + kBY - 1) / kBY, (nz + 2 * kBZ - 1) / (2 * kBZ));
   const bool two = (long long)grid.x * grid.y * grid.z >= 4ll * 3 * sms;  // 3 CTAs per SM
   if (!two) grid.z = (nz + kBZ - 1) / kBZ;
@@ -367,9 +365,7 @@ cudaError_t launch_grid(const dsdp_receptor* rec, int nx, int ny, int nz, float 
 template <int FMT>
 cudaError_t launch_gather(const MapView& M, const float* pts, const uint8_t* types, int n, int repeats, float* out,
                           cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int blocks = min((n + 255) / 256, sms * 8);
   gather_bench_kernel<FMT><<<blocks, 256, 0, st>>>(M, pts, types, n, repeats, out);
   return cudaGetLastError();

@@ -4,6 +4,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -115,6 +116,16 @@ static dsdp_status check_view(const dsdp_grid_view* g) {
   return DSDP_OK;
 }
 
+int device_sms() {
+  static std::atomic<int> known[64];
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (dev >= 0 && dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // A job's coordinate scratch: FP64 coordinates while rescoring, the chains' records
@@ -167,6 +178,8 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
 // that the last slices are a small part of the launch, few enough that a slice
 // (a few MC steps, hundreds of evaluations) hides its record's load and store.
 constexpr int kSliceRounds = 16;
+
+constexpr int kSmemPerSm = 228 * 1024;
 
 static ChainQueueMode queue_mode(const dsdp_plan* P) {
   return (P->flags & DSDP_PLAN_PERSISTENT) ? kQueue : P->auto_queue ? kQueueIfMany : kNoQueue;
@@ -274,6 +287,7 @@ extern "C" dsdp_status dsdp_score_eval_device(const dsdp_grid_view* grid, const 
   a.grad = d_grad;
   a.flags = flags;
   a.apl = n_atoms <= 32 ? 1 : 2;
+  a.n_torsions = T;
   a.blob_smem = (int)((const BlobHeader*)h_blob)->stage_bytes;
   a.scratch = scratch_layout(n_atoms, T);
   return check_cuda(launch_score_dispatch(map_fmt(grid->dtype, grid->mode), a, (cudaStream_t)stream),
@@ -523,6 +537,12 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
     a.overlap = gi > 0 && queue != kNoQueue;
     a.variant = P->variant;
+    // 96 registers are for more than 16 warps per SM: where the ligands' shared memory
+    // allows no more, the 128-register kernel (64 ligands of 10-60 atoms 59.6 against
+    // 62.1 ms)
+    if (P->auto_queue && a.variant == 1 &&
+        kSmemPerSm / (a.blob_smem + a.warps_per_cta * a.scratch.bytes + 1024) * a.warps_per_cta <= 16)
+      a.variant = 0;
     a.team = P->team;
     cudaError_t e = launch_chains_dispatch(g.fmt, a, st);
     if (e != cudaSuccess) return check_cuda(e, "dock_chains_kernel launch");

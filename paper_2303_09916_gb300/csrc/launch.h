@@ -42,6 +42,7 @@ struct ScoreLaunch {
   float* grad;
   uint32_t flags;
   int apl;
+  int n_torsions;
   int blob_smem;
   ScratchLayout scratch;
 };
@@ -56,6 +57,15 @@ DSDP_DECLARE_FMT(3)
 DSDP_DECLARE_FMT(4)
 DSDP_DECLARE_FMT(5)
 #undef DSDP_DECLARE_FMT
+
+// SMs of the current device (asked for once per device).
+int device_sms();
+// Lets a kernel use `smem` bytes of dynamic shared memory; below 48 KB it may anyway,
+// and the call would cost a fifth of a launch.
+inline cudaError_t allow_smem(const void* kernel, size_t smem) {
+  return smem <= 47 * 1024 ? cudaSuccess
+                           : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
 
 MapView map_view_of(const dsdp_grid_view* g);
 cudaError_t launch_rescore(const void* jobs, const void* tiles, int n_tiles, cudaStream_t st);

@@ -411,7 +411,7 @@ cudaError_t launch_topk(const void* jobs, int n_jobs, int max_chains, cudaStream
   int np2 = 1;
   while (np2 < max_chains) np2 <<= 1;
   const size_t smem = (size_t)np2 * (sizeof(double) + sizeof(int));
-  cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)topk_kernel, smem);
   if (e != cudaSuccess) return e;
   topk_kernel<<<n_jobs, 512, smem, st>>>(reinterpret_cast<const DevJob*>(jobs), np2);
   return cudaGetLastError();

@@ -34,7 +34,7 @@
 #include <math.h>
 #include <stdint.h>
 
-#include "dsdp_internal.h"
+#include "launch.h"
 
 namespace dsdp {
 namespace {
@@ -334,9 +334,7 @@ extern "C" dsdp_status dsdp_voxelize_device(int32_t n_atoms, const float* d_xyz,
   unsigned long long* acc = (unsigned long long*)d_work;
   const int total = kVoxN * kVoxN * kVoxN * kVoxC;
   const float lox = (float)(center[0] - 35.0), loy = (float)(center[1] - 35.0), loz = (float)(center[2] - 35.0);
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int want = (n_atoms + 7) / 8, cap = sms * 8;  // 8 warps (atoms) per CTA
   const int grid = want < cap ? want : cap;
   const CellLists lists = cell_lists(d_out, n_atoms);
