@@ -20,7 +20,53 @@ constexpr int kRescoreWarps = 8;  // poses of a tile
 // 8 leave SMs with 16 and SMs with 24 of them, in CTAs of 2 with 20 and 22.
 constexpr int kSplit = 4, kCtaWarps = kRescoreWarps / kSplit;
 constexpr int kRecTile = 512;
-constexpr int kExpTable = 256;
+
+// gauss1 + gauss2 of the surface distance d in [-4, 5) as Taylor polynomials of degree
+// 9 about the middles of intervals of 1/32 A (the first term left out is below 3e-19,
+// a thousandth of FP64's rounding of the energies): with f = exp(-4 (c + x)^2),
+// f' = -8 (c + x) f gives (n + 1) a_{n+1} = -8 c a_n - 8 a_{n-1}; the second Gaussian alike.
+constexpr int kIntervals = 288, kDegree = 9;
+constexpr double kFirstD = -4.0;
+struct alignas(16) SmoothRow {
+  double center;
+  double a[kDegree + 1];
+  double pad;
+};
+struct SmoothTable {
+  SmoothRow row[kIntervals];
+};
+// exp(x), -100 < x <= 0: x = n ln 2 + r, Taylor series of exp(r)
+constexpr double exp_series(double x) {
+  int n = 0;
+  while (x + n * 0.69314718055994530942 < -0.34657359027997265) ++n;
+  const double r = (x + n * 0.693147180369123816490) + n * 1.90821492927058770002e-10;  // ln 2 in two parts
+  double term = 1.0, sum = 0.0;
+  double part[26] = {};
+  for (int k = 0; k < 26; ++k) {
+    part[k] = term;
+    term = term * r / (k + 1);
+  }
+  for (int k = 25; k >= 0; --k) sum += part[k];  // small terms first
+  for (; n > 0; --n) sum *= 0.5;
+  return sum;
+}
+constexpr SmoothTable make_smooth_table() {
+  SmoothTable t{};
+  for (int i = 0; i < kIntervals; ++i) {
+    const double c = kFirstD + (i + 0.5) / 32.0, m = c - 3.0;  // c^2, m^2 are exact
+    double a[kDegree + 2] = {}, b[kDegree + 2] = {};
+    a[0] = exp_series(-4.0 * c * c);
+    b[0] = exp_series(-0.25 * m * m);
+    for (int n = 0; n <= kDegree; ++n) {
+      a[n + 1] = (-8.0 * c * a[n] - (n > 0 ? 8.0 * a[n - 1] : 0.0)) / (n + 1);
+      b[n + 1] = (-0.5 * m * b[n] - (n > 0 ? 0.5 * b[n - 1] : 0.0)) / (n + 1);
+    }
+    t.row[i].center = c;
+    for (int n = 0; n <= kDegree; ++n) t.row[i].a[n] = kWGauss1D * a[n] + kWGauss2D * b[n];
+  }
+  return t;
+}
+__device__ const SmoothTable g_smooth = make_smooth_table();
 
 struct DQuat {
   double w, x, y, z;
@@ -37,58 +83,50 @@ __device__ __forceinline__ double3 dqrot(const DQuat& q, double3 v) {
 }
 __device__ __forceinline__ double shd(double v, int src) { return __shfl_sync(kFull, v, src); }
 
-// exp(-t), 0 <= t < 700, by table-driven argument reduction (P. T. P. Tang, ACM TOMS
-// 15, 144 (1989)): exp(-t) = 2^m T[j] exp(r) with 256 m + j the integer nearest
-// -256 t / ln 2, T[j] = 2^(j / 256) and |r| <= ln 2 / 512, where the Taylor
-// polynomial of degree 4 is off by less than 4e-17.  Nine FP64 operations.
-__device__ __forceinline__ double exp_neg(double t, const double* table) {
-  constexpr double kPerLn2 = 256.0 / 0.69314718055994530942;
-  constexpr double kStepHi = 0.69314718055994530942 / 256.0;
-  constexpr double kStepLo = 2.3190468138462996e-17 / 256.0;  // ln 2 minus its FP64 value, over 256
-  constexpr double kRound = 6755399441055744.0;               // 1.5 2^52: adding it leaves the nearest integer
-  const double n = fma(t, -kPerLn2, kRound);
-  const int k = __double2loint(n);
-  const double kd = n - kRound;
-  const double r = fma(-kd, kStepLo, fma(-kd, kStepHi, -t));
-  const double q = fma(r, fma(r, fma(r, 1.0 / 24.0, 1.0 / 6.0), 0.5), 1.0);
-  const double T = table[k & (kExpTable - 1)];
-  const double e = fma(T, r * q, T);
-  return __hiloint2double(__double2hiint(e) + ((k >> 8) << 20), __double2loint(e));
-}
-
-// Square root of r2 >= 0 from the FP32 reciprocal square root by two Newton steps
-// on the root (the first leaves 2^-43 relative, the second FP64 rounding).
-__device__ __forceinline__ double sqrt_d(double r2) {
-  const float y = rsqrt_ftz(fmaxf((float)r2, 1e-30f));
-  const double yd = (double)y, h = (double)(0.5f * y);
-  double r = r2 * yd;
-  r = fma(fma(-r, r, r2), h, r);
-  return fma(fma(-r, r, r2), h, r);
-}
-
-// Tables of the pair terms, in shared memory: 2^(j / 256); per pair of types
-// 9 ti + tj the sum of the radii and the terms it carries (pair_bits).  (Read from
-// the constant bank, the per-lane indices would take up to nine reads each.)
+// Tables of the pair terms, in shared memory: per pair of types 9 ti + tj the sum of
+// the radii and the terms it carries (pair_bits).  (Read from the constant bank, the
+// per-lane indices would take up to nine reads each.)
 struct PairTables {
-  double exp2[kExpTable];
   double radii[81];
+  float radii32[81];
   int bits[81];
 };
 __device__ __forceinline__ void fill_pair_tables(PairTables& P) {
-  for (int k = threadIdx.x; k < kExpTable; k += blockDim.x) P.exp2[k] = ::exp2(k * (1.0 / kExpTable));
   for (int k = threadIdx.x; k < 81; k += blockDim.x) {
     P.radii[k] = c_xs_radius_d[k / 9] + c_xs_radius_d[k % 9];
+    P.radii32[k] = (float)P.radii[k];
     P.bits[k] = pair_bits(k / 9, k % 9);
   }
 }
 
-// Vina-form pair energy at squared distance r2 < 64 (the terms of vina_pair_x2).
+// Vina-form pair energy at squared distance r2 < 66 (the terms of vina_pair_x2), 0
+// from the cutoff on.  The distance: square root from the FP32 reciprocal square root
+// by two Newton steps on the root (the first leaves 2^-43 relative, the second FP64
+// rounding).  The interval of the smooth terms is found in FP32; a neighbour's
+// polynomial serves as well beside a border.
 __device__ __forceinline__ double pair_energy(double r2, int types, const PairTables& P) {
-  const double r = sqrt_d(r2);
+  const float f2 = (float)r2;
+  const float y = rsqrt_ftz(fmaxf(f2, 1e-30f));
+  const double yd = (double)y;
+  const double h = __hiloint2double(__double2hiint(yd) - (1 << 20), __double2loint(yd));  // y / 2
+  double r = r2 * yd;
+  r = fma(fma(-r, r, r2), h, r);
+  r = fma(fma(-r, r, r2), h, r);
   if (!(r < kCutoffD)) return 0.0;
-  const double d = r - P.radii[types], c = d - 3.0;
-  double e = kWGauss1D * exp_neg(4.0 * (d * d), P.exp2);
-  e = fma(kWGauss2D, exp_neg(0.25 * (c * c), P.exp2), e);
+  const int i = (int)((f2 * y - P.radii32[types] - (float)kFirstD) * 32.f);
+  const double2* row = reinterpret_cast<const double2*>(g_smooth.row + min(max(i, 0), kIntervals - 1));
+  const double2 c0 = __ldg(row), c1 = __ldg(row + 1), c2 = __ldg(row + 2), c3 = __ldg(row + 3), c4 = __ldg(row + 4),
+                c5 = __ldg(row + 5);
+  const double d = r - P.radii[types], x = d - c0.x;
+  double e = fma(c5.x, x, c4.y);
+  e = fma(e, x, c4.x);
+  e = fma(e, x, c3.y);
+  e = fma(e, x, c3.x);
+  e = fma(e, x, c2.y);
+  e = fma(e, x, c2.x);
+  e = fma(e, x, c1.y);
+  e = fma(e, x, c1.x);
+  e = fma(e, x, c0.y);
   if (d < 1.5) {  // the short-range terms
     const int bits = P.bits[types];
     if (d < 0.0) e = fma(kWRepulsionD * d, d, e);
@@ -105,8 +143,8 @@ __device__ __forceinline__ double pair_energy(double r2, int types, const PairTa
 // ballot, and evaluates them in FP64 32 at a time with every lane busy.
 //
 // Bound: the FP64 pipe (two results a cycle and SM), so the pair terms are written
-// for few FP64 operations: about 40 a pair where the library's exp and square root
-// took about 70.
+// for few FP64 operations (smooth terms by polynomial, the square root from FP32): about
+// 27 a pair.
 __global__ void __launch_bounds__(32 * kCtaWarps) rescore_kernel(const DevJob* __restrict__ jobs,
                                                                  const Tile* __restrict__ tiles) {
   __shared__ float4 s_rec[kRecTile];
