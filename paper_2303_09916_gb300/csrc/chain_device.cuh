@@ -260,7 +260,10 @@ __device__ __forceinline__ float energy_placed(const MapView& M, const LigView& 
   e_lane += e_pair.x + e_pair.y;
 #pragma unroll
   for (int s = 0; s < APL; ++s)
-    if (P.atom[s] >= 0) e_lane += map_energy<FMT>(M, P.type[s] & 0xff, map_cell(M, P.pos[s]));
+  {  // (a slot without an atom reads atom 0's corners)
+    const float em = map_energy_pairs<FMT>(M, P.type[s] & 0xff, map_cell(M, P.pos[s]));
+    if (P.atom[s] >= 0) e_lane += em;
+  }
   return warp_sum(e_lane);
 }
 

@@ -416,15 +416,9 @@ __device__ __forceinline__ float map_interp(const MapView& M, int t, const MapCe
   return e;
 }
 
-// The score of map_interp alone, by the same operations.
-template <int FMT>
-__device__ __forceinline__ float map_energy(const MapView& M, int t, const MapCell& c) {
-  const unsigned sxy = (unsigned)M.nx * (unsigned)M.ny;
-  const unsigned base = (unsigned)t * sxy * (unsigned)M.nz + c.base;
-  const float v000 = load_score<FMT>(M.maps, base), v100 = load_score<FMT>(M.maps, base + 1);
-  const float v010 = load_score<FMT>(M.maps, base + M.nx), v110 = load_score<FMT>(M.maps, base + M.nx + 1);
-  const float v001 = load_score<FMT>(M.maps, base + sxy), v101 = load_score<FMT>(M.maps, base + sxy + 1);
-  const float v011 = load_score<FMT>(M.maps, base + sxy + M.nx), v111 = load_score<FMT>(M.maps, base + sxy + M.nx + 1);
+// The score of map_interp alone, by the same operations, from the cell's corners.
+__device__ __forceinline__ float map_energy(const MapCell& c, float v000, float v100, float v010, float v110,
+                                            float v001, float v101, float v011, float v111) {
   const float fx = c.fx, fy = c.fy, fz = c.fz;
   const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
   const float w000 = gx0 * gy0 * gz0, w100 = fx * gy0 * gz0, w010 = gx0 * fy * gz0, w110 = fx * fy * gz0;
@@ -435,6 +429,30 @@ __device__ __forceinline__ float map_energy(const MapView& M, int t, const MapCe
   if (c.ey != 0.f) e += kWallSlope * fabsf(c.ey);
   if (c.ez != 0.f) e += kWallSlope * fabsf(c.ez);
   return e;
+}
+
+// map_energy of the lane's atom (type t), all lanes of the warp together.  The two
+// corners along x are neighbours in memory, and a load instruction takes the longer
+// the more cache lines its lanes touch: lanes 2 k and 2 k + 1 read the lower and the
+// upper corner of one's four edges, then of the other's, and swap what is not theirs.
+template <int FMT>
+__device__ __forceinline__ float map_energy_pairs(const MapView& M, int t, const MapCell& c) {
+  const unsigned odd = threadIdx.x & 1;
+  const unsigned sxy = (unsigned)M.nx * (unsigned)M.ny;
+  const unsigned own = (unsigned)t * sxy * (unsigned)M.nz + c.base;
+  const unsigned other = __shfl_xor_sync(kFull, own, 1);
+  const unsigned a = (odd ? other : own) + odd, b = (odd ? own : other) + odd;
+  const unsigned at[4] = {0u, (unsigned)M.nx, sxy, sxy + (unsigned)M.nx};
+  float va[4], vb[4], lo[4], hi[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) va[k] = load_score<FMT>(M.maps, a + at[k]), vb[k] = load_score<FMT>(M.maps, b + at[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float got = __shfl_xor_sync(kFull, odd ? va[k] : vb[k], 1);
+    lo[k] = odd ? got : va[k];
+    hi[k] = odd ? vb[k] : got;
+  }
+  return map_energy(c, lo[0], hi[0], lo[1], hi[1], lo[2], hi[2], lo[3], hi[3]);
 }
 
 template <int FMT>

@@ -149,7 +149,7 @@ template <int FMT, int VAR, int APLS>
 __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>()))
     dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
                        int blob_smem, ScratchLayout lay) {
-  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && (APLS == 1 || (APLS == 2 && fmt_channels(FMT) == 1))>(jobs, tiles, n_tiles, queue, blob_smem, lay);
+  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && APLS == 1>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
 // Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
