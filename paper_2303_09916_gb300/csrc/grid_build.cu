@@ -20,7 +20,7 @@
 //        below half a unit in the last place of gauss2's (half the atoms in range);
 //   mid  (d >= 0): no repulsion, which is exactly 0;
 //   near: all terms.
-// The sums run in units of gauss2's weight and slope, which multiply once at the end.
+// The slopes' sums run in units of gauss2's, which multiplies once at the end.
 // The scan over all receptor atoms is the rest: two blocks a warp (SB = 2) halve it
 // and are taken from four waves of CTAs on; below, the smaller bricks fill the SMs
 // better.
@@ -37,12 +37,10 @@ constexpr float kFarMid = 2.41f;  // surface distance from which gauss1 does not
 // 2^(-u^2) = exp(-b^2) for u = kB2 b; b = (d - 3) / 2
 constexpr float kRootLog2E = 1.2011224087864498f;  // sqrt(1 / ln 2)
 constexpr float kU = 0.5f * kRootLog2E;            // u = kU d - 3 kU
-// units of the sums: energies of kWGauss2, slopes of -kWGauss2 / kRootLog2E (per u exp(-b^2))
+// unit of the slopes' sums: -kWGauss2 / kRootLog2E (per u exp(-b^2))
 constexpr float kSlopeUnit = -kWGauss2 / kRootLog2E;
-constexpr float kE1 = kWGauss1 / kWGauss2;             // gauss1
-constexpr float kS1 = -8.f * kWGauss1 / kSlopeUnit;    //   slope -8 d exp(-4 d^2)
-constexpr float kE3 = kWRepulsion / kWGauss2;          // repulsion m^2, slope 2 m
-constexpr float kS3 = 2.f * kWRepulsion / kSlopeUnit;
+constexpr float kS1 = -8.f * kWGauss1 / kSlopeUnit;  // gauss1: -8 d exp(-4 d^2)
+constexpr float kS3 = 2.f * kWRepulsion / kSlopeUnit;  // repulsion: 2 m
 
 // hydrophobic term of surface distance d (1 below 0.5, linear to 0 at 1.5),
 // added to e and de/dd
@@ -98,7 +96,7 @@ __device__ __forceinline__ void store_node(void* maps, size_t idx, float e, floa
 }
 
 // Sums of one vertex: gauss / repulsion per radius, packed (1.9, 1.8) and (1.7,
-// 2.0): energy and gradient (units above); hydrophobic term of C_H; H-bond terms of
+// 2.0): energy and gradient (in the slopes' unit); hydrophobic term of C_H; H-bond terms of
 // N_D (with receptor acceptors), N_A and O_A (with receptor donors), O_DA (with
 // donors or acceptors): (e, gx, gy, gz).
 struct VertexSums {
@@ -130,16 +128,16 @@ __device__ __forceinline__ void add_radii(float2 d, float2 u, float2 ux, float2 
   const float2 uu = __fmul2_rn(u, u);
   const float2 g2 = make_float2(ex2_approx(-uu.x), ex2_approx(-uu.y));
   float2 p = __fmul2_rn(u, g2);
-  E = __fadd2_rn(E, g2);
+  E = __ffma2_rn(g2, splat2(kWGauss2), E);
   if (KIND != kFar) {
     const float2 dd = __fmul2_rn(d, __fmul2_rn(d, splat2(-4.f * kLog2E)));
     const float2 g1 = make_float2(ex2_approx(dd.x), ex2_approx(dd.y));
-    E = __ffma2_rn(g1, splat2(kE1), E);
+    E = __ffma2_rn(g1, splat2(kWGauss1), E);
     p = __ffma2_rn(__fmul2_rn(g1, d), splat2(kS1), p);
   }
   if (KIND == kNear) {
     const float2 m = make_float2(fminf(d.x, 0.f), fminf(d.y, 0.f));
-    E = __ffma2_rn(__fmul2_rn(m, m), splat2(kE3), E);
+    E = __ffma2_rn(__fmul2_rn(m, m), splat2(kWRepulsion), E);
     p = __ffma2_rn(m, splat2(kS3), p);
   }
   X = __ffma2_rn(p, ux, X);
@@ -295,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 3) grid_build_kernel(int n_rec, cons
     const size_t nxyz = (size_t)nx * ny * nz;
     const size_t v = ((size_t)iz * ny + iy) * nx + ix;
     auto store = [&](int t, float e, float x, float y, float z, const float4& H) {
-      store_node<FMT>(maps, t * nxyz + v, fmaf(e, kWGauss2, H.x), fmaf(x, kSlopeUnit, H.y), fmaf(y, kSlopeUnit, H.z),
+      store_node<FMT>(maps, t * nxyz + v, e + H.x, fmaf(x, kSlopeUnit, H.y), fmaf(y, kSlopeUnit, H.z),
                       fmaf(z, kSlopeUnit, H.w));
     };
     const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
