@@ -652,6 +652,10 @@ struct ChainRecord {
   uint32_t pad;
 };
 static_assert(sizeof(ChainRecord) <= kSliceRecordBytes, "the plan's scratch holds a record per chain");
+__device__ __forceinline__ ChainRecord* chain_record(const DevJob& J, int chain) {
+  return reinterpret_cast<ChainRecord*>(reinterpret_cast<uint8_t*>(J.chain_coords) +
+                                        (size_t)chain * kSliceRecordBytes);
+}
 struct ChainSlice {
   ChainRecord* rec;  // null: the call runs the whole chain
   int* next_step;    // the step the chain stands at, 0 before its start
@@ -1042,7 +1046,8 @@ struct TeamSlot {
 // after the other.  Here warp w evaluates trial t0 + w, all at once, and the first
 // acceptable one in the search's order is taken: the decisions, and so the chain,
 // are run_chain's bit for bit.  Everything between evaluations every warp does for
-// itself, in scratch of its own; one barrier per round.
+// itself, in scratch of its own; one barrier per round.  first > 0: from the chain's
+// record, which stands at that MC step.
 //
 // Bound: latency (a round is one evaluation and one update, 3.2 us; energies first and
 // the winner's gradient after a second barrier: 8 % slower alone and no faster with
@@ -1050,19 +1055,32 @@ struct TeamSlot {
 // system (384 chains, 2.6 evaluations a round with teams of 4) takes 6.1 ms of chain
 // stage against 12.0, one plain-2k system (64 chains, teams of 8) 6.3 against 14.4.
 template <int APL, int FMT>
-__device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W, TeamSlot* ex, int chain) {
+__device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W, TeamSlot* ex, int chain, int first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = blockDim.x >> 5;
   const MapView M = make_map_view(J);
   LaneLig<APL> R;
   load_lane_lig<APL>(L, R);
   const int n_ramp = ramp_steps(L);
   const int T = L.T, nx = 7 + T, D = 6 + T, max_iters = J.n_opt_iters;
-  Conf xt = draw_start(J, T, chain);
-  if (J.trace && J.trace_starts && warp == 0) trace_start(J, chain, xt, T);
+  Conf xt;
   float e_cur = 0.f, e_best = 0.f;
   uint32_t evals = 0;
+  if (first == 0) {
+    xt = draw_start(J, T, chain);
+    if (J.trace && J.trace_starts && warp == 0) trace_start(J, chain, xt, T);
+  } else {
+    const ChainRecord* const rec = chain_record(J, chain);
+    if (lane < nx) {
+      W.cur[lane] = __ldcg(rec->cur + lane);
+      W.best[lane] = __ldcg(rec->best + lane);
+    }
+    e_cur = __ldcg(&rec->e_cur);
+    e_best = __ldcg(&rec->e_best);
+    evals = __ldcg(&rec->evals);
+    __syncwarp();
+  }
   int round = 0;
-  for (int step = 0;; ++step) {
+  for (int step = first;; ++step) {
     if (step > 0) xt = mutated_conf(J, L, W, chain, (uint32_t)step, T);
     // ---- the start, evaluated by warp 0
     float e = 0.f, g = 0.f;

@@ -63,12 +63,19 @@ __host__ __device__ constexpr int chain_min_blocks() {
 // an item of a tile that is still running is left to the CTA that runs it
 // (tickets), which goes on with the tile's next slice.  The slices come in the
 // order of the work that their chains have left, most first (plan_tiles).
+//
+// The queue runs dry while the slowest chains still have slices to go: in the end a
+// few of them decide how long the launch takes.  Once no more than team_when CTAs
+// are left, they leave their chains in the records, and dock_team_kernel finishes
+// those, several warps to a chain.
 struct ChainQueue {
   int* counter;              // the next item
+  int* exited;               // CTAs that found nothing left to do
   int* tickets;              // [n_tiles] items taken and not finished
   int* next_step;            // [n_tiles][W] the step each chain stands at
   const SliceBlock* blocks;  // by item_begin
   int n_blocks, n_items;
+  int team_when;             // 0: every chain is finished here
 };
 
 // The next tile for this CTA, n_tiles when none is left (one thread).  The first
@@ -107,6 +114,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
   if (threadIdx.x == 0) {
     s_job = -1;
     s_tile = queue.n_items ? queue_next(queue, n_tiles) : (int)blockIdx.x;
+    if (queue.n_items && s_tile >= n_tiles) atomicAdd(queue.exited, 1);
   }
   __syncthreads();
   for (;;) {
@@ -125,8 +133,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
       const int chain = tile.chain0 + warp;
       ChainSlice sl{nullptr, nullptr, 0};
       if (queue.n_blocks) {
-        sl.rec = reinterpret_cast<ChainRecord*>(reinterpret_cast<uint8_t*>(J.chain_coords) +
-                                                (size_t)chain * kSliceRecordBytes);
+        sl.rec = chain_record(J, chain);
         sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
         sl.steps = J.slice_steps;
       }
@@ -137,7 +144,14 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();  // this slice's records, before the ticket is given back
-      if (atomicSub(queue.tickets + s_tile, 1) == 1) s_tile = queue_next(queue, n_tiles);
+      if (atomicSub(queue.tickets + s_tile, 1) == 1) {
+        s_tile = queue_next(queue, n_tiles);
+      } else if (queue.team_when && jobs[s_job].optimizer == DSDP_OPT_BFGS &&
+                 *(volatile int*)queue.counter >= queue.n_items &&
+                 (int)gridDim.x - *(volatile int*)queue.exited <= queue.team_when) {
+        s_tile = n_tiles;
+      }
+      if (s_tile >= n_tiles) atomicAdd(queue.exited, 1);
     }
     __syncthreads();
   }
@@ -155,21 +169,27 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, AP
 // Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
 // of kMaxTeam warps the registers must allow per SM; with one chain per SM at most,
 // one (64 plain-2k chains 5.9 ms against 6.2), else two, which is 128 registers and
-// four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5).
+// four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5).  next_step: the
+// chains that a time-sliced launch left unfinished (ChainQueue), from their records;
+// null: whole chains.
 template <int FMT, int MB>
 __global__ void __launch_bounds__(32 * kMaxTeam, MB)
-    dock_team_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int blob_smem,
-                     ScratchLayout lay) {
+    dock_team_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, const int* next_step,
+                     int blob_smem, ScratchLayout lay) {
   extern __shared__ __align__(16) uint8_t smem[];
+  // as in dock_chains_kernel: a next group may start where this one leaves room
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const Tile tile = tiles[blockIdx.x];
   const DevJob& J = jobs[tile.job];
+  const int first = next_step ? __ldcg(next_step + blockIdx.x) : 0;
+  if (first > J.n_steps) return;
   stage_blob(smem, J.blob, reinterpret_cast<const BlobHeader*>(J.blob)->stage_bytes);
   const LigView L = view_blob(smem);
   uint8_t* const scratch = smem + blob_smem;
   const WarpScratch W = warp_scratch_at(scratch + (threadIdx.x >> 5) * lay.bytes, lay);
   TeamSlot* const ex = reinterpret_cast<TeamSlot*>(scratch + (blockDim.x >> 5) * lay.bytes);
-  if (L.n_atoms <= 32) run_team<1, FMT>(J, L, W, ex, tile.chain0);
-  else run_team<2, FMT>(J, L, W, ex, tile.chain0);
+  if (L.n_atoms <= 32) run_team<1, FMT>(J, L, W, ex, tile.chain0, first);
+  else run_team<2, FMT>(J, L, W, ex, tile.chain0, first);
 }
 
 // Score + gradient of a batch of conformations: one warp per conformation,
@@ -213,15 +233,15 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   int grid = a.n_tiles;
-  ChainQueue q{a.counter, a.tickets, a.next_step, a.blocks, 0, 0};
+  ChainQueue q{a.counter, a.exited, a.tickets, a.next_step, a.blocks, 0, 0, a.team_when};
   if (a.queue != kNoQueue) {
     int per_sm = 0;
     const int sms = device_sms();
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * a.warps_per_cta, smem);
     if (e != cudaSuccess) return e;
     const int slots = per_sm * sms > 1 ? per_sm * sms : 1;
-    if (a.n_tiles > slots) {
-      grid = slots;
+    if (a.n_tiles > slots || a.team_when) {
+      grid = a.n_tiles < slots ? a.n_tiles : slots;
       q.n_blocks = a.n_blocks;
       q.n_items = a.n_items;
     } else if (a.queue == kQueue) {
@@ -249,7 +269,8 @@ cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
   const cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),
-                                          reinterpret_cast<const Tile*>(a.tiles), a.blob_smem, a.scratch);
+                                          reinterpret_cast<const Tile*>(a.tiles), a.team_resumes ? a.next_step : nullptr,
+                                          a.blob_smem, a.scratch);
   return cudaGetLastError();
 }
 

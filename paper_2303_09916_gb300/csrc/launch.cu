@@ -31,11 +31,13 @@ struct dsdp_plan {
   void* d_jobs = nullptr;
   void* d_tiles = nullptr;
   void* d_rtiles = nullptr;
-  // work queue: [kMaxGroups counters, one per group][tickets per tile][next step per tile and warp]; zeroed by each launch
+  // work queue: [kMaxGroups counters, one per group][kMaxGroups exit counts][tickets per tile][next step per tile and warp]; zeroed by each launch
   int* d_queue = nullptr;
   size_t queue_bytes = 0;
   size_t queue_next_off = 0;  // of the next steps, in ints
   bool auto_queue = false;    // no fixed choice: queue when a group has more tiles than fit at once
+  bool any_bfgs = false;
+  bool resident = false;      // 16 chains per SM or fewer
   int team = 1;               // no fixed choice, few chains: warps of each (dock_team_kernel)
   void* d_blocks = nullptr;
   int n_rtiles = 0;
@@ -176,8 +178,11 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
 
 // Slices of the launch's longest chains when it time-slices (ChainQueue): enough
 // that the last slices are a small part of the launch, few enough that a slice
-// (a few MC steps, hundreds of evaluations) hides its record's load and store.
-constexpr int kSliceRounds = 16;
+// (a few MC steps, hundreds of evaluations) hides its record's load and store.  When
+// all chains have a place at once they seldom move and what counts is how soon the
+// slowest reach the teams: slices of one MC step (1,536 chains as above: 11.6 ms, in
+// 16 slices 12.8).
+constexpr int kSliceRounds = 16, kSliceRoundsResident = 64;
 
 constexpr int kSmemPerSm = 228 * 1024;
 
@@ -235,6 +240,13 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
       P->groups.push_back(g);
     }
 }
+
+// Chains per SM that a time-sliced launch leaves to teams of 4 (chain stage of 1,536
+// chains of 20-36 atoms: never 17.1 ms, from 4 per SM on 13.7, from 8 on 11.6; 2,000
+// typical-4k chains 8.25, 8.0, 7.3).  Not when a group's chains outnumber their places
+// and another group waits for these: the teams must wait for the whole group, and the
+// other starts behind them (64 ligands of 10-60 atoms: never 60.5 ms, from 8 on 62).
+constexpr int kTailTeams = 8;
 
 // Warps of a chain (dock_team_kernel) when the plan's chains leave most of the GPU
 // idle; 1 when they do not.  Up to one chain per SM a team of 8 (64 plain-2k chains
@@ -381,7 +393,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
   size_t total_chains = 0, max_blocks = 0;
-  bool all_bfgs = true;
+  bool all_bfgs = true, any_bfgs = false;
   {
     // Length of a job's chains, relative: evaluations (MC steps; Barzilai-Borwein
     // runs all its iterations, BFGS about 60 of 100) times the cost of one (the
@@ -397,12 +409,18 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
       longest = std::max(longest, cost);
       total_chains += (size_t)dj[j].n_chains;
     }
-    for (int j = 0; j < n_jobs; ++j) all_bfgs = all_bfgs && dj[j].optimizer == DSDP_OPT_BFGS;
+    for (int j = 0; j < n_jobs; ++j) {
+      const bool bfgs = dj[j].optimizer == DSDP_OPT_BFGS;
+      all_bfgs = all_bfgs && bfgs;
+      any_bfgs = any_bfgs || bfgs;
+    }
+    P->any_bfgs = any_bfgs;
+    P->resident = total_chains <= (size_t)16 * P->sms;
     P->job_order.resize(n_jobs);
     for (int j = 0; j < n_jobs; ++j) {
       P->job_order[j] = j;
       // slices of about the same length whatever the job
-      const int steps = dj[j].n_steps + 1, want = (int)ceil(kSliceRounds * P->shape[j].cost / longest);
+      const int steps = dj[j].n_steps + 1, want = (int)ceil((P->resident ? kSliceRoundsResident : kSliceRounds) * P->shape[j].cost / longest);
       dj[j].slice_steps = (steps + want - 1) / want;
       P->shape[j].slices = (steps + dj[j].slice_steps - 1) / dj[j].slice_steps;
       max_blocks += P->shape[j].slices;
@@ -421,19 +439,16 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     P->tune_key = tune_key(fmt_mask, apl_max, total_chains);
     int var = 0, pers = (flags & DSDP_PLAN_PERSISTENT) ? 1 : 0;
     if (tile_config == 0) {
-      // Without a recorded choice, by what is resident at 16 warps per SM (128
-      // registers).  Up to one such wave every chain has a place at once: no queue,
-      // and ligands above 32 atoms, whose staged blobs are large, in tiles of 4
-      // chains.  More chains: the time-sliced queue, one chain per CTA (64 ligands
-      // of 10-60 atoms x 128 chains 71 ms, in tiles of 2 and 4 72 - 77 ms; 16
-      // typical-4k systems 29.6 against 31.0 and 33 ms).  From two waves on the
-      // 96-register kernel, whose 20 resident warps per SM issue more per cycle (16
-      // typical-4k systems 29.6 against 31.0 ms), below the 128-register kernel,
-      // whose fewer instructions per evaluation win on a part-filled GPU (one
-      // typical-4k system 17.3 against 19.1 ms).
+      // Without a recorded choice, by the number of chains.  Up to 8 per SM: teams, or
+      // (Barzilai-Borwein has no line search) one warp per chain, ligands above 32
+      // atoms, whose staged blobs are large, in tiles of 4 chains.  More: the
+      // time-sliced queue, one chain per CTA (16 typical-4k systems 29.6 ms, in tiles
+      // of 2 and 4 31.0 and 33).  From two waves of 16 per SM on the 96-register kernel,
+      // whose 20 resident warps per SM issue more per cycle, below the 128-register
+      // kernel, whose fewer instructions per evaluation win on a part-filled GPU.
       const size_t wave = (size_t)16 * P->sms;
       var = total_chains >= 2 * wave ? 1 : 0;
-      const bool many = total_chains > wave;
+      const bool many = total_chains > wave / 2;
       W = apl_max == 2 && !many ? 4 : 1;
       if (tune_lookup(P->tune_key, &var, &pers, &W)) {
         if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
@@ -455,8 +470,8 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   P->n_rtiles = (int)rtiles.size();
   const size_t b_jobs = up256(sizeof(DevJob) * n_jobs), b_tiles = up256(sizeof(Tile) * total_chains),
                b_rtiles = up256(sizeof(Tile) * rtiles.size()), b_blocks = up256(sizeof(SliceBlock) * max_blocks);
-  P->queue_next_off = kMaxGroups + total_chains;
-  P->queue_bytes = sizeof(int) * (kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);  // tiles of W <= 4 may be part filled
+  P->queue_next_off = 2 * kMaxGroups + total_chains;
+  P->queue_bytes = sizeof(int) * (2 * kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);  // tiles of W <= 4 may be part filled
   const size_t b_cnt = up256(P->queue_bytes);
   P->arena_bytes = b_jobs + b_tiles + b_rtiles + b_blocks + b_cnt + scratch;
   P->arena = ctx_alloc(ctx, P->arena_bytes, nullptr);
@@ -504,6 +519,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
 extern "C" int32_t dsdp_plan_kernel_count(const dsdp_plan* P) {
   if (!P) return 0;
   int n = (int)P->groups.size();
+  if (P->auto_queue && P->any_bfgs && (P->resident || n == 1)) n *= 2;  // teams for the chains left over
   if (!(P->flags & DSDP_PLAN_NO_RESCORE)) n += 2;
   return n;
 }
@@ -525,7 +541,8 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.n_tiles = g.n_tiles;
     a.queue = queue;
     a.counter = P->d_queue + gi;
-    a.tickets = P->d_queue + kMaxGroups + g.first_tile;
+    a.exited = P->d_queue + kMaxGroups + gi;
+    a.tickets = P->d_queue + 2 * kMaxGroups + g.first_tile;
     a.next_step = P->d_queue + P->queue_next_off + (size_t)g.first_tile * P->warps_per_cta;
     a.blocks = (const SliceBlock*)P->d_blocks + g.first_block;
     a.n_blocks = g.n_blocks;
@@ -544,8 +561,16 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
         kSmemPerSm / (a.blob_smem + a.warps_per_cta * a.scratch.bytes + 1024) * a.warps_per_cta <= 16)
       a.variant = 0;
     a.team = P->team;
+    a.team_resumes = false;
+    a.team_when = P->auto_queue && P->any_bfgs && (P->resident || P->groups.size() == 1) ? kTailTeams * P->sms : 0;
     cudaError_t e = launch_chains_dispatch(g.fmt, a, st);
     if (e != cudaSuccess) return check_cuda(e, "dock_chains_kernel launch");
+    if (a.team_when) {  // the chains it leaves
+      a.team = 4;
+      a.team_resumes = true;
+      e = launch_chains_dispatch(g.fmt, a, st);
+      if (e != cudaSuccess) return check_cuda(e, "dock_team_kernel launch");
+    }
   }
   if ((stages & DSDP_STAGE_RESCORE) && !(P->flags & DSDP_PLAN_NO_RESCORE)) {
     cudaError_t e = launch_rescore(P->d_jobs, P->d_rtiles, P->n_rtiles, st);

@@ -19,6 +19,7 @@ struct ChainLaunch {
   int n_tiles;
   ChainQueueMode queue;
   int* counter;       // the queue's device arrays (ChainQueue), zeroed before the launch
+  int* exited;
   int* tickets;
   int* next_step;
   const SliceBlock* blocks;  // device; the items of a time-sliced launch
@@ -26,6 +27,8 @@ struct ChainLaunch {
   bool overlap;       // independent of the launch before it on the stream: its CTAs may start as that one's leave
   int warps_per_cta;
   int team;           // warps of a chain (dock_team_kernel); 1: none of it
+  bool team_resumes;  // the team finishes what a time-sliced launch left
+  int team_when;      // CTAs left when a time-sliced launch leaves the rest to a team; 0: never
   int apl;            // largest atoms-per-lane tile present
   int apl_mask;       // tiles present: bit 0 one atom per lane (<= 32 atoms), bit 1 two (<= 64)
   int blob_smem;      // bytes reserved for the largest staged blob prefix

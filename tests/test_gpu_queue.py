@@ -17,23 +17,27 @@ from paper_2303_09916_gb300 import dsdp  # noqa: E402
 BOX, H = 14.0, 0.375
 # (atoms, torsions, map format, chains, MC steps, optimiser): more than 20 x 152 chains in each group of the first two;
 # chain counts that leave part-filled tiles, ligands of less than 10 atoms (their records outgrow the coordinates),
-# one MC step (a single-slice chain beside many-slice ones)
+# one MC step (a single-slice chain beside many-slice ones).  The first set outnumbers the chains' places; the others
+# have a place for each, and their slowest chains are finished by teams of warps: of one tile size with
+# Barzilai-Borwein chains among them, and of both
+FEW = [[(30, 8, 0, 900, 5, 0), (24, 5, 0, 600, 3, 0), (32, 6, 0, 300, 4, 1)],
+       [(20, 4, 1, 700, 6, 0), (60, 15, 1, 500, 3, 0), (33, 8, 1, 300, 2, 0)]]
 JOBS = [(30, 8, 0, 3501, 5, 0), (9, 2, 0, 703, 1, 0), (32, 6, 0, 130, 3, 1), (40, 10, 0, 3103, 3, 0), (60, 15, 0, 61, 2, 0),
         (12, 0, 1, 90, 4, 0)]
 
 
-def _jobs(dev, stream):
+def _jobs(dev, stream, spec):
     rec = synth.receptor(1200, 23)
     xyz, ty = torch.from_numpy(rec.xyz).to(dev), torch.from_numpy(rec.xs_type).to(dev)
     box = dsdp.make_box(rec.pocket_center, BOX, H)
     n = [int(np.ceil(BOX / H))] * 3
     keep, jobs, maps = [xyz, ty], [], {}
-    for dtype in (0, 1):
+    for dtype in {s[2] for s in spec}:
         nb = dsdp.dsdp_grid_map_bytes(box, dtype)
         maps[dtype] = torch.empty(nb, dtype=torch.uint8, device=dev)
         dsdp.dsdp_grid_build_device(len(ty), xyz.data_ptr(), ty.data_ptr(), box, dtype, 0, maps[dtype].data_ptr(), nb,
                                     stream)
-    for i, (atoms, T, dtype, chains, steps, opt) in enumerate(JOBS):
+    for i, (atoms, T, dtype, chains, steps, opt) in enumerate(spec):
         lig = synth.ligand(atoms, T, 90 + i, center=rec.pocket_center)
         blob = dsdp.dsdp_ligand_pack(lig)
         nx = 7 + lig.n_torsions
@@ -68,13 +72,13 @@ def _take(outs):
     return got
 
 
-@pytest.mark.parametrize("graph", [False, True])
-def test_sliced_chains_are_the_whole_chains(graph):
+@pytest.mark.parametrize("spec,graph", [(JOBS, False), (JOBS, True), (FEW[0], False), (FEW[1], False), (FEW[1], True)])
+def test_sliced_chains_are_the_whole_chains(spec, graph):
     dev = torch.device("cuda", 0)
     side = torch.cuda.Stream()
     with torch.cuda.stream(side):
         stream = side.cuda_stream
-        jobs, keep, outs, maps = _jobs(dev, stream)
+        jobs, keep, outs, maps = _jobs(dev, stream, spec)
         plan = dsdp.dsdp_plan_create(None, jobs, 0, 1)  # 128 registers, one chain per CTA, no queue
         dsdp.dsdp_plan_launch(plan, stream)
         want = _take(outs)
