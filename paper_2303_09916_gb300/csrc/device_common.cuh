@@ -431,26 +431,39 @@ __device__ __forceinline__ float map_energy(const MapCell& c, float v000, float 
   return e;
 }
 
-// map_energy of the lane's atom (type t), all lanes of the warp together.  The two
-// corners along x are neighbours in memory, and a load instruction takes the longer
-// the more cache lines its lanes touch: lanes 2 k and 2 k + 1 read the lower and the
-// upper corner of one's four edges, then of the other's, and swap what is not theirs.
+// The corners of the cell of the lane's atom (type t), all lanes of the warp
+// together, and map_energy from them.  The two corners along x are neighbours in
+// memory, and a load instruction takes the longer the more cache lines its lanes
+// touch: lanes 2 k and 2 k + 1 read the lower and the upper corner of one's four
+// edges, then of the other's, and swap what is not theirs (on use, so that the loads
+// may be on their way while something else is computed).
+struct CornerPairs {
+  float va[4], vb[4];
+};
 template <int FMT>
-__device__ __forceinline__ float map_energy_pairs(const MapView& M, int t, const MapCell& c) {
+__device__ __forceinline__ CornerPairs load_corner_pairs(const MapView& M, int t, unsigned cell) {
   const unsigned odd = threadIdx.x & 1;
   const unsigned sxy = (unsigned)M.nx * (unsigned)M.ny;
-  const unsigned own = (unsigned)t * sxy * (unsigned)M.nz + c.base;
+  const unsigned own = (unsigned)t * sxy * (unsigned)M.nz + cell;
   const unsigned other = __shfl_xor_sync(kFull, own, 1);
   const unsigned a = (odd ? other : own) + odd, b = (odd ? own : other) + odd;
   const unsigned at[4] = {0u, (unsigned)M.nx, sxy, sxy + (unsigned)M.nx};
-  float va[4], vb[4], lo[4], hi[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) va[k] = load_score<FMT>(M.maps, a + at[k]), vb[k] = load_score<FMT>(M.maps, b + at[k]);
+  CornerPairs v;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float got = __shfl_xor_sync(kFull, odd ? va[k] : vb[k], 1);
-    lo[k] = odd ? got : va[k];
-    hi[k] = odd ? vb[k] : got;
+    v.va[k] = load_score<FMT>(M.maps, a + at[k]);
+    v.vb[k] = load_score<FMT>(M.maps, b + at[k]);
+  }
+  return v;
+}
+__device__ __forceinline__ float map_energy_pairs(const MapCell& c, const CornerPairs& v) {
+  const bool odd = threadIdx.x & 1;
+  float lo[4], hi[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float got = __shfl_xor_sync(kFull, odd ? v.va[k] : v.vb[k], 1);
+    lo[k] = odd ? got : v.va[k];
+    hi[k] = odd ? v.vb[k] : got;
   }
   return map_energy(c, lo[0], hi[0], lo[1], hi[1], lo[2], hi[2], lo[3], hi[3]);
 }
