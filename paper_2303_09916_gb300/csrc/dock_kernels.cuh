@@ -33,18 +33,6 @@ template <>
 struct ChainOcc<3> {
   static constexpr int kMinBlocks = 7;  // 73 -> 72 registers
 };
-// The minimum CTAs per SM a kernel is compiled for.  Variant 1 of the
-// one-atom-per-lane tiles takes none (0: the launch bound then names only the
-// CTA size): the compiler's own allocation for it is 96 registers without
-// spills (tests/test_kernel_registers_cpu.py checks every variant's count), and
-// that kernel ran the 32-system typical-4k chain stage in 67.4 ms against 69.0
-// for the same budget reached through a bound of 5 CTAs per SM (three runs
-// each): the bound changes how the compiler schedules, not the register count.
-template <int VAR, int APLS>
-__host__ __device__ constexpr int chain_min_blocks() {
-  return ChainOcc<VAR>::kMinBlocks;
-}
-
 // Chains: a CTA runs one tile of up to W chains of one job; W = blockDim / 32.
 // The job's ligand blob is staged into shared memory once per tile; ligands of
 // up to 32 atoms run one atom per lane, larger ones two, whatever else the
@@ -160,7 +148,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
 }
 
 template <int FMT, int VAR, int APLS>
-__global__ void __launch_bounds__(32 * kMaxChainWarps, (chain_min_blocks<VAR, APLS>()))
+__global__ void __launch_bounds__(32 * kMaxChainWarps, ChainOcc<VAR>::kMinBlocks)
     dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
                        int blob_smem, ScratchLayout lay) {
   chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && APLS == 1>(jobs, tiles, n_tiles, queue, blob_smem, lay);
@@ -232,6 +220,8 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   auto k = dock_chains_kernel<FMT, VAR, APLS>;
   cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
+  const int cached = kChainSmemPerSm / (int)(smem + 1024);  // CTAs per SM (1 KB each is the system's)
+  const bool carve = APLS == 1 && cached * a.warps_per_cta >= kChainSmemWarps;
   int grid = a.n_tiles;
   ChainQueue q{a.counter, a.exited, a.tickets, a.next_step, a.blocks, 0, 0, a.team_when};
   if (a.queue != kNoQueue) {
@@ -239,6 +229,7 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
     const int sms = device_sms();
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * a.warps_per_cta, smem);
     if (e != cudaSuccess) return e;
+    if (carve && cached < per_sm) per_sm = cached;
     const int slots = per_sm * sms > 1 ? per_sm * sms : 1;
     if (a.n_tiles > slots || a.team_when) {
       grid = a.n_tiles < slots ? a.n_tiles : slots;
@@ -253,11 +244,16 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = a.overlap ? 1 : 0;
+  cudaLaunchAttribute attr[2]{};
+  cfg.attrs = attr;
+  if (a.overlap) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (carve) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[cfg.numAttrs++].val.sharedMemCarveout = 100 * kChainSmemPerSm / kSmemPerSm;
+  }
   return cudaLaunchKernelEx(&cfg, k, reinterpret_cast<const DevJob*>(a.jobs), reinterpret_cast<const Tile*>(a.tiles),
                             a.n_tiles, q, a.blob_smem, a.scratch);
 }

@@ -184,7 +184,6 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
 // 16 slices 12.8).
 constexpr int kSliceRounds = 16, kSliceRoundsResident = 64;
 
-constexpr int kSmemPerSm = 228 * 1024;
 
 static ChainQueueMode queue_mode(const dsdp_plan* P) {
   return (P->flags & DSDP_PLAN_PERSISTENT) ? kQueue : P->auto_queue ? kQueueIfMany : kNoQueue;

@@ -70,6 +70,16 @@ inline cudaError_t allow_smem(const void* kernel, size_t smem) {
                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+constexpr int kSmemPerSm = 228 * 1024;
+// Shared memory an SM sets aside for the chains of one-atom-per-lane tiles where it
+// holds 16 of them; what is left of the SM's 256 KB caches the corners of the atoms'
+// cells, which successive evaluations of a chain mostly share: with 228 KB set aside 32
+// typical-4k systems take 80 ms on the 96-register kernel, with less 52.  Unasked, the
+// driver leaves an SM that never drains with the split of whichever kernel it ran
+// before: four such steps in flight, grid builds and rescoring between them, ran 418
+// systems/s, with this 564 (one at a time 539 either way).
+constexpr int kChainSmemPerSm = 164 * 1024, kChainSmemWarps = 16;
+
 MapView map_view_of(const dsdp_grid_view* g);
 cudaError_t launch_rescore(const void* jobs, const void* tiles, int n_tiles, cudaStream_t st);
 int rescore_tile_chains();
