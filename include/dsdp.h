@@ -359,19 +359,21 @@ typedef struct {
 
 typedef struct dsdp_plan dsdp_plan;
 enum {
-  DSDP_PLAN_PERSISTENT = 1, /* one CTA set sized to the GPU pulls chain tiles from a queue */
+  DSDP_PLAN_PERSISTENT = 1, /* one CTA set sized to the GPU takes slices of chains from a queue */
   DSDP_PLAN_NO_RESCORE = 2  /* stop after the chains (no FP64 rescoring / top-k) */
 };
 /* Prepare a launch of n_jobs jobs (uneven ligands allowed): uploads job and
  * tile tables, sizes scratch (allocated with the ctx allocator; ctx may be NULL
  * for plain cudaMalloc).  One warp runs one chain; a CTA runs a tile of W
  * chains of one job (W = 1, 2 or 4) and stages that job's ligand once.
- * tile_config: 0 = automatic (the choice dsdp_plan_autotune recorded for a plan
- * of the same shape -- map formats, atoms per lane, chain count rounded up to
- * a power of two -- else the 96-register kernel for plans of at least
- * 32 x (SM count) chains and the 128-register kernel for smaller ones, with
- * W = 1, or W = 4 when a ligand has more than 32 atoms); 1 .. 12 = a fixed
- * choice 1 + variant +
+ * tile_config: 0 = automatic: the choice dsdp_plan_autotune recorded for a plan
+ * of the same shape (map formats, atoms per lane, chain count rounded up to
+ * a power of two), else by the plan's size.  Up to 8 chains per SM, all of them
+ * BFGS: teams of 4 warps per chain (8 up to one chain per SM), which evaluate a
+ * line search's trial points at once.  Above: the work queue in slices, longest
+ * chains first, W = 1, the 96-register kernel from 32 x (SM count) chains on and
+ * the 128-register kernel below that or where shared memory allows no more than
+ * 16 warps per SM.  1 .. 12 = a fixed choice 1 + variant +
  * 4 log2(W): register budget (variant 0: 128 registers, 16 warps per SM; 1: 96,
  * 20 warps; 2: 80, 24 warps; 3: 72, 28 warps) and W = 1, 2 or 4.  Budgets 80
  * and 72 are compiled for ligands of up to 32 atoms only (one atom per lane);
@@ -386,7 +388,8 @@ dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsdp_job_devic
  * a group holds only ligands of at most 32 atoms), each tile of W = 1, 2, 4
  * chains per CTA, with and without the
  * persistent work queue, keeps the fastest for this plan and records it for
- * later plans of the same shape (process-wide).  *chosen = 1 + variant
+ * later plans of the same shape (process-wide); the automatic arrangement is
+ * measured first and stays where no fixed one beats it.  *chosen = 1 + variant
  * + 4 * log2(W) + 12 * persistent (1 .. 24; the first part is the plan's
  * tile_config).  ms_by_config: NULL, or 24 floats receiving the measured chain
  * stage time (ms per launch) of configuration chosen - 1, -1 where a
@@ -404,7 +407,8 @@ enum { DSDP_STAGE_CHAINS = 1, DSDP_STAGE_RESCORE = 2, DSDP_STAGE_ALL = 3 };
 /* Enqueue only some stages (e.g. to time the chain kernels alone); stages
  * must run in order: chains before rescoring. */
 dsdp_status dsdp_plan_launch_stage(dsdp_plan* plan, uint32_t stages, void* stream);
-/* Kernel launches one dsdp_plan_launch performs. */
+/* Kernel launches one dsdp_plan_launch performs (a sliced launch's teams for its
+ * slowest chains counted). */
 int32_t dsdp_plan_kernel_count(const dsdp_plan* plan);
 dsdp_status dsdp_plan_destroy(dsdp_ctx* ctx, dsdp_plan* plan);
 
