@@ -229,7 +229,6 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
     const int sms = device_sms();
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * a.warps_per_cta, smem);
     if (e != cudaSuccess) return e;
-    if (carve && cached < per_sm) per_sm = cached;
     const int slots = per_sm * sms > 1 ? per_sm * sms : 1;
     if (a.n_tiles > slots || a.team_when) {
       grid = a.n_tiles < slots ? a.n_tiles : slots;
@@ -252,7 +251,7 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   }
   if (carve) {
     attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[cfg.numAttrs++].val.sharedMemCarveout = 100 * kChainSmemPerSm / kSmemPerSm;
+    attr[cfg.numAttrs++].val.sharedMemCarveout = kChainSmemPercent;
   }
   return cudaLaunchKernelEx(&cfg, k, reinterpret_cast<const DevJob*>(a.jobs), reinterpret_cast<const Tile*>(a.tiles),
                             a.n_tiles, q, a.blob_smem, a.scratch);

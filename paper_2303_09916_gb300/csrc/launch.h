@@ -77,8 +77,9 @@ constexpr int kSmemPerSm = 228 * 1024;
 // typical-4k systems take 80 ms on the 96-register kernel, with less 52.  Unasked, the
 // driver leaves an SM that never drains with the split of whichever kernel it ran
 // before: four such steps in flight, grid builds and rescoring between them, ran 418
-// systems/s, with this 564 (one at a time 539 either way).
-constexpr int kChainSmemPerSm = 164 * 1024, kChainSmemWarps = 16;
+// systems/s, with this 597 (one at a time 539 and 571).  Percent asked for, chain stage
+// on the 96-register kernel: 45 52.9 ms, 59 48.9, 71 52.2, 73 51.5, 87 80.4.
+constexpr int kChainSmemPerSm = 164 * 1024, kChainSmemWarps = 16, kChainSmemPercent = 59;
 
 MapView map_view_of(const dsdp_grid_view* g);
 cudaError_t launch_rescore(const void* jobs, const void* tiles, int n_tiles, cudaStream_t st);
