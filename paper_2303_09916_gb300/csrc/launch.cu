@@ -128,6 +128,31 @@ int device_sms() {
   return sms;
 }
 
+// A kernel has one limit per device, which every thread's launches share: it only ever
+// grows, so that a launch cannot lower it between another thread's call and launch.
+cudaError_t raise_smem(const void* kernel, size_t smem) {
+  struct Limit {
+    const void* kernel;
+    int device;
+    size_t bytes;
+  };
+  static std::mutex mu;
+  static std::vector<Limit> limits;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  Limit* l = nullptr;
+  for (Limit& x : limits)
+    if (x.kernel == kernel && x.device == dev) l = &x;
+  const size_t most = l ? std::max(l->bytes, smem) : smem;
+  const cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (set != cudaSuccess) return set;
+  if (l) l->bytes = most;
+  else limits.push_back(Limit{kernel, dev, most});
+  return cudaSuccess;
+}
+
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // A job's coordinate scratch: FP64 coordinates while rescoring, the chains' records

@@ -65,9 +65,9 @@ DSDP_DECLARE_FMT(5)
 int device_sms();
 // Lets a kernel use `smem` bytes of dynamic shared memory; below 48 KB it may anyway,
 // and the call would cost a fifth of a launch.
+cudaError_t raise_smem(const void* kernel, size_t smem);
 inline cudaError_t allow_smem(const void* kernel, size_t smem) {
-  return smem <= 47 * 1024 ? cudaSuccess
-                           : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return smem <= 47 * 1024 ? cudaSuccess : raise_smem(kernel, smem);
 }
 
 constexpr int kSmemPerSm = 228 * 1024;
