@@ -384,8 +384,8 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
   for (int s = 0; s < APL; ++s) {
     if ((flags & DSDP_TERM_INTER) && atom[s] >= 0) {
       float3 gi;
-      // the cell is located here, where it is used: holding it across the intra
-      // block miscompiled the two-atoms-per-lane kernels (gradient x channel lost)
+      // the cell is located here, where it is used, not held across the intra block:
+      // it would take eight registers of each atom there
       e_lane += map_interp<FMT>(M, type[s] & 0xff, map_cell(M, pos[s]), gi);
       g[s] = g[s] + gi;
     }

@@ -359,6 +359,41 @@ __device__ __forceinline__ MapCell map_cell(const MapView& M, float3 r) {
   return c;
 }
 
+// The eight corners' weights, in memory order (x fastest), and the sums over them and
+// over the four corners of a face: fixed sequences of fused operations, so that every
+// kernel that reads a cell, for its score alone or with its gradient, gets the same
+// bits whatever the compiler would have fused there.
+struct CornerWeights {
+  float w[8];
+};
+__device__ __forceinline__ CornerWeights corner_weights(const MapCell& c) {
+  const float fx = c.fx, fy = c.fy, fz = c.fz;
+  const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
+  return CornerWeights{{gx0 * gy0 * gz0, fx * gy0 * gz0, gx0 * fy * gz0, fx * fy * gz0, gx0 * gy0 * fz, fx * gy0 * fz,
+                        gx0 * fy * fz, fx * fy * fz}};
+}
+__device__ __forceinline__ float corner_sum(const CornerWeights& k, float v0, float v1, float v2, float v3, float v4,
+                                            float v5, float v6, float v7) {
+  float e = __fmaf_rn(k.w[0], v0, __fmul_rn(k.w[1], v1));
+  e = __fmaf_rn(k.w[2], v2, e);
+  e = __fmaf_rn(k.w[3], v3, e);
+  e = __fmaf_rn(k.w[4], v4, e);
+  e = __fmaf_rn(k.w[5], v5, e);
+  e = __fmaf_rn(k.w[6], v6, e);
+  return __fmaf_rn(k.w[7], v7, e);
+}
+__device__ __forceinline__ float face_sum(float w0, float v0, float w1, float v1, float w2, float v2, float w3,
+                                          float v3) {
+  return __fmaf_rn(w3, v3, __fmaf_rn(w2, v2, __fmaf_rn(w0, v0, __fmul_rn(w1, v1))));
+}
+// The score with the out-of-grid wall: kWallSlope per Angstrom of excess along each axis.
+__device__ __forceinline__ float wall_energy(const MapCell& c, float e) {
+  if (c.ex != 0.f) e = __fmaf_rn(kWallSlope, fabsf(c.ex), e);
+  if (c.ey != 0.f) e = __fmaf_rn(kWallSlope, fabsf(c.ey), e);
+  if (c.ez != 0.f) e = __fmaf_rn(kWallSlope, fabsf(c.ez), e);
+  return e;
+}
+
 // Trilinear score (Eq. 2) and gradient (Eq. 4 from the gradient maps, or
 // Eq. 3 as the derivative of the interpolant) for map type t in cell c, with the
 // out-of-grid wall: evaluated at the clamped point plus kWallSlope per
@@ -376,63 +411,34 @@ __device__ __forceinline__ float map_interp(const MapView& M, int t, const MapCe
   const float4 v101 = load_node<FMT>(M.maps, base + sxy + 1);
   const float4 v011 = load_node<FMT>(M.maps, base + sxy + M.nx);
   const float4 v111 = load_node<FMT>(M.maps, base + sxy + M.nx + 1);
-  const float fx = c.fx, fy = c.fy, fz = c.fz;
-  const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
-  const float w000 = gx0 * gy0 * gz0, w100 = fx * gy0 * gz0, w010 = gx0 * fy * gz0, w110 = fx * fy * gz0;
-  const float w001 = gx0 * gy0 * fz, w101 = fx * gy0 * fz, w011 = gx0 * fy * fz, w111 = fx * fy * fz;
-  float e = w000 * v000.x + w100 * v100.x + w010 * v010.x + w110 * v110.x + w001 * v001.x + w101 * v101.x +
-            w011 * v011.x + w111 * v111.x;
+  const CornerWeights k = corner_weights(c);
+  const float e = corner_sum(k, v000.x, v100.x, v010.x, v110.x, v001.x, v101.x, v011.x, v111.x);
   if (fmt_channels(FMT) == 4) {
-    g.x = w000 * v000.y + w100 * v100.y + w010 * v010.y + w110 * v110.y + w001 * v001.y + w101 * v101.y +
-          w011 * v011.y + w111 * v111.y;
-    g.y = w000 * v000.z + w100 * v100.z + w010 * v010.z + w110 * v110.z + w001 * v001.z + w101 * v101.z +
-          w011 * v011.z + w111 * v111.z;
-    g.z = w000 * v000.w + w100 * v100.w + w010 * v010.w + w110 * v110.w + w001 * v001.w + w101 * v101.w +
-          w011 * v011.w + w111 * v111.w;
+    g.x = corner_sum(k, v000.y, v100.y, v010.y, v110.y, v001.y, v101.y, v011.y, v111.y);
+    g.y = corner_sum(k, v000.z, v100.z, v010.z, v110.z, v001.z, v101.z, v011.z, v111.z);
+    g.z = corner_sum(k, v000.w, v100.w, v010.w, v110.w, v001.w, v101.w, v011.w, v111.w);
   } else {
     // d/dx of the trilinear interpolant: difference of the x = 1 and x = 0 faces / h
-    const float f0 = gy0 * gz0 * v000.x + fy * gz0 * v010.x + gy0 * fz * v001.x + fy * fz * v011.x;
-    const float f1 = gy0 * gz0 * v100.x + fy * gz0 * v110.x + gy0 * fz * v101.x + fy * fz * v111.x;
-    const float e0 = gx0 * gz0 * v000.x + fx * gz0 * v100.x + gx0 * fz * v001.x + fx * fz * v101.x;
-    const float e1 = gx0 * gz0 * v010.x + fx * gz0 * v110.x + gx0 * fz * v011.x + fx * fz * v111.x;
-    const float d0 = gx0 * gy0 * v000.x + fx * gy0 * v100.x + gx0 * fy * v010.x + fx * fy * v110.x;
-    const float d1 = gx0 * gy0 * v001.x + fx * gy0 * v101.x + gx0 * fy * v011.x + fx * fy * v111.x;
+    const float fx = c.fx, fy = c.fy, fz = c.fz;
+    const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
+    const float f0 = face_sum(gy0 * gz0, v000.x, fy * gz0, v010.x, gy0 * fz, v001.x, fy * fz, v011.x);
+    const float f1 = face_sum(gy0 * gz0, v100.x, fy * gz0, v110.x, gy0 * fz, v101.x, fy * fz, v111.x);
+    const float e0 = face_sum(gx0 * gz0, v000.x, fx * gz0, v100.x, gx0 * fz, v001.x, fx * fz, v101.x);
+    const float e1 = face_sum(gx0 * gz0, v010.x, fx * gz0, v110.x, gx0 * fz, v011.x, fx * fz, v111.x);
+    const float d0 = face_sum(gx0 * gy0, v000.x, fx * gy0, v100.x, gx0 * fy, v010.x, fx * fy, v110.x);
+    const float d1 = face_sum(gx0 * gy0, v001.x, fx * gy0, v101.x, gx0 * fy, v011.x, fx * fy, v111.x);
     g.x = (f1 - f0) * M.inv_h;
     g.y = (e1 - e0) * M.inv_h;
     g.z = (d1 - d0) * M.inv_h;
   }
-  if (c.ex != 0.f) {
-    e += kWallSlope * fabsf(c.ex);
-    g.x = c.ex > 0.f ? kWallSlope : -kWallSlope;
-  }
-  if (c.ey != 0.f) {
-    e += kWallSlope * fabsf(c.ey);
-    g.y = c.ey > 0.f ? kWallSlope : -kWallSlope;
-  }
-  if (c.ez != 0.f) {
-    e += kWallSlope * fabsf(c.ez);
-    g.z = c.ez > 0.f ? kWallSlope : -kWallSlope;
-  }
-  return e;
-}
-
-// The score of map_interp alone, by the same operations, from the cell's corners.
-__device__ __forceinline__ float map_energy(const MapCell& c, float v000, float v100, float v010, float v110,
-                                            float v001, float v101, float v011, float v111) {
-  const float fx = c.fx, fy = c.fy, fz = c.fz;
-  const float gx0 = 1.f - fx, gy0 = 1.f - fy, gz0 = 1.f - fz;
-  const float w000 = gx0 * gy0 * gz0, w100 = fx * gy0 * gz0, w010 = gx0 * fy * gz0, w110 = fx * fy * gz0;
-  const float w001 = gx0 * gy0 * fz, w101 = fx * gy0 * fz, w011 = gx0 * fy * fz, w111 = fx * fy * fz;
-  float e = w000 * v000 + w100 * v100 + w010 * v010 + w110 * v110 + w001 * v001 + w101 * v101 + w011 * v011 +
-            w111 * v111;
-  if (c.ex != 0.f) e += kWallSlope * fabsf(c.ex);
-  if (c.ey != 0.f) e += kWallSlope * fabsf(c.ey);
-  if (c.ez != 0.f) e += kWallSlope * fabsf(c.ez);
-  return e;
+  if (c.ex != 0.f) g.x = c.ex > 0.f ? kWallSlope : -kWallSlope;
+  if (c.ey != 0.f) g.y = c.ey > 0.f ? kWallSlope : -kWallSlope;
+  if (c.ez != 0.f) g.z = c.ez > 0.f ? kWallSlope : -kWallSlope;
+  return wall_energy(c, e);
 }
 
 // The corners of the cell of the lane's atom (type t), all lanes of the warp
-// together, and map_energy from them.  The two corners along x are neighbours in
+// together, and map_interp's score from them.  The two corners along x are neighbours in
 // memory, and a load instruction takes the longer the more cache lines its lanes
 // touch: lanes 2 k and 2 k + 1 read the lower and the upper corner of one's four
 // edges, then of the other's, and swap what is not theirs (on use, so that the loads
@@ -465,7 +471,7 @@ __device__ __forceinline__ float map_energy_pairs(const MapCell& c, const Corner
     lo[k] = odd ? got : v.va[k];
     hi[k] = odd ? v.vb[k] : got;
   }
-  return map_energy(c, lo[0], hi[0], lo[1], hi[1], lo[2], hi[2], lo[3], hi[3]);
+  return wall_energy(c, corner_sum(corner_weights(c), lo[0], hi[0], lo[1], hi[1], lo[2], hi[2], lo[3], hi[3]));
 }
 
 template <int FMT>
