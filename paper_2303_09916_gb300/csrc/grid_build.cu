@@ -32,7 +32,8 @@ namespace {
 constexpr int kBX = 8, kBY = 8, kBZ = 4, kThreads = kBX * kBY * kBZ;
 constexpr int kChunk = 1536;       // kept atoms staged at once
 constexpr int kTests = 2;          // atoms a thread tests per barrier
-constexpr float kFarMid = 2.41f;  // surface distance from which gauss1 does not change an FP32 sum with gauss2
+constexpr float kSlack = 0.01f;   // what the boxes' tests allow for rounding, in Angstrom (box_slack)
+constexpr float kFarMid = 2.40f + kSlack;  // surface distance from which gauss1 does not change an FP32 sum with gauss2
 
 // 2^(-u^2) = exp(-b^2) for u = kB2 b; b = (d - 3) / 2
 constexpr float kRootLog2E = 1.2011224087864498f;  // sqrt(1 / ln 2)
@@ -207,6 +208,7 @@ template <int FMT, int SB>
 __global__ void __launch_bounds__(kThreads, 3) grid_build_kernel(int n_rec, const float* __restrict__ xyz,
                                                                  const uint8_t* __restrict__ type, int nx, int ny,
                                                                  int nz, float ox, float oy, float oz, float h,
+                                                                 float reach2, float more_slack,
                                                                  void* __restrict__ maps) {
   constexpr int kWarps = kThreads / 32;
   __shared__ float4 s_atom[kChunk];
@@ -215,8 +217,6 @@ __global__ void __launch_bounds__(kThreads, 3) grid_build_kernel(int n_rec, cons
   const int bx0 = blockIdx.x * kBX, by0 = blockIdx.y * kBY, bz0 = blockIdx.z * kBZ * SB;
   const float bcx = ox + h * ((float)bx0 + 0.5f * (kBX - 1)), bcy = oy + h * ((float)by0 + 0.5f * (kBY - 1)),
               bcz = oz + h * ((float)bz0 + 0.5f * (kBZ * SB - 1));
-  // the boxes' tests allow 0.01 A for rounding
-  const float reach2 = (kCutoff + 0.01f) * (kCutoff + 0.01f);
   int count = 0;
   bool staged = false;  // the kept atoms of the whole receptor are in s_atom
 #pragma unroll 1
@@ -278,7 +278,8 @@ __global__ void __launch_bounds__(kThreads, 3) grid_build_kernel(int n_rec, cons
           const bool have = k0 + lane < count;
           const float4 a = have ? s_atom[k0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
           const float d2 = have ? box_dist2(a, wcx, wcy, wcz, 1.5f * h, 1.5f * h, 0.5f * h) : reach2;
-          const float far = 2.0f + kFarMid + c_xs_radius[__float_as_int(a.w)], mid = far - kFarMid + 0.01f;
+          const float far = 2.0f + kFarMid + c_xs_radius[__float_as_int(a.w)] + more_slack,
+                      mid = far - kFarMid + kSlack;
           unsigned m_far = __ballot_sync(kFull, d2 < reach2 && d2 >= far * far);
           unsigned m_mid = __ballot_sync(kFull, d2 < far * far && d2 >= mid * mid);
           unsigned m_near = __ballot_sync(kFull, d2 < mid * mid);
@@ -348,6 +349,18 @@ __global__ void __launch_bounds__(256) gather_bench_kernel(MapView M, const floa
   }
 }
 
+// What the tests of an atom against a brick's or a warp's box allow for rounding: at m
+// Angstrom from the origin a vertex and a box's centre are each at most 2^-24 m off
+// (twice that unfused) along an axis, 4.2e-7 m of distance for both.
+float box_slack(int nx, int ny, int nz, float ox, float oy, float oz, float h) {
+  const int n[3] = {nx, ny, nz};
+  const float o[3] = {ox, oy, oz};
+  double m = 0.0;
+  for (int a = 0; a < 3; ++a)
+    m = fmax(m, fmax(fabs((double)o[a]), fabs((double)o[a] + (double)h * (n[a] + 2 * kBX))));
+  return fmaxf(kSlack, (float)(5e-7 * m));
+}
+
 template <int FMT>
 cudaError_t launch_grid(const dsdp_receptor* rec, int nx, int ny, int nz, float ox, float oy, float oz, float h,
                         void* maps, cudaStream_t st) {
@@ -356,7 +369,9 @@ cudaError_t launch_grid(const dsdp_receptor* rec, int nx, int ny, int nz, float 
   const bool two = (long long)grid.x * grid.y * grid.z >= 4ll * 3 * sms;  // 3 CTAs per SM
   if (!two) grid.z = (nz + kBZ - 1) / kBZ;
   auto k = two ? grid_build_kernel<FMT, 2> : grid_build_kernel<FMT, 1>;
-  k<<<grid, kThreads, 0, st>>>(rec->n, rec->xyz, rec->xs_type, nx, ny, nz, ox, oy, oz, h, maps);
+  const float slack = box_slack(nx, ny, nz, ox, oy, oz, h);
+  k<<<grid, kThreads, 0, st>>>(rec->n, rec->xyz, rec->xs_type, nx, ny, nz, ox, oy, oz, h,
+                               (kCutoff + slack) * (kCutoff + slack), slack - kSlack, maps);
   return cudaGetLastError();
 }
 
