@@ -240,10 +240,12 @@ void layout_results(Job* j) {
   j->res_bytes = o;
 }
 
-// Estimated plan scratch of a job (rescoring arrays and tables).
+// Estimated plan scratch of a job: rescoring arrays and tables (80 bytes a chain, of
+// which the tables are 26; the rest covers what the chains' records of a ligand of
+// one or two atoms are larger than its coordinates).
 uint64_t plan_scratch_estimate(const Job* j) {
   const uint64_t C = (uint64_t)j->params.n_chains;
-  return 4096 + 3 * 8 * C + C * std::max<uint64_t>(8 * j->n_atoms * 3, kSliceRecordBytes) + 64 * C + 16 * C;
+  return 4096 + 3 * 8 * C + 8 * C * j->n_atoms * 3 + 64 * C + 16 * C;
 }
 
 // Device memory, pinned buffer and blob upload of one job on stream st, and

@@ -654,15 +654,16 @@ __device__ __forceinline__ float3 site_start(const DevJob& J, const ChainStream&
 // (dock_chains_kernel) keeps in global memory while another chain has the warp.
 // Another SM may have written it: it is read and written past L1.
 struct ChainRecord {
-  float cur[kConfFloats], best[kConfFloats];
   float e_cur, e_best;
   uint32_t evals;
   uint32_t pad;
+  // [2][7 + T]: the current and the best conformation
+  __device__ __forceinline__ float* conf() { return reinterpret_cast<float*>(this + 1); }
 };
-static_assert(sizeof(ChainRecord) <= kSliceRecordBytes, "the plan's scratch holds a record per chain");
-__device__ __forceinline__ ChainRecord* chain_record(const DevJob& J, int chain) {
+static_assert(sizeof(ChainRecord) == slice_record_bytes(-7), "a record's size");
+__device__ __forceinline__ ChainRecord* chain_record(const DevJob& J, int T, int chain) {
   return reinterpret_cast<ChainRecord*>(reinterpret_cast<uint8_t*>(J.chain_coords) +
-                                        (size_t)chain * kSliceRecordBytes);
+                                        (size_t)chain * (sizeof(ChainRecord) + 8 * (7 + T)));
 }
 struct ChainSlice {
   ChainRecord* rec;  // null: the call runs the whole chain
@@ -868,8 +869,8 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
     if (lane < kHStride) Vg[lane] = Vd[lane] = 0.f;
     if (mutate) {
       if (lane < 7 + T) {
-        W.cur[lane] = __ldcg(sl.rec->cur + lane);
-        W.best[lane] = __ldcg(sl.rec->best + lane);
+        W.cur[lane] = __ldcg(sl.rec->conf() + lane);
+        W.best[lane] = __ldcg(sl.rec->conf() + 7 + T + lane);
       }
       V.e_cur = __ldcg(&sl.rec->e_cur);
       V.e_best = __ldcg(&sl.rec->e_best);
@@ -1017,8 +1018,8 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       if (step == V.stop) {  // end of this slice: the chain waits in its record
         ChainRecord* const rec = V.rec;
         if (lane < nx) {
-          __stcg(rec->cur + lane, W.cur[lane]);
-          __stcg(rec->best + lane, W.best[lane]);
+          __stcg(rec->conf() + lane, W.cur[lane]);
+          __stcg(rec->conf() + nx + lane, W.best[lane]);
         }
         if (lane == 0) {
           __stcg(&rec->e_cur, e_cur);
@@ -1077,10 +1078,10 @@ __device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W
     xt = draw_start(J, T, chain);
     if (J.trace && J.trace_starts && warp == 0) trace_start(J, chain, xt, T);
   } else {
-    const ChainRecord* const rec = chain_record(J, chain);
+    ChainRecord* const rec = chain_record(J, T, chain);
     if (lane < nx) {
-      W.cur[lane] = __ldcg(rec->cur + lane);
-      W.best[lane] = __ldcg(rec->best + lane);
+      W.cur[lane] = __ldcg(rec->conf() + lane);
+      W.best[lane] = __ldcg(rec->conf() + nx + lane);
     }
     e_cur = __ldcg(&rec->e_cur);
     e_best = __ldcg(&rec->e_best);

@@ -121,7 +121,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
       const int chain = tile.chain0 + warp;
       ChainSlice sl{nullptr, nullptr, 0};
       if (queue.n_blocks) {
-        sl.rec = chain_record(J, chain);
+        sl.rec = chain_record(J, L.T, chain);
         sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
         sl.steps = J.slice_steps;
       }

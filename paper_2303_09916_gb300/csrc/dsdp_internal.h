@@ -124,8 +124,9 @@ struct DevJob {
 
 // Bytes of a chain's record in a time-sliced launch (ChainRecord, chain_device.cuh).
 // The records share the rescoring's coordinate scratch (24 n_atoms bytes per
-// chain), which is not in use while the chains run.
-constexpr int kSliceRecordBytes = 8 * (7 + kMaxDim) + 16;
+// chain, which holds them from four atoms on whatever the torsions), which is not in
+// use while the chains run.
+constexpr int slice_record_bytes(int n_torsions) { return 8 * (7 + n_torsions) + 16; }
 
 // Internal plan flag: other launches share the GPU with this plan's (no teams).
 constexpr uint32_t kPlanShared = 1u << 30;

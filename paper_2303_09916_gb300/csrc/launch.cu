@@ -157,8 +157,8 @@ static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // A job's coordinate scratch: FP64 coordinates while rescoring, the chains' records
 // (ChainRecord) while a time-sliced launch runs them.
-static size_t coord_bytes(int n_chains, int n_atoms) {
-  return (size_t)n_chains * std::max(sizeof(double) * 3 * n_atoms, (size_t)kSliceRecordBytes);
+static size_t coord_bytes(int n_chains, int n_atoms, int n_torsions) {
+  return (size_t)n_chains * std::max(sizeof(double) * 3 * n_atoms, (size_t)slice_record_bytes(n_torsions));
 }
 
 // Autotuner choices by plan shape: (format mask, atoms-per-lane, log2 of the
@@ -367,7 +367,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     if (!J.d_chain_best_e) scratch += up256(sizeof(float) * (size_t)p.n_chains);
     if (!J.d_chain_evals) scratch += up256(sizeof(uint32_t) * (size_t)p.n_chains);
     scratch += 3 * up256(sizeof(double) * (size_t)p.n_chains);
-    scratch += up256(coord_bytes(p.n_chains, atoms[j]));
+    scratch += up256(coord_bytes(p.n_chains, atoms[j], tors[j]));
     DevJob& d = dj[j];
     memset(&d, 0, sizeof(d));
     d.blob = (const uint8_t*)J.d_blob;
@@ -525,7 +525,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     d.chain_score = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_inter = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_intra = (double*)take(sizeof(double) * (size_t)d.n_chains);
-    d.chain_coords = (double*)take(coord_bytes(d.n_chains, atoms[j]));
+    d.chain_coords = (double*)take(coord_bytes(d.n_chains, atoms[j], tors[j]));
   }
   cudaError_t e = cudaMemcpy(P->d_jobs, dj.data(), sizeof(DevJob) * n_jobs, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = plan_use_warps(P, W);
