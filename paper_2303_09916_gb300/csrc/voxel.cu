@@ -308,6 +308,11 @@ __global__ void __launch_bounds__(256) voxel_finish_kernel(const unsigned long l
   }
 }
 
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return x < y + nb && y < x + na;
+}
+
 }  // namespace
 }  // namespace dsdp
 
@@ -338,8 +343,13 @@ extern "C" dsdp_status dsdp_voxelize_device(int32_t n_atoms, const float* d_xyz,
   const int want = (n_atoms + 7) / 8, cap = sms * 8;  // 8 warps (atoms) per CTA
   const int grid = want < cap ? want : cap;
   const CellLists lists = cell_lists(d_out, n_atoms);
+  // the lists lie in the output: not where the output may take an input's place
+  const size_t out_bytes = sizeof(float) * (size_t)total, atoms = (size_t)n_atoms;
+  const bool listed = n_atoms > 0 && n_atoms <= kMaxListed && !overlap(d_out, out_bytes, d_xyz, 12 * atoms) &&
+                      !overlap(d_out, out_bytes, d_radius, 4 * atoms) &&
+                      !overlap(d_out, out_bytes, d_features, 4 * kVoxF * atoms);
   cudaError_t e = cudaSuccess;
-  if (n_atoms > 0 && n_atoms <= kMaxListed) {
+  if (listed) {
     voxel_bin_kernel<<<1 + sms, 1024, 0, st>>>(n_atoms, d_xyz, d_radius, lox, loy, loz, lists, acc);
     voxel_atoms_kernel<true>
         <<<grid, 256, 0, st>>>(n_atoms, d_xyz, d_radius, d_features, lox, loy, loz, lists, acc);
