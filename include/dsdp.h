@@ -367,8 +367,9 @@ enum {
  * for plain cudaMalloc).  One warp runs one chain; a CTA runs a tile of W
  * chains of one job (W = 1, 2 or 4) and stages that job's ligand once.
  * tile_config: 0 = automatic: the choice dsdp_plan_autotune recorded for a plan
- * of the same shape (map formats, atoms per lane, chain count rounded up to
- * a power of two), else by the plan's size.  Up to 8 chains per SM, all of them
+ * of the same shape (map formats, atoms per lane, optimisers, chain count
+ * rounded up to a power of two and on the same side of the limits below, SM
+ * count), else by the plan's size.  Up to 8 chains per SM, all of them
  * BFGS: teams of 4 warps per chain (8 up to one chain per SM), which evaluate a
  * line search's trial points at once.  Above: the work queue in slices, longest
  * chains first, W = 1, the 96-register kernel from 32 x (SM count) chains on and

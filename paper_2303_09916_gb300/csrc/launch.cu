@@ -35,10 +35,18 @@ struct dsdp_plan {
   int* d_queue = nullptr;
   size_t queue_bytes = 0;
   size_t queue_next_off = 0;  // of the next steps, in ints
-  bool auto_queue = false;    // no fixed choice: queue when a group has more tiles than fit at once
+  // What runs the chains without a fixed choice: the register budget, chains per CTA,
+  // warps of each chain (dock_team_kernel), and whether a group with more tiles than fit
+  // at once takes the queue.
+  struct Arrangement {
+    int variant, warps, team;
+    bool queue;
+  };
+  Arrangement automatic{0, 1, 1, false};  // by the plan's size, whatever it runs now
+  bool auto_queue = false;    // as it runs now (variant, warps_per_cta): the queue, teams
+  int team = 1;
   bool any_bfgs = false;
   bool resident = false;      // 16 chains per SM or fewer
-  int team = 1;               // no fixed choice, few chains: warps of each (dock_team_kernel)
   void* d_blocks = nullptr;
   int n_rtiles = 0;
   // per job, to lay groups and tiles out again for another configuration
@@ -161,9 +169,8 @@ static size_t coord_bytes(int n_chains, int n_atoms, int n_torsions) {
   return (size_t)n_chains * std::max(sizeof(double) * 3 * n_atoms, (size_t)slice_record_bytes(n_torsions));
 }
 
-// Autotuner choices by plan shape: (format mask, atoms-per-lane, log2 of the
-// chain count) -> (variant, persistent).  Written by dsdp_plan_autotune, read
-// by plans created with tile_config 0.
+// Autotuner choices by plan shape (tune_key): (variant, persistent, warps).  Written
+// by dsdp_plan_autotune, read by plans created with tile_config 0.
 struct TuneEntry {
   uint64_t key;
   int variant, persistent, warps;
@@ -171,10 +178,17 @@ struct TuneEntry {
 static std::mutex g_tune_mu;
 static std::vector<TuneEntry> g_tune;
 
-static uint64_t tune_key(uint32_t fmt_mask, int apl, size_t chains) {
+// Format mask, atoms per lane, log2 of the chain count, the optimisers, and what the
+// choice stands in for: a fixed configuration that beats one automatic arrangement says
+// nothing of another (one warp a chain is the fastest for 384 Barzilai-Borwein chains
+// and takes twice a team's time for BFGS).
+static uint64_t tune_key(uint32_t fmt_mask, int apl, size_t chains, bool all_bfgs, bool any_bfgs,
+                         const dsdp_plan::Arrangement& automatic, int sms) {
   int lg = 0;
   while ((size_t(1) << lg) < chains) ++lg;
-  return ((uint64_t)fmt_mask << 16) | ((uint64_t)apl << 8) | (uint64_t)lg;
+  return (uint64_t)lg | ((uint64_t)apl << 8) | ((uint64_t)fmt_mask << 16) | ((uint64_t)all_bfgs << 24) |
+         ((uint64_t)any_bfgs << 25) | ((uint64_t)automatic.queue << 26) | ((uint64_t)automatic.variant << 27) |
+         ((uint64_t)automatic.team << 28) | ((uint64_t)sms << 32);
 }
 
 static bool tune_lookup(uint64_t key, int* variant, int* persistent, int* warps) {
@@ -201,6 +215,15 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
   g_tune.push_back(TuneEntry{key, variant, persistent, warps});
 }
 
+static void tune_erase(uint64_t key) {
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  for (size_t i = 0; i < g_tune.size(); ++i)
+    if (g_tune[i].key == key) {
+      g_tune.erase(g_tune.begin() + i);
+      return;
+    }
+}
+
 // Slices of the launch's longest chains when it time-slices (ChainQueue): enough
 // that the last slices are a small part of the launch, few enough that a slice
 // (a few MC steps, hundreds of evaluations) hides its record's load and store.  When
@@ -208,7 +231,6 @@ static void tune_store(uint64_t key, int variant, int persistent, int warps) {
 // slowest reach the teams: slices of one MC step (1,536 chains as above: 11.6 ms, in
 // 16 slices 12.8).
 constexpr int kSliceRounds = 16, kSliceRoundsResident = 64;
-
 
 static ChainQueueMode queue_mode(const dsdp_plan* P) {
   return (P->flags & DSDP_PLAN_PERSISTENT) ? kQueue : P->auto_queue ? kQueueIfMany : kNoQueue;
@@ -460,25 +482,29 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
       fmt_mask |= 1u << g.fmt;
       apl_max = std::max(apl_max, g.apl);
     }
-    P->tune_key = tune_key(fmt_mask, apl_max, total_chains);
-    int var = 0, pers = (flags & DSDP_PLAN_PERSISTENT) ? 1 : 0;
+    // By the number of chains.  Up to 8 per SM: teams, or (Barzilai-Borwein has no line
+    // search) one warp per chain, ligands above 32 atoms, whose staged blobs are large, in
+    // tiles of 4 chains.  More: the time-sliced queue, one chain per CTA (16 typical-4k
+    // systems 29.6 ms, in tiles of 2 and 4 31.0 and 33).  From two waves of 16 per SM on
+    // the 96-register kernel, whose 20 resident warps per SM issue more per cycle, below
+    // the 128-register kernel, whose fewer instructions per evaluation win on a
+    // part-filled GPU.
+    const size_t wave = (size_t)16 * P->sms;
+    const bool many = total_chains > wave / 2;
+    dsdp_plan::Arrangement& A = P->automatic;
+    A.variant = total_chains >= 2 * wave ? 1 : 0;
+    A.queue = many;
+    A.team = all_bfgs && !(flags & kPlanShared) ? team_warps(total_chains, P->sms) : 1;
+    A.warps = apl_max == 2 && !many && A.team == 1 ? 4 : 1;
+    P->tune_key = tune_key(fmt_mask, apl_max, total_chains, all_bfgs, any_bfgs, A, P->sms);
+    int var = A.variant, pers = (flags & DSDP_PLAN_PERSISTENT) ? 1 : 0;
     if (tile_config == 0) {
-      // Without a recorded choice, by the number of chains.  Up to 8 per SM: teams, or
-      // (Barzilai-Borwein has no line search) one warp per chain, ligands above 32
-      // atoms, whose staged blobs are large, in tiles of 4 chains.  More: the
-      // time-sliced queue, one chain per CTA (16 typical-4k systems 29.6 ms, in tiles
-      // of 2 and 4 31.0 and 33).  From two waves of 16 per SM on the 96-register kernel,
-      // whose 20 resident warps per SM issue more per cycle, below the 128-register
-      // kernel, whose fewer instructions per evaluation win on a part-filled GPU.
-      const size_t wave = (size_t)16 * P->sms;
-      var = total_chains >= 2 * wave ? 1 : 0;
-      const bool many = total_chains > wave / 2;
       W = apl_max == 2 && !many ? 4 : 1;
       if (tune_lookup(P->tune_key, &var, &pers, &W)) {
         if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
       } else {
-        P->auto_queue = many;
-        P->team = all_bfgs && !pers && !(flags & kPlanShared) ? team_warps(total_chains, P->sms) : 1;
+        P->auto_queue = A.queue;
+        P->team = pers ? 1 : A.team;
         if (P->team > 1) W = 1;
       }
     } else {
@@ -616,15 +642,22 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
     for (int i = 0; i < 24; ++i) ms_by_config[i] = -1.f;
   if (repeats < 1) repeats = 1;
   const cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e = cudaStreamSynchronize(st);  // a launch before may still read the tiles
+  if (e != cudaSuccess) return check_cuda(e, "autotune");
   cudaEvent_t a, b;
-  cudaError_t e = cudaEventCreate(&a);
+  e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e != cudaSuccess) return check_cuda(e, "autotune events");
   const uint32_t base_flags = P->flags & ~(uint32_t)DSDP_PLAN_PERSISTENT;
   // the automatic arrangement (queue when needed, teams) first: kept if nothing beats it
-  const bool auto_queue = P->auto_queue;
-  const int team = P->team, auto_var = P->variant, auto_w = P->warps_per_cta;
-  const uint32_t auto_flags = P->flags;
+  const dsdp_plan::Arrangement& A = P->automatic;
+  auto use_automatic = [&] {
+    P->flags = base_flags;
+    P->variant = A.variant;
+    P->auto_queue = A.queue;
+    P->team = A.team;
+    return plan_use_warps(P, A.warps);
+  };
   float auto_ms = 1e30f;
   float best = 1e30f;
   int best_var = P->variant, best_pers = (P->flags & DSDP_PLAN_PERSISTENT) ? 1 : 0, best_w = P->warps_per_cta;
@@ -640,7 +673,10 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
     cudaEventElapsedTime(ms, a, b);
     return r;
   };
-  if (auto_queue || team > 1) s = measure(&auto_ms);
+  if (A.queue || A.team > 1) {  // else it is one of the fixed ones
+    s = check_cuda(use_automatic(), "autotune tiles");
+    if (s == DSDP_OK) s = measure(&auto_ms);
+  }
   P->auto_queue = false;  // with and without the queue are measured apart
   P->team = 1;
   for (int c = 0; c < 6 && s == DSDP_OK; ++c) {
@@ -673,11 +709,8 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   cudaEventDestroy(b);
   if (chosen) *chosen = 1 + best_var + 4 * (best_w == 4 ? 2 : best_w - 1) + 12 * best_pers;
   if (s == DSDP_OK && auto_ms <= best) {  // later plans of this shape find it by themselves
-    P->variant = auto_var;
-    P->flags = auto_flags;
-    P->auto_queue = auto_queue;
-    P->team = team;
-    return check_cuda(plan_use_warps(P, auto_w), "plan tiles");
+    tune_erase(P->tune_key);
+    return check_cuda(use_automatic(), "plan tiles");
   }
   P->variant = best_var;
   P->flags = base_flags | (best_pers ? DSDP_PLAN_PERSISTENT : 0u);
