@@ -84,7 +84,7 @@ def parse():
     p.add_argument("--e2e-window", type=int, default=3,
                    help="steps in flight through the host API (the end-to-end pass; 1 with --no-pipeline)")
     p.add_argument("--tile-config", type=int, default=-1,
-                   help="chain kernel launch configuration: -1 autotune (default); 1..24 fixed, numbered as the "
+                   help="chain kernel launch configuration: -1 autotune (default); 0 automatic; 1..24 fixed, numbered as the "
                         "autotuner reports them: 1 + variant (0: 128 registers, 1: 96, 2: 80, 3: 72) + 4 log2(chains "
                         "per CTA) + 12 work queue")
     args = p.parse_args()
@@ -139,8 +139,9 @@ def systems(rank, batch):
 
 
 def plan_tile_config(chosen):
-    """dsdp_plan_create's tile_config (1 + variant + 4 log2 W) of an autotuner choice."""
-    return 1 + (chosen - 1) % 12
+    """dsdp_plan_create's tile_config (1 + variant + 4 log2 W) of an autotuner choice, 0 of the
+    automatic arrangement."""
+    return 1 + (chosen - 1) % 12 if chosen else 0
 
 
 def plan_flags(dsdp, chosen):
@@ -149,7 +150,10 @@ def plan_flags(dsdp, chosen):
 
 
 def describe_tile_config(chosen):
-    """The autotuner's choice (1 + variant + 4 log2 W + 12 persistent) in words."""
+    """The autotuner's choice (1 + variant + 4 log2 W + 12 persistent, 0 the automatic arrangement)
+    in words."""
+    if chosen == 0:
+        return "automatic (by the plan's size)"
     if not 1 <= chosen <= 24:
         return "?"
     c = chosen - 1
@@ -437,7 +441,8 @@ def run_device(args, rank, world, dev, dist):
     build_grids(slots[0], sptr)
     autotune_ms = None
     if args.tile_config < 0:  # register budget, chains per CTA, work queue
-        tile_config, autotune_ms = dsdp.dsdp_plan_autotune(plan, sptr, 2, with_times=True)
+        _, autotune_ms = dsdp.dsdp_plan_autotune(plan, sptr, 2, with_times=True)
+        tile_config = dsdp.dsdp_plan_config(plan)  # what the plan keeps
     else:
         dsdp.dsdp_plan_destroy(None, plan)
         plan = dsdp.dsdp_plan_create(None, slots[0]["jobs"], plan_flags(dsdp, args.tile_config),
@@ -698,7 +703,8 @@ def run_uneven_graph(args, dev, steps=3):
         keeps.append(keep)
     build_grid(dsdp, grid, dsdp.DSDP_MAP_F32, sptr)
     plan = dsdp.dsdp_plan_create(None, jobs, 0, 0)
-    chosen, tune_ms = dsdp.dsdp_plan_autotune(plan, sptr, 2, with_times=True)
+    _, tune_ms = dsdp.dsdp_plan_autotune(plan, sptr, 2, with_times=True)
+    chosen = dsdp.dsdp_plan_config(plan)
     cap = torch.cuda.Stream()
     graph = torch.cuda.CUDAGraph()
     torch.cuda.synchronize()
@@ -734,7 +740,8 @@ def _timed_plan(dsdp, torch, items, dtype, sptr, steps, optimizer=0, tuned=None)
         for _, keep in items:
             build_grid(dsdp, keep["grid"], dtype, sptr)
         if tuned is not None:
-            tuned["chain_kernel"] = describe_tile_config(dsdp.dsdp_plan_autotune(plan, sptr, 1))
+            dsdp.dsdp_plan_autotune(plan, sptr, 1)
+            tuned["chain_kernel"] = describe_tile_config(dsdp.dsdp_plan_config(plan))
         dsdp.dsdp_plan_launch(plan, sptr)
         torch.cuda.synchronize()
         a, b = torch.cuda.Event(True), torch.cuda.Event(True)
@@ -904,7 +911,8 @@ def run_configs(args, rank, dev, steps=2):
         try:
             for _, keep in items:
                 build_grid(dsdp, keep["grid"], dsdp.DSDP_MAP_F32, sptr)
-            chosen = dsdp.dsdp_plan_autotune(plan, sptr, 1)
+            dsdp.dsdp_plan_autotune(plan, sptr, 1)
+            chosen = dsdp.dsdp_plan_config(plan)
             torch.cuda.synchronize()
             a, b = torch.cuda.Event(True), torch.cuda.Event(True)
             a.record()

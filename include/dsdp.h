@@ -390,12 +390,18 @@ dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsdp_job_devic
  * chains per CTA, with and without the
  * persistent work queue, keeps the fastest for this plan and records it for
  * later plans of the same shape (process-wide); the automatic arrangement is
- * measured first and stays where no fixed one beats it.  *chosen = 1 + variant
+ * measured first and stays where no fixed one beats it (dsdp_plan_config).
+ * *chosen = the fastest fixed configuration, 1 + variant
  * + 4 * log2(W) + 12 * persistent (1 .. 24; the first part is the plan's
  * tile_config).  ms_by_config: NULL, or 24 floats receiving the measured chain
  * stage time (ms per launch) of configuration chosen - 1, -1 where a
  * configuration was not run.  Synchronises the stream. */
 dsdp_status dsdp_plan_autotune(dsdp_plan* plan, void* stream, int32_t repeats, int32_t* chosen, float* ms_by_config);
+/* What the plan runs: 0 = the automatic arrangement, else the fixed configuration
+ * c = 1 .. 24 as dsdp_plan_autotune numbers them.  A plan of the same jobs made with
+ * tile_config 0 for 0, else 1 + (c - 1) % 12 and DSDP_PLAN_PERSISTENT for c > 12, runs
+ * the same. */
+int32_t dsdp_plan_config(const dsdp_plan* plan);
 /* Enqueue the plan's kernels on `stream` (chains, then FP64 rescoring and
  * top-k).  No allocation and no host synchronisation: a launch can be
  * captured into a CUDA graph and replayed.  Different plans may run at once

@@ -574,6 +574,15 @@ extern "C" int32_t dsdp_plan_kernel_count(const dsdp_plan* P) {
   return n;
 }
 
+static int config_number(int variant, int warps, bool persistent) {
+  return 1 + variant + 4 * (warps == 4 ? 2 : warps - 1) + (persistent ? 12 : 0);
+}
+
+extern "C" int32_t dsdp_plan_config(const dsdp_plan* P) {
+  if (!P || P->auto_queue || P->team > 1) return 0;
+  return config_number(P->variant, P->warps_per_cta, P->flags & DSDP_PLAN_PERSISTENT);
+}
+
 extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, void* stream) {
   if (!P) return set_error(DSDP_ERR_INVALID_ARG, "plan is NULL");
   if (stages == 0 || (stages & ~(uint32_t)DSDP_STAGE_ALL)) return set_error(DSDP_ERR_INVALID_ARG, "bad stages");
@@ -696,7 +705,7 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
       float ms = 0.f;
       s = measure(&ms);
       if (s != DSDP_OK) break;
-      if (ms_by_config) ms_by_config[var + 4 * (w == 4 ? 2 : w - 1) + 12 * pers] = ms / repeats;
+      if (ms_by_config) ms_by_config[config_number(var, w, pers) - 1] = ms / repeats;
       if (ms < best) {
         best = ms;
         best_var = var;
@@ -707,7 +716,7 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  if (chosen) *chosen = 1 + best_var + 4 * (best_w == 4 ? 2 : best_w - 1) + 12 * best_pers;
+  if (chosen) *chosen = config_number(best_var, best_w, best_pers);
   if (s == DSDP_OK && auto_ms <= best) {  // later plans of this shape find it by themselves
     tune_erase(P->tune_key);
     return check_cuda(use_automatic(), "plan tiles");

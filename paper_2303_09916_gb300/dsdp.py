@@ -137,6 +137,7 @@ _sig = {
     "dsdp_plan_launch": (C.c_int32, [C.c_void_p, C.c_void_p]),
     "dsdp_plan_launch_stage": (C.c_int32, [C.c_void_p, C.c_uint32, C.c_void_p]),
     "dsdp_plan_kernel_count": (C.c_int32, [C.c_void_p]),
+    "dsdp_plan_config": (C.c_int32, [C.c_void_p]),
     "dsdp_plan_autotune": (C.c_int32, [C.c_void_p, C.c_void_p, C.c_int32, P(C.c_int32), P(C.c_float)]),
     "dsdp_plan_destroy": (C.c_int32, [C.c_void_p, C.c_void_p]),
     "dsdp_gather_bench_device": (C.c_int32, [P(dsdp_grid_view), C.c_void_p, C.c_void_p, C.c_int32, C.c_int32,
@@ -417,8 +418,8 @@ def dsdp_plan_create(ctx, jobs, flags=0, tile_config=0):
 
 
 def dsdp_plan_autotune(plan, stream: int = 0, repeats: int = 1, with_times: bool = False):
-    """The chosen configuration (1 + variant + 4 log2 W + 12 persistent); with
-    with_times also {configuration: ms per chain launch} of every one measured."""
+    """The fastest fixed configuration (1 + variant + 4 log2 W + 12 persistent; what the
+    plan keeps: dsdp_plan_config); with with_times also {configuration: ms per chain launch} of every one measured."""
     chosen = C.c_int32()
     ms = (C.c_float * 24)()
     _check(_lib.dsdp_plan_autotune(plan, stream or None, int(repeats), C.byref(chosen), ms))
@@ -437,6 +438,11 @@ def dsdp_plan_launch_stage(plan, stages, stream: int = 0):
 
 def dsdp_plan_kernel_count(plan) -> int:
     return int(_lib.dsdp_plan_kernel_count(plan))
+
+
+def dsdp_plan_config(plan) -> int:
+    """What the plan runs: 0 the automatic arrangement, 1..24 a fixed configuration."""
+    return int(_lib.dsdp_plan_config(plan))
 
 
 def dsdp_plan_destroy(ctx, plan):

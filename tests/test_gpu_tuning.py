@@ -82,3 +82,27 @@ def test_tuning_measures_the_automatic_arrangement_of_every_plan(jobs):
         plan = _create(make(chains, dsdp.DSDP_OPT_BFGS))
         assert captured_kernels(stream, lambda: dsdp.dsdp_plan_launch(plan, stream)) == [(chains, 4 * 32)]
         dsdp.dsdp_plan_destroy(None, plan)
+
+
+@pytest.mark.parametrize("chains_per_sm,optimizer", [(0.5, 0), (2, 0), (12, 0), (2, 1), (12, 1), (40, 0)])
+def test_a_plan_made_from_the_kept_configuration_runs_what_the_tuned_plan_runs(jobs, chains_per_sm, optimizer):
+    make, stream, _ = jobs
+    chains = int(chains_per_sm * torch.cuda.get_device_properties(0).multi_processor_count)
+    spec = make(chains, optimizer, steps=6)
+    plan = _create(spec)
+    kept = dsdp.dsdp_plan_config(plan)  # before: the automatic arrangement, or the fixed one that it is
+    runs = captured_kernels(stream, lambda: dsdp.dsdp_plan_launch(plan, stream))
+    again = _create(spec, 1 + (kept - 1) % 12 if kept else 0)
+    assert captured_kernels(stream, lambda: dsdp.dsdp_plan_launch(again, stream)) == runs
+    dsdp.dsdp_plan_destroy(None, again)
+    chosen, ms = dsdp.dsdp_plan_autotune(plan, stream, 2, with_times=True)
+    kept = dsdp.dsdp_plan_config(plan)
+    assert kept in (0, chosen) and ms[chosen] == min(ms.values())
+    again = dsdp.dsdp_plan_create(None, spec, dsdp.DSDP_PLAN_NO_RESCORE | (dsdp.DSDP_PLAN_PERSISTENT if kept > 12 else 0),
+                                  1 + (kept - 1) % 12 if kept else 0)
+    assert dsdp.dsdp_plan_config(again) == kept
+    assert dsdp.dsdp_plan_kernel_count(again) == dsdp.dsdp_plan_kernel_count(plan)
+    runs = [captured_kernels(stream, lambda: dsdp.dsdp_plan_launch(p, stream)) for p in (plan, again)]
+    assert runs[0] == runs[1] and len(runs[0]) == dsdp.dsdp_plan_kernel_count(plan)
+    for p in (plan, again):
+        dsdp.dsdp_plan_destroy(None, p)
