@@ -371,7 +371,10 @@ enum {
  * rounded up to a power of two and on the same side of the limits below, SM
  * count), else by the plan's size.  Up to 8 chains per SM, all of them
  * BFGS: teams of 4 warps per chain (8 up to one chain per SM), which evaluate a
- * line search's trial points at once.  Above: the work queue in slices, longest
+ * line search's trial points at once -- one warp per chain while other plans'
+ * chains are under way on other streams and all together are more than 16 per SM
+ * (18 with ligands above 32 atoms; a launch under stream capture goes by its own
+ * chains).  Above: the work queue in slices, longest
  * chains first, W = 1, the 96-register kernel from 32 x (SM count) chains on and
  * the 128-register kernel below that or where shared memory allows no more than
  * 16 warps per SM.  1 .. 12 = a fixed choice 1 + variant +
@@ -402,6 +405,8 @@ dsdp_status dsdp_plan_autotune(dsdp_plan* plan, void* stream, int32_t repeats, i
  * tile_config 0 for 0, else 1 + (c - 1) % 12 and DSDP_PLAN_PERSISTENT for c > 12, runs
  * the same. */
 int32_t dsdp_plan_config(const dsdp_plan* plan);
+/* Warps that ran each chain together in the plan's last launch (1, 4 or 8; 0 before it). */
+int32_t dsdp_plan_team(const dsdp_plan* plan);
 /* Enqueue the plan's kernels on `stream` (chains, then FP64 rescoring and
  * top-k).  No allocation and no host synchronisation: a launch can be
  * captured into a CUDA graph and replayed.  Different plans may run at once

@@ -332,8 +332,8 @@ Batch* batch_launch(dsdp_ctx* ctx, const std::vector<Job*>& jobs, int stream) {
   Batch* b = new Batch();
   b->jobs = jobs;
   b->stream = stream;
-  dsdp_status s = dsdp_plan_create(ctx, (int32_t)jd.size(), jd.data(), ctx->batches.empty() && ctx->queue.empty() ? 0u : kPlanShared, 0,
-                                   &b->plan);
+  const bool alone = ctx->batches.empty() && ctx->queue.empty();
+  dsdp_status s = plan_create(ctx, (int)jd.size(), jd.data(), 0, 0, alone, &b->plan);
   for (size_t i = 0; s == DSDP_OK && i < jobs.size(); ++i)  // the maps may still be in the making
     if (jobs[i]->grid->ready) s = check_cuda(cudaStreamWaitEvent(st, jobs[i]->grid->ready, 0), "grid wait");
   if (s == DSDP_OK) {

@@ -128,8 +128,10 @@ struct DevJob {
 // use while the chains run.
 constexpr int slice_record_bytes(int n_torsions) { return 8 * (7 + n_torsions) + 16; }
 
-// Internal plan flag: other launches share the GPU with this plan's (no teams).
-constexpr uint32_t kPlanShared = 1u << 30;
+// dsdp_plan_create; alone: no other launches share the GPU with this plan's for certain
+// (else its chains run without teams).
+dsdp_status plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* jobs, uint32_t flags, int tile_config,
+                        bool alone, dsdp_plan** out);
 
 struct Tile {
   int32_t job;

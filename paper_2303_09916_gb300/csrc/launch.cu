@@ -26,10 +26,12 @@ struct dsdp_plan {
   struct Group {
     int fmt, apl, first_tile, n_tiles, blob_smem, max_atoms, max_torsions, apl_mask;
     int first_block, n_blocks, n_items;  // time-sliced queue (SliceBlock)
+    int first_chain, n_chains;           // tiles of one chain each (teams)
   };
   std::vector<Group> groups;
   void* d_jobs = nullptr;
   void* d_tiles = nullptr;
+  void* d_singles = nullptr;  // room for the same chains in tiles of one; null if teams are never taken
   void* d_rtiles = nullptr;
   // work queue: [kMaxGroups counters, one per group][kMaxGroups exit counts][tickets per tile][next step per tile and warp]; zeroed by each launch
   int* d_queue = nullptr;
@@ -45,8 +47,10 @@ struct dsdp_plan {
   Arrangement automatic{0, 1, 1, false};  // by the plan's size, whatever it runs now
   bool auto_queue = false;    // as it runs now (variant, warps_per_cta): the queue, teams
   int team = 1;
+  int last_team = 0;          // of the last launch (chains in flight elsewhere may take its teams)
   bool any_bfgs = false;
   bool resident = false;      // 16 chains per SM or fewer
+  int apl_max = 1;            // atoms per lane of the largest ligand
   void* d_blocks = nullptr;
   int n_rtiles = 0;
   // per job, to lay groups and tiles out again for another configuration
@@ -58,6 +62,13 @@ struct dsdp_plan {
   std::vector<Shape> shape;
   std::vector<int> job_order;  // jobs by chain length, longest first
   int sms = 148;
+  // The plan's last chain launch, among those of the process's other plans (ChainsInFlight).
+  struct Flight {
+    cudaEvent_t done = nullptr;  // null: not tracked
+    int device = 0, chains = 0;
+    cudaStream_t stream = nullptr;
+    bool busy = false;  // launched and not seen to have ended
+  } flight;
 };
 
 namespace dsdp {
@@ -248,6 +259,7 @@ static ChainQueueMode queue_mode(const dsdp_plan* P) {
 static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vector<SliceBlock>& blocks) {
   tiles.clear();
   blocks.clear();
+  int n_chains = 0;
   P->groups.clear();
   const bool split = queue_mode(P) != kNoQueue;
   struct Item {
@@ -275,6 +287,9 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
         for (int r = 0; r < s.slices; ++r) items.push_back(Item{s.cost * (s.slices - r) / s.slices, first, n});
       }
       g.n_tiles = (int)tiles.size() - g.first_tile;
+      g.first_chain = n_chains;
+      for (int t = g.first_tile; t < (int)tiles.size(); ++t) g.n_chains += tiles[t].count;
+      n_chains += g.n_chains;
       if (!g.n_tiles) continue;
       std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.left > b.left; });
       g.first_block = (int)blocks.size();
@@ -298,13 +313,95 @@ constexpr int kTailTeams = 8;
 // idle; 1 when they do not.  Up to one chain per SM a team of 8 (64 plain-2k chains
 // 6.3 ms against 6.7 in teams of 4; 200 typical-4k chains 2.8 against 2.6), up to 8
 // per SM teams of 4 (1,200 chains 6.9 ms, one warp each 8.1; 1,536 chains 9.7 against
-// 8.3; four such launches of 384 chains at once 7.3 against 9.3, eight 13.5 against
-// 11.9 -- the job queue, which knows, does without teams then): beyond, the trial points that a line search does not come to cost more than
+// 8.3): beyond, the trial points that a line search does not come to cost more than
 // the shorter way saves.  Teams are a warp per SM sub-partition or two: 5 and 6 warps
 // measured slower than 4.
 static int team_warps(size_t chains, int sms) {
   if (chains <= (size_t)sms) return kMaxTeam;
   return chains <= (size_t)(8 * sms) ? 4 : 1;
+}
+
+// Chain launches on their way.  Which way is the fastest for a plan of few chains
+// depends on all the chains that run at the same time, so each plan marks the end of
+// its last chain launch with an event, and a plan that could take teams counts what
+// other streams have under way on its device.  The count only chooses between ways that
+// give the same bits.  A launch under stream capture neither counts nor is counted: when
+// and beside what it will run is not known.
+static std::mutex g_flight_mu;
+static std::vector<dsdp_plan::Flight*> g_flights;
+
+static void track_flight(dsdp_plan::Flight* f, int chains) {
+  f->chains = chains;
+  if (cudaGetDevice(&f->device) != cudaSuccess ||
+      cudaEventCreateWithFlags(&f->done, cudaEventDisableTiming) != cudaSuccess) {
+    f->done = nullptr;
+    cudaGetLastError();
+    return;
+  }
+  std::lock_guard<std::mutex> lk(g_flight_mu);
+  g_flights.push_back(f);
+}
+
+static void untrack_flight(dsdp_plan::Flight* f) {
+  if (!f->done) return;
+  {
+    std::lock_guard<std::mutex> lk(g_flight_mu);
+    g_flights.erase(std::remove(g_flights.begin(), g_flights.end(), f), g_flights.end());
+  }
+  cudaEventDestroy(f->done);
+}
+
+static void mark_flight(dsdp_plan::Flight* f, cudaStream_t st) {
+  if (!f->done) return;
+  std::lock_guard<std::mutex> lk(g_flight_mu);
+  f->stream = st;
+  f->busy = cudaEventRecord(f->done, st) == cudaSuccess;
+  if (!f->busy) cudaGetLastError();
+}
+
+// Chains that other streams of the plan's device have under way: of each stream its
+// largest launch (a stream's launches run one after the other), of the streams the
+// seven largest (beside its own, a device runs eight unless the environment says more).
+static size_t chains_in_flight(const dsdp_plan::Flight& own, cudaStream_t st) {
+  constexpr int kStreams = 7;
+  cudaStream_t stream[kStreams];
+  int chains[kStreams], n = 0;
+  // another thread's capture must not be ended by a query of this one
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  {
+    std::lock_guard<std::mutex> lk(g_flight_mu);
+    for (dsdp_plan::Flight* f : g_flights) {
+      if (!f->busy || f == &own || f->device != own.device || f->stream == st) continue;
+      if (cudaEventQuery(f->done) != cudaErrorNotReady) {
+        f->busy = false;
+        continue;
+      }
+      int k = 0;
+      while (k < n && stream[k] != f->stream) ++k;
+      if (k == n && n < kStreams) chains[n++] = 0;
+      if (k == kStreams) k = (int)(std::min_element(chains, chains + n) - chains);
+      if (f->chains > chains[k]) chains[k] = f->chains, stream[k] = f->stream;
+    }
+  }
+  if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();  // no error
+  if (swapped) cudaThreadExchangeStreamCaptureMode(&mode);
+  size_t sum = 0;
+  for (int k = 0; k < n; ++k) sum += chains[k];
+  return sum;
+}
+
+// Warps of a chain of a plan of `chains`, with `others` under way beside them (round of
+// launches of 10 steps, typical-4k, ms with one warp a chain / teams of 4 / of 8): streams
+// x chains 2 x 128 3.7 / 1.94 / 1.80, 4 x 128 4.4 / 2.5 / 2.9, 8 x 128 4.7 / 3.2 / 5.3;
+// 4 x 384 5.1 / 4.1 / 7.9, 5 x 5.0 / 4.8, 6 x 5.7 / 5.7, 7 x 5.6 / 6.8, 8 x 6.5 / 7.5.
+// Two atoms per lane (45): 4 x 128 9.3 / 4.3 / 4.1, 8 x 128 10.1 / 5.4 / 7.7; 8 x 384 10.7
+// in tiles of 4 chains / 12.4.  (One launch alone loses its teams' gain earlier,
+// team_warps: its chains keep step.)
+static int shared_team_warps(size_t chains, size_t others, int apl_max, int sms) {
+  const size_t all = chains + others;
+  if (chains <= (size_t)sms && all <= (size_t)((apl_max == 2 ? 4 : 2) * sms)) return kMaxTeam;
+  return all <= (size_t)((apl_max == 2 ? 18 : 16) * sms) ? 4 : 1;
 }
 
 static cudaError_t plan_use_warps(dsdp_plan* P, int W) {
@@ -317,6 +414,12 @@ static cudaError_t plan_use_warps(dsdp_plan* P, int W) {
     e = cudaMemcpy(P->d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !blocks.empty())
     e = cudaMemcpy(P->d_blocks, blocks.data(), sizeof(SliceBlock) * blocks.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && P->d_singles) {
+    std::vector<Tile> singles;
+    for (const Tile& t : tiles)
+      for (int c = 0; c < t.count; ++c) singles.push_back(Tile{t.job, t.chain0 + c, 1, 0});
+    e = cudaMemcpy(P->d_singles, singles.data(), sizeof(Tile) * singles.size(), cudaMemcpyHostToDevice);
+  }
   return e;
 }
 
@@ -354,6 +457,11 @@ extern "C" dsdp_status dsdp_score_eval_device(const dsdp_grid_view* grid, const 
 
 extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsdp_job_device* jobs, uint32_t flags,
                                         int32_t tile_config, dsdp_plan** out) {
+  return plan_create(ctx, n_jobs, jobs, flags, tile_config, true, out);
+}
+
+dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* jobs, uint32_t flags, int tile_config,
+                              bool alone, dsdp_plan** out) {
   if (!out) return set_error(DSDP_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   if (n_jobs < 1 || !jobs) return set_error(DSDP_ERR_INVALID_ARG, "plan needs >= 1 job");
@@ -435,7 +543,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   dsdp_plan* P = new dsdp_plan();
   P->ctx = ctx;
   P->n_jobs = n_jobs;
-  P->flags = flags & ~kPlanShared;
+  P->flags = flags;
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
   size_t total_chains = 0, max_blocks = 0;
@@ -489,23 +597,23 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     // the 96-register kernel, whose 20 resident warps per SM issue more per cycle, below
     // the 128-register kernel, whose fewer instructions per evaluation win on a
     // part-filled GPU.
+    P->apl_max = apl_max;
     const size_t wave = (size_t)16 * P->sms;
     const bool many = total_chains > wave / 2;
     dsdp_plan::Arrangement& A = P->automatic;
     A.variant = total_chains >= 2 * wave ? 1 : 0;
     A.queue = many;
-    A.team = all_bfgs && !(flags & kPlanShared) ? team_warps(total_chains, P->sms) : 1;
-    A.warps = apl_max == 2 && !many && A.team == 1 ? 4 : 1;
+    A.team = all_bfgs && alone ? team_warps(total_chains, P->sms) : 1;
+    A.warps = apl_max == 2 && !many ? 4 : 1;
     P->tune_key = tune_key(fmt_mask, apl_max, total_chains, all_bfgs, any_bfgs, A, P->sms);
     int var = A.variant, pers = (flags & DSDP_PLAN_PERSISTENT) ? 1 : 0;
     if (tile_config == 0) {
-      W = apl_max == 2 && !many ? 4 : 1;
+      W = A.warps;
       if (tune_lookup(P->tune_key, &var, &pers, &W)) {
         if (pers) P->flags |= DSDP_PLAN_PERSISTENT;
       } else {
         P->auto_queue = A.queue;
         P->team = pers ? 1 : A.team;
-        if (P->team > 1) W = 1;
       }
     } else {
       var = (tile_config - 1) % 4;
@@ -518,7 +626,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   for (int j = 0; j < n_jobs; ++j)
     for (int c = 0; c < dj[j].n_chains; c += rw) rtiles.push_back(Tile{j, c, std::min(rw, dj[j].n_chains - c), 0});
   P->n_rtiles = (int)rtiles.size();
-  const size_t b_jobs = up256(sizeof(DevJob) * n_jobs), b_tiles = up256(sizeof(Tile) * total_chains),
+  const size_t b_jobs = up256(sizeof(DevJob) * n_jobs), b_tiles = up256(sizeof(Tile) * total_chains) * (P->automatic.team > 1 ? 2 : 1),
                b_rtiles = up256(sizeof(Tile) * rtiles.size()), b_blocks = up256(sizeof(SliceBlock) * max_blocks);
   P->queue_next_off = 2 * kMaxGroups + total_chains;
   P->queue_bytes = sizeof(int) * (2 * kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);  // tiles of W <= 4 may be part filled
@@ -533,6 +641,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
   uint8_t* a = (uint8_t*)P->arena;
   P->d_jobs = a;
   P->d_tiles = a + b_jobs;
+  if (P->automatic.team > 1) P->d_singles = a + b_jobs + b_tiles / 2;
   P->d_rtiles = a + b_jobs + b_tiles;
   P->d_blocks = a + b_jobs + b_tiles + b_rtiles;
   P->d_queue = (int*)(a + b_jobs + b_tiles + b_rtiles + b_blocks);
@@ -562,6 +671,7 @@ extern "C" dsdp_status dsdp_plan_create(dsdp_ctx* ctx, int32_t n_jobs, const dsd
     delete P;
     return check_cuda(e, "plan upload");
   }
+  track_flight(&P->flight, (int)total_chains);
   *out = P;
   return DSDP_OK;
 }
@@ -573,6 +683,8 @@ extern "C" int32_t dsdp_plan_kernel_count(const dsdp_plan* P) {
   if (!(P->flags & DSDP_PLAN_NO_RESCORE)) n += 2;
   return n;
 }
+
+extern "C" int32_t dsdp_plan_team(const dsdp_plan* P) { return P ? P->last_team : 0; }
 
 static int config_number(int variant, int warps, bool persistent) {
   return 1 + variant + 4 * (warps == 4 ? 2 : warps - 1) + (persistent ? 12 : 0);
@@ -588,6 +700,17 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
   if (stages == 0 || (stages & ~(uint32_t)DSDP_STAGE_ALL)) return set_error(DSDP_ERR_INVALID_ARG, "bad stages");
   const cudaStream_t st = (cudaStream_t)stream;
   const ChainQueueMode queue = queue_mode(P);
+  int team = P->team;
+  bool track = false;
+  if (stages & DSDP_STAGE_CHAINS) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(st, &capture);
+    if (e != cudaSuccess) cudaGetLastError();
+    track = e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+    if (team > 1 && track && P->flight.done)
+      team = shared_team_warps((size_t)P->flight.chains, chains_in_flight(P->flight, st), P->apl_max, P->sms);
+    P->last_team = team;
+  }
   if ((stages & DSDP_STAGE_CHAINS) && queue != kNoQueue) {
     const cudaError_t e = cudaMemsetAsync(P->d_queue, 0, P->queue_bytes, st);
     if (e != cudaSuccess) return check_cuda(e, "plan queue reset");
@@ -619,7 +742,11 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     if (P->auto_queue && a.variant == 1 &&
         kSmemPerSm / (a.blob_smem + a.warps_per_cta * a.scratch.bytes + 1024) * a.warps_per_cta <= 16)
       a.variant = 0;
-    a.team = P->team;
+    a.team = team;
+    if (team > 1) {
+      a.tiles = (const Tile*)P->d_singles + g.first_chain;
+      a.n_tiles = g.n_chains;
+    }
     a.team_resumes = false;
     a.team_when = P->auto_queue && P->any_bfgs && (P->resident || P->groups.size() == 1) ? kTailTeams * P->sms : 0;
     cudaError_t e = launch_chains_dispatch(g.fmt, a, st);
@@ -631,6 +758,7 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
       if (e != cudaSuccess) return check_cuda(e, "dock_team_kernel launch");
     }
   }
+  if (track) mark_flight(&P->flight, st);
   if ((stages & DSDP_STAGE_RESCORE) && !(P->flags & DSDP_PLAN_NO_RESCORE)) {
     cudaError_t e = launch_rescore(P->d_jobs, P->d_rtiles, P->n_rtiles, st);
     if (e != cudaSuccess) return check_cuda(e, "rescore_kernel launch");
@@ -731,6 +859,7 @@ extern "C" dsdp_status dsdp_plan_autotune(dsdp_plan* P, void* stream, int32_t re
 
 extern "C" dsdp_status dsdp_plan_destroy(dsdp_ctx* ctx, dsdp_plan* P) {
   if (!P) return DSDP_OK;
+  untrack_flight(&P->flight);
   if (P->arena) ctx_free(ctx ? ctx : P->ctx, P->arena, P->arena_bytes, nullptr);
   delete P;
   return DSDP_OK;

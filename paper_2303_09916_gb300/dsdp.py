@@ -138,6 +138,7 @@ _sig = {
     "dsdp_plan_launch_stage": (C.c_int32, [C.c_void_p, C.c_uint32, C.c_void_p]),
     "dsdp_plan_kernel_count": (C.c_int32, [C.c_void_p]),
     "dsdp_plan_config": (C.c_int32, [C.c_void_p]),
+    "dsdp_plan_team": (C.c_int32, [C.c_void_p]),
     "dsdp_plan_autotune": (C.c_int32, [C.c_void_p, C.c_void_p, C.c_int32, P(C.c_int32), P(C.c_float)]),
     "dsdp_plan_destroy": (C.c_int32, [C.c_void_p, C.c_void_p]),
     "dsdp_gather_bench_device": (C.c_int32, [P(dsdp_grid_view), C.c_void_p, C.c_void_p, C.c_int32, C.c_int32,
@@ -443,6 +444,11 @@ def dsdp_plan_kernel_count(plan) -> int:
 def dsdp_plan_config(plan) -> int:
     """What the plan runs: 0 the automatic arrangement, 1..24 a fixed configuration."""
     return int(_lib.dsdp_plan_config(plan))
+
+
+def dsdp_plan_team(plan) -> int:
+    """Warps that ran each chain together in the plan's last launch (0 before it)."""
+    return int(_lib.dsdp_plan_team(plan))
 
 
 def dsdp_plan_destroy(ctx, plan):

@@ -106,3 +106,45 @@ def test_a_plan_made_from_the_kept_configuration_runs_what_the_tuned_plan_runs(j
     assert runs[0] == runs[1] and len(runs[0]) == dsdp.dsdp_plan_kernel_count(plan)
     for p in (plan, again):
         dsdp.dsdp_plan_destroy(None, p)
+
+
+def test_plans_in_flight_share_the_gpu_without_teams(jobs):
+    """The way of a plan's chains goes by all chains under way at its launch: two plans of 8
+    chains per SM each run for long on two streams; a third plan's teams then stay while
+    one of them counts (its own stream's launches come before it) and go with both."""
+    make, stream, _ = jobs
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    torch.cuda.synchronize()
+    side = [torch.cuda.Stream() for _ in range(3)]
+    long_ = [_create(make(8 * sms + k, 0, atoms=30, steps=600), 1) for k in range(2)]
+    ends = [torch.cuda.Event() for _ in long_]
+    small, tiny, other = _create(make(2 * sms, 0)), _create(make(sms, 0)), _create(make(2 * sms, 0))
+    seen = []
+
+    def launch(plan, st):
+        dsdp.dsdp_plan_launch(plan, st.cuda_stream)
+        seen.append(dsdp.dsdp_plan_team(plan))
+
+    assert dsdp.dsdp_plan_team(small) == 0
+    launch(small, side[2])
+    launch(tiny, side[2])
+    torch.cuda.synchronize()
+    assert seen == [4, 8]
+    dsdp.dsdp_plan_launch(long_[0], side[0].cuda_stream)
+    ends[0].record(side[0])
+    launch(tiny, side[2])  # 9 per SM
+    launch(small, side[2])  # 10
+    dsdp.dsdp_plan_launch(long_[1], side[1].cuda_stream)
+    ends[1].record(side[1])
+    launch(small, side[2])  # 18
+    launch(other, side[1])  # 10 to 12 beside its own stream's
+    under_way = not any(e.query() for e in ends)
+    assert captured_kernels(stream, lambda: dsdp.dsdp_plan_launch(small, stream)) == [(2 * sms, 4 * 32)]
+    torch.cuda.synchronize()
+    launch(small, side[2])
+    torch.cuda.synchronize()
+    launch(tiny, side[1])
+    torch.cuda.synchronize()
+    assert under_way and seen[2:] == [4, 4, 1, 4, 4, 8]
+    for p in [*long_, small, tiny, other]:
+        dsdp.dsdp_plan_destroy(None, p)
