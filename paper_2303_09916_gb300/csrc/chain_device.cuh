@@ -657,13 +657,13 @@ struct ChainRecord {
   float e_cur, e_best;
   uint32_t evals;
   uint32_t pad;
-  // [2][7 + T]: the current and the best conformation
-  __device__ __forceinline__ float* conf() { return reinterpret_cast<float*>(this + 1); }
+  // [7 + T]: component k of the current and of the best conformation
+  __device__ __forceinline__ float2* conf() { return reinterpret_cast<float2*>(this + 1); }
 };
 static_assert(sizeof(ChainRecord) == slice_record_bytes(-7), "a record's size");
-__device__ __forceinline__ ChainRecord* chain_record(const DevJob& J, int T, int chain) {
+__device__ __forceinline__ ChainRecord* chain_record(const DevJob& J, int chain) {
   return reinterpret_cast<ChainRecord*>(reinterpret_cast<uint8_t*>(J.chain_coords) +
-                                        (size_t)chain * (sizeof(ChainRecord) + 8 * (7 + T)));
+                                        (size_t)chain * J.record_bytes);
 }
 struct ChainSlice {
   ChainRecord* rec;  // null: the call runs the whole chain
@@ -869,8 +869,9 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
     if (lane < kHStride) Vg[lane] = Vd[lane] = 0.f;
     if (mutate) {
       if (lane < 7 + T) {
-        W.cur[lane] = __ldcg(sl.rec->conf() + lane);
-        W.best[lane] = __ldcg(sl.rec->conf() + 7 + T + lane);
+        const float2 c = __ldcg(sl.rec->conf() + lane);
+        W.cur[lane] = c.x;
+        W.best[lane] = c.y;
       }
       V.e_cur = __ldcg(&sl.rec->e_cur);
       V.e_best = __ldcg(&sl.rec->e_best);
@@ -1017,10 +1018,7 @@ __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& 
       }
       if (step == V.stop) {  // end of this slice: the chain waits in its record
         ChainRecord* const rec = V.rec;
-        if (lane < nx) {
-          __stcg(rec->conf() + lane, W.cur[lane]);
-          __stcg(rec->conf() + nx + lane, W.best[lane]);
-        }
+        if (lane < nx) __stcg(rec->conf() + lane, make_float2(W.cur[lane], W.best[lane]));
         if (lane == 0) {
           __stcg(&rec->e_cur, e_cur);
           __stcg(&rec->e_best, e_best);
@@ -1078,10 +1076,11 @@ __device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W
     xt = draw_start(J, T, chain);
     if (J.trace && J.trace_starts && warp == 0) trace_start(J, chain, xt, T);
   } else {
-    ChainRecord* const rec = chain_record(J, T, chain);
+    ChainRecord* const rec = chain_record(J, chain);
     if (lane < nx) {
-      W.cur[lane] = __ldcg(rec->conf() + lane);
-      W.best[lane] = __ldcg(rec->conf() + nx + lane);
+      const float2 c = __ldcg(rec->conf() + lane);
+      W.cur[lane] = c.x;
+      W.best[lane] = c.y;
     }
     e_cur = __ldcg(&rec->e_cur);
     e_best = __ldcg(&rec->e_best);

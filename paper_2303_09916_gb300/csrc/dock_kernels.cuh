@@ -121,7 +121,7 @@ __device__ __forceinline__ void chain_cta(const DevJob* __restrict__ jobs, const
       const int chain = tile.chain0 + warp;
       ChainSlice sl{nullptr, nullptr, 0};
       if (queue.n_blocks) {
-        sl.rec = chain_record(J, L.T, chain);
+        sl.rec = chain_record(J, chain);
         sl.next_step = queue.next_step + (size_t)t * (blockDim.x >> 5) + warp;
         sl.steps = J.slice_steps;
       }
@@ -159,8 +159,11 @@ __global__ void __launch_bounds__(32 * kMaxChainWarps, ChainOcc<VAR>::kMinBlocks
 // one (64 plain-2k chains 5.9 ms against 6.2), else two, which is 128 registers and
 // four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5).  next_step: the
 // chains that a time-sliced launch left unfinished (ChainQueue), from their records;
-// null: whole chains.
-template <int FMT, int MB>
+// null: whole chains.  APLS as in dock_chains_kernel; two atoms per lane alone run the
+// kernel of both (384 chains of 45 atoms, 20 steps: 6.11 ms; by itself that kernel
+// spills 44 bytes at 128 registers, 6.32), one atom per lane its own (Eq. 3 maps 6.93
+// ms, with both 7.07; Eq. 4 3.24).
+template <int FMT, int MB, int APLS>
 __global__ void __launch_bounds__(32 * kMaxTeam, MB)
     dock_team_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, const int* next_step,
                      int blob_smem, ScratchLayout lay) {
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(32 * kMaxTeam, MB)
   uint8_t* const scratch = smem + blob_smem;
   const WarpScratch W = warp_scratch_at(scratch + (threadIdx.x >> 5) * lay.bytes, lay);
   TeamSlot* const ex = reinterpret_cast<TeamSlot*>(scratch + (blockDim.x >> 5) * lay.bytes);
-  if (L.n_atoms <= 32) run_team<1, FMT>(J, L, W, ex, tile.chain0, first);
+  if (APLS == 1 || (APLS == 3 && L.n_atoms <= 32)) run_team<1, FMT>(J, L, W, ex, tile.chain0, first);
   else run_team<2, FMT>(J, L, W, ex, tile.chain0, first);
 }
 
@@ -257,10 +260,10 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
                             a.n_tiles, q, a.blob_smem, a.scratch);
 }
 
-template <int FMT>
+template <int FMT, int APLS>
 cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
   const size_t smem = (size_t)a.blob_smem + (size_t)a.team * (a.scratch.bytes + 2 * sizeof(TeamSlot));
-  auto k = a.team == kMaxTeam ? dock_team_kernel<FMT, 1> : dock_team_kernel<FMT, 2>;
+  auto k = a.team == kMaxTeam ? dock_team_kernel<FMT, 1, APLS> : dock_team_kernel<FMT, 2, APLS>;
   const cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),
@@ -271,7 +274,7 @@ cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
 
 template <int FMT>
 cudaError_t launch_chains_impl(const ChainLaunch& a, cudaStream_t st) {
-  if (a.team > 1) return launch_team<FMT>(a, st);
+  if (a.team > 1) return a.apl_mask == 1 ? launch_team<FMT, 1>(a, st) : launch_team<FMT, 3>(a, st);
   if (a.warps_per_cta != 1 && a.warps_per_cta != 2 && a.warps_per_cta != kMaxChainWarps) return cudaErrorInvalidValue;
   if (a.apl_mask == 1) {
     switch (a.variant) {

@@ -98,6 +98,7 @@ struct DevJob {
   int32_t n_sites;     // 0: initial positions uniform in the box
   float site_r2;       // site radius squared (FP32)
   int32_t slice_steps;  // MC steps of a slice in a time-sliced launch
+  int32_t record_bytes;  // of a chain's record there (slice_record_bytes)
   float* chain_best_conf;
   float* chain_best_e;
   uint32_t* chain_evals;

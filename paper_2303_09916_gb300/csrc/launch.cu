@@ -660,6 +660,7 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
     d.chain_score = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_inter = (double*)take(sizeof(double) * (size_t)d.n_chains);
     d.chain_intra = (double*)take(sizeof(double) * (size_t)d.n_chains);
+    d.record_bytes = slice_record_bytes(tors[j]);
     d.chain_coords = (double*)take(coord_bytes(d.n_chains, atoms[j], tors[j]));
   }
   cudaError_t e = cudaMemcpy(P->d_jobs, dj.data(), sizeof(DevJob) * n_jobs, cudaMemcpyHostToDevice);
