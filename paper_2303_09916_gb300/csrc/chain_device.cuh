@@ -280,8 +280,8 @@ __device__ __forceinline__ float energy_placed(const MapView& M, const LigView& 
 // step pairs of the one-atom-per-lane intra loop are unrolled.  FLAT: the passes that
 // may hold hydrophobic or H-bond pairs compute both terms for all (with weight 0
 // where a pair has none: the same bits) instead of branching, and are unrolled too --
-// more instructions, a shorter way through them.
-template <int APL, int FMT, int IU = 2, bool FLAT = false>
+// more instructions, a shorter way through them.  RU: how many of those passes.
+template <int APL, int FMT, int IU = 2, bool FLAT = false, int RU = FLAT ? 2 : 1>
 __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L, const LaneLig<APL>& R,
                                               int n_ramp, const WarpScratch& W, const Conf& c, const Placed<APL>& P,
                                               float& grad, uint32_t flags) {
@@ -334,7 +334,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         az = __ffma2_rn(make_float2(c0.z, c1.z), splat2(-1.f), __fadd2_rn(az, fz));
       };
       int st = 0;
-#pragma unroll (FLAT ? 2 : 1)
+#pragma unroll RU
       for (; st < n_ramp; st += 2) pass(st, true);
 #pragma unroll IU
       for (; st < L.n_steps; st += 2) pass(st, false);
@@ -372,7 +372,7 @@ __device__ __forceinline__ float score_placed(const MapView& M, const LigView& L
         else g[0].x -= c1.x, g[0].y -= c1.y, g[0].z -= c1.z;
       };
       int st = 0;
-#pragma unroll (FLAT ? 2 : 1)
+#pragma unroll RU
       for (; st < n_ramp; st += 2) pass(st, true);
 #pragma unroll (FLAT ? 2 : 1)
       for (; st < L.n_steps; st += 2) pass(st, false);

@@ -186,9 +186,14 @@ __global__ void __launch_bounds__(32 * kMaxTeam, MB)
 // Score + gradient of a batch of conformations: one warp per conformation,
 // warps striding over the batch (the ligand is staged once per CTA, while the first
 // conformation is on its way).  FLAT (score_placed): a batch of at most one warp
-// per scheduler, which takes as long as one evaluation does.
+// per scheduler, which takes as long as one evaluation does.  Registers: no spills.
+// FLAT has a CTA per SM and takes up to 128 (600 conformations of 30 / 45 / 64 atoms on
+// FP32 maps 4.6 / 6.8 / 9.4 us, at 80 registers 4.9 / 8.2 / 11.9); of many conformations
+// one atom per lane takes 96, 20 warps per SM (100,003 of 30 atoms 182 us, Eq. 3 maps
+// 166; at 80, 24 warps, 184 and 197) and unrolls the passes with hydrophobic and H-bond
+// pairs too (180 and 164), two take the 80 that they need.
 template <int APL, int FMT, bool FLAT>
-__global__ void __launch_bounds__(128, 6) score_eval_kernel(MapView M, const uint8_t* __restrict__ blob,
+__global__ void __launch_bounds__(128, FLAT ? 4 : APL == 1 ? 5 : 6) score_eval_kernel(MapView M, const uint8_t* __restrict__ blob,
                                                             const float* __restrict__ conf, int n_conf, int T,
                                                             float* __restrict__ energy, float* __restrict__ grad,
                                                             uint32_t flags, int blob_smem, ScratchLayout lay) {
@@ -208,7 +213,7 @@ __global__ void __launch_bounds__(128, 6) score_eval_kernel(MapView M, const uin
     float g;
     Placed<APL> P;
     place_atoms<APL>(L, x, P);
-    const float e = score_placed<APL, FMT, 2, FLAT>(M, L, R, n_ramp, W, x, P, g, flags);
+    const float e = score_placed<APL, FMT, 2, FLAT, FLAT || APL == 1 ? 2 : 1>(M, L, R, n_ramp, W, x, P, g, flags);
     if (lane == 0 && energy) energy[c] = e;
     if (grad && lane < 6 + T) grad[(size_t)c * (6 + T) + lane] = g;
     c += warps;
