@@ -35,11 +35,14 @@ struct alignas(16) SmoothRow {
 struct SmoothTable {
   SmoothRow row[kIntervals];
 };
-// exp(x), -100 < x <= 0: x = n ln 2 + r, Taylor series of exp(r)
+// exp(x), -100 < x <= 0: x = r - n ln 2, Taylor series of exp(r).  ln 2 in two parts, its
+// first 33 binary digits and the rest: n times the first is exact, and so is its sum
+// with x, a multiple of 2^-14 here.
+constexpr double kLn2Head = 5954088943.0 / 8589934592.0, kLn2Rest = 7.44061711001239684737714e-11;
 constexpr double exp_series(double x) {
   int n = 0;
   while (x + n * 0.69314718055994530942 < -0.34657359027997265) ++n;
-  const double r = (x + n * 0.693147180369123816490) + n * 1.90821492927058770002e-10;  // ln 2 in two parts
+  const double r = (x + n * kLn2Head) + n * kLn2Rest;
   double term = 1.0, sum = 0.0;
   double part[26] = {};
   for (int k = 0; k < 26; ++k) {
