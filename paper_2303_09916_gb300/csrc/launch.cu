@@ -27,6 +27,7 @@ struct dsdp_plan {
     int fmt, apl, first_tile, n_tiles, blob_smem, max_atoms, max_torsions, apl_mask;
     int first_block, n_blocks, n_items;  // time-sliced queue (SliceBlock)
     int first_chain, n_chains;           // tiles of one chain each (teams)
+    bool maps_near;                      // (ChainLaunch)
   };
   std::vector<Group> groups;
   void* d_jobs = nullptr;
@@ -58,10 +59,13 @@ struct dsdp_plan {
     int fmt, apl, blob, atoms, torsions, chains;
     double cost;  // length of a chain, relative
     int slices;   // of each of its chains
+    const void* maps;
+    size_t map_bytes;
   };
   std::vector<Shape> shape;
   std::vector<int> job_order;  // jobs by chain length, longest first
   int sms = 148;
+  size_t l2_bytes = 0;
   // The plan's last chain launch, among those of the process's other plans (ChainsInFlight).
   struct Flight {
     cudaEvent_t done = nullptr;  // null: not tracked
@@ -137,14 +141,23 @@ static dsdp_status check_view(const dsdp_grid_view* g) {
   return DSDP_OK;
 }
 
+static int device_attribute(cudaDeviceAttr attr, std::atomic<int>* known) {
+  int dev = 0, v = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && (v = known[dev].load(std::memory_order_relaxed)) > 0) return v;
+  cudaDeviceGetAttribute(&v, attr, dev);
+  if (dev >= 0 && dev < 64) known[dev].store(v, std::memory_order_relaxed);
+  return v;
+}
+
 int device_sms() {
   static std::atomic<int> known[64];
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (dev >= 0 && dev < 64) known[dev].store(sms, std::memory_order_relaxed);
-  return sms;
+  return device_attribute(cudaDevAttrMultiProcessorCount, known);
+}
+
+static size_t device_l2_bytes() {
+  static std::atomic<int> known[64];
+  return (size_t)device_attribute(cudaDevAttrL2CacheSize, known);
 }
 
 // A kernel has one limit per device, which every thread's launches share: it only ever
@@ -267,12 +280,14 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
     int tile, n;
   };
   std::vector<Item> items;
+  std::vector<std::pair<const void*, size_t>> maps;
   for (int f = 0; f < 6; ++f)
     for (int apl = split ? 2 : 0; apl >= (split ? 1 : 0); --apl) {  // 0: both
       dsdp_plan::Group g{};
       g.fmt = f;
       g.first_tile = (int)tiles.size();
       items.clear();
+      maps.clear();
       for (int j : P->job_order) {
         const dsdp_plan::Shape& s = P->shape[j];
         if (s.fmt != f || (apl && s.apl != apl)) continue;
@@ -281,6 +296,7 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
         g.blob_smem = std::max(g.blob_smem, s.blob);
         g.max_atoms = std::max(g.max_atoms, s.atoms);
         g.max_torsions = std::max(g.max_torsions, s.torsions);
+        maps.emplace_back(s.maps, s.map_bytes);
         const int first = (int)tiles.size() - g.first_tile;
         for (int c = 0; c < s.chains; c += W) tiles.push_back(Tile{j, c, std::min(W, s.chains - c), 0});
         const int n = (int)tiles.size() - g.first_tile - first;
@@ -290,6 +306,11 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
       g.first_chain = n_chains;
       for (int t = g.first_tile; t < (int)tiles.size(); ++t) g.n_chains += tiles[t].count;
       n_chains += g.n_chains;
+      std::sort(maps.begin(), maps.end());
+      size_t map_bytes = 0;
+      for (size_t k = 0; k < maps.size(); ++k)
+        if (k + 1 == maps.size() || maps[k].first != maps[k + 1].first) map_bytes += maps[k].second;
+      g.maps_near = map_bytes <= kNearL2s * P->l2_bytes;
       if (!g.n_tiles) continue;
       std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.left > b.left; });
       g.first_block = (int)blocks.size();
@@ -549,6 +570,7 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
   P->flags = flags;
   P->max_chains = max_chains;
   P->sms = ctx_sm_count(ctx);
+  P->l2_bytes = device_l2_bytes();
   size_t total_chains = 0, max_blocks = 0;
   bool all_bfgs = true, any_bfgs = false;
   {
@@ -562,7 +584,9 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
       const BlobHeader* h = (const BlobHeader*)jobs[j].h_blob;
       const double cost = (dj[j].n_steps + 1.0) * (dj[j].optimizer == DSDP_OPT_BB ? 1.6 : 1.0) *
                           (dj[j].n_opt_iters + 1.0) * (14.0 * apl[j] + h->n_steps);
-      P->shape[j] = dsdp_plan::Shape{fmt[j], apl[j], blob_bytes[j], atoms[j], tors[j], dj[j].n_chains, cost, 0};
+      P->shape[j] = dsdp_plan::Shape{fmt[j], apl[j], blob_bytes[j], atoms[j], tors[j], dj[j].n_chains, cost, 0, dj[j].maps,
+                                      (size_t)DSDP_NUM_MAP_TYPES * dj[j].n[0] * dj[j].n[1] * dj[j].n[2] *
+                                          fmt_channels(fmt[j]) * fmt_elem_bytes(fmt[j])};
       longest = std::max(longest, cost);
       total_chains += (size_t)dj[j].n_chains;
     }
@@ -736,6 +760,7 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.warps_per_cta = P->warps_per_cta;
     a.apl = g.apl;
     a.apl_mask = g.apl_mask;
+    a.maps_near = g.maps_near && P->groups.size() == 1;
     a.blob_smem = (g.blob_smem + 15) & ~15;
     a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
     a.overlap = gi > 0 && queue != kNoQueue;

@@ -8,9 +8,13 @@ class _KernelParams(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v2
         ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
 
 
-def captured_kernels(stream, enqueue):
+CARVEOUT = 14  # CU_LAUNCH_ATTRIBUTE_PREFERRED_SHARED_MEMORY_CARVEOUT
+
+
+def captured_kernels(stream, enqueue, attribute=None):
     """[(CTAs, threads of a CTA)] of the kernels that enqueue() launches on `stream` (an
-    address; not the default stream), in the order of the graph's nodes.  Nothing runs."""
+    address; not the default stream), in the order of the graph's nodes; with an
+    attribute (of integer value) its values instead.  Nothing runs."""
     cu = ctypes.CDLL("libcuda.so.1")
 
     def check(status):
@@ -30,6 +34,11 @@ def captured_kernels(stream, enqueue):
         kind = ctypes.c_int()
         check(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
         if kind.value != 0:  # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        if attribute is not None:
+            value = (ctypes.c_int * 16)()  # CUlaunchAttributeValue
+            check(cu.cuGraphKernelNodeGetAttribute(ctypes.c_void_p(node), attribute, ctypes.byref(value)))
+            out.append(value[0])
             continue
         p = _KernelParams()
         check(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
