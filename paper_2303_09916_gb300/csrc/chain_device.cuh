@@ -245,8 +245,9 @@ __device__ __forceinline__ float energy_placed(const MapView& M, const LigView& 
       dy = __ffma2_rn(make_float2(b0.y, b1.y), splat2(-1.f), py);
       dz = __ffma2_rn(make_float2(b0.z, b1.z), splat2(-1.f), pz);
     } else {
-      const float3 a0 = t0.x & (1u << 10) ? P.pos[APL - 1] : P.pos[0], a1 = t1.x & (1u << 10) ? P.pos[APL - 1] : P.pos[0];
-      const float3 s0 = t0.x & (1u << 11) ? P.pos[APL - 1] : P.pos[0], s1 = t1.x & (1u << 11) ? P.pos[APL - 1] : P.pos[0];
+      const float3 lo = P.pos[0], hi = P.pos[APL - 1];
+      const float3 a0 = t0.x & (1u << 10) ? hi : lo, a1 = t1.x & (1u << 10) ? hi : lo;
+      const float3 s0 = t0.x & (1u << 11) ? hi : lo, s1 = t1.x & (1u << 11) ? hi : lo;
       const float3 b0 = shfl3(s0, (int)t0.x), b1 = shfl3(s1, (int)t1.x);
       dx = make_float2(a0.x - b0.x, a1.x - b1.x);
       dy = make_float2(a0.y - b0.y, a1.y - b1.y);
@@ -834,7 +835,8 @@ __device__ __forceinline__ void trace_start(const DevJob& J, int chain, const Co
 // With a record in `sl`, the call runs one slice from the step the chain stands
 // at and leaves it in the record; without, the whole chain.
 // REVIEW: read the ligand's view from the staged blob at each evaluation instead of
-// holding it in registers (the 96-register kernel of mixed tiles spills otherwise).
+// holding it in registers (the 96-register kernels of mixed tiles and of one-channel maps
+// spill otherwise).
 template <int APL, int FMT, int IU = 2, bool REVIEW = false, bool FLAT = false>
 __device__ void run_chain(const DevJob& J, const LigView& L, const WarpScratch& W, int chain, const ChainSlice& sl) {
   enum : int { kStart = 0, kTrial = 1, kBB = 2 };
@@ -1058,9 +1060,9 @@ struct TeamSlot {
 //
 // Bound: latency (a round is one evaluation and one update, 3.2 us; energies first and
 // the winner's gradient after a second barrier: 8 % slower alone and no faster with
-// eight launches at once).  One typical-4k
-// system (384 chains, 2.6 evaluations a round with teams of 4) takes 6.1 ms of chain
-// stage against 12.0, one plain-2k system (64 chains, teams of 8) 6.3 against 14.4.
+// eight launches at once).  One typical-4k system (384 chains, 2.6 evaluations a round
+// with teams of 4) takes 5.9 - 6.2 ms of chain stage against 10.7 - 11.2 with one warp a
+// chain, one plain-2k system (64 chains, teams of 8) 5.8 - 6.2 against 13.1 - 14.1.
 template <int APL, int FMT>
 __device__ void run_team(const DevJob& J, const LigView& L, const WarpScratch& W, TeamSlot* ex, int chain, int first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = blockDim.x >> 5;

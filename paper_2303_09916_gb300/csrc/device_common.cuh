@@ -319,9 +319,12 @@ __device__ __forceinline__ float4 load_node(const void* maps, unsigned idx) {
 // The score of a node alone.
 template <int FMT>
 __device__ __forceinline__ float load_score(const void* maps, unsigned idx) {
-  if (FMT == 0) return __ldg(reinterpret_cast<const float*>(maps) + 4 * (size_t)idx);
-  if (FMT == 1) return __bfloat162float(__ushort_as_bfloat16(__ldg(reinterpret_cast<const unsigned short*>(maps) + 4 * (size_t)idx)));
-  if (FMT == 2) return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(maps) + 4 * (size_t)idx)));
+  const size_t at = 4 * (size_t)idx;
+  if (FMT == 0) return __ldg(reinterpret_cast<const float*>(maps) + at);
+  if (FMT == 1 || FMT == 2) {
+    const unsigned short raw = __ldg(reinterpret_cast<const unsigned short*>(maps) + at);
+    return FMT == 1 ? __bfloat162float(__ushort_as_bfloat16(raw)) : __half2float(__ushort_as_half(raw));
+  }
   return load_node<FMT>(maps, idx).x;
 }
 

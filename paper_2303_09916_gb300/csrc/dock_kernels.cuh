@@ -151,13 +151,15 @@ template <int FMT, int VAR, int APLS>
 __global__ void __launch_bounds__(32 * kMaxChainWarps, ChainOcc<VAR>::kMinBlocks)
     dock_chains_kernel(const DevJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles, ChainQueue queue,
                        int blob_smem, ScratchLayout lay) {
-  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1)), VAR == 0 && APLS == 1>(jobs, tiles, n_tiles, queue, blob_smem, lay);
+  constexpr bool kReview = VAR == 1 && (APLS == 3 || (APLS == 1 && fmt_channels(FMT) == 1));
+  chain_cta<FMT, APLS, APLS == 3 ? 1 : 2, kReview, VAR == 0 && APLS == 1>(jobs, tiles, n_tiles, queue, blob_smem, lay);
 }
 
 // Teams (run_team): CTA b runs tile b, a single chain, with all its warps.  MB: CTAs
 // of kMaxTeam warps the registers must allow per SM; with one chain per SM at most,
-// one (64 plain-2k chains 5.9 ms against 6.2), else two, which is 128 registers and
-// four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5).  next_step: the
+// one (64 plain-2k chains take 5 % less time than with two), else two, which is 128
+// registers and four teams of 4 per SM (384 typical-4k chains 6.1 ms against 7.5 with
+// one).  next_step: the
 // chains that a time-sliced launch left unfinished (ChainQueue), from their records;
 // null: whole chains.  APLS as in dock_chains_kernel; two atoms per lane alone run the
 // kernel of both (384 chains of 45 atoms, 20 steps: 6.11 ms; by itself that kernel
@@ -193,10 +195,10 @@ __global__ void __launch_bounds__(32 * kMaxTeam, MB)
 // 166; at 80, 24 warps, 184 and 197) and unrolls the passes with hydrophobic and H-bond
 // pairs too (180 and 164), two take the 80 that they need.
 template <int APL, int FMT, bool FLAT>
-__global__ void __launch_bounds__(128, FLAT ? 4 : APL == 1 ? 5 : 6) score_eval_kernel(MapView M, const uint8_t* __restrict__ blob,
-                                                            const float* __restrict__ conf, int n_conf, int T,
-                                                            float* __restrict__ energy, float* __restrict__ grad,
-                                                            uint32_t flags, int blob_smem, ScratchLayout lay) {
+__global__ void __launch_bounds__(128, FLAT ? 4 : APL == 1 ? 5 : 6)
+    score_eval_kernel(MapView M, const uint8_t* __restrict__ blob, const float* __restrict__ conf, int n_conf, int T,
+                      float* __restrict__ energy, float* __restrict__ grad, uint32_t flags, int blob_smem,
+                      ScratchLayout lay) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5);
@@ -272,8 +274,8 @@ cudaError_t launch_team(const ChainLaunch& a, cudaStream_t st) {
   const cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   k<<<a.n_tiles, 32 * a.team, smem, st>>>(reinterpret_cast<const DevJob*>(a.jobs),
-                                          reinterpret_cast<const Tile*>(a.tiles), a.team_resumes ? a.next_step : nullptr,
-                                          a.blob_smem, a.scratch);
+                                          reinterpret_cast<const Tile*>(a.tiles),
+                                          a.team_resumes ? a.next_step : nullptr, a.blob_smem, a.scratch);
   return cudaGetLastError();
 }
 

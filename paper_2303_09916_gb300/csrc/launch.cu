@@ -34,7 +34,8 @@ struct dsdp_plan {
   void* d_tiles = nullptr;
   void* d_singles = nullptr;  // room for the same chains in tiles of one; null if teams are never taken
   void* d_rtiles = nullptr;
-  // work queue: [kMaxGroups counters, one per group][kMaxGroups exit counts][tickets per tile][next step per tile and warp]; zeroed by each launch
+  // work queue: [kMaxGroups counters, one per group][kMaxGroups exit counts][tickets per tile]
+  // [next step per tile and warp]; zeroed by each launch
   int* d_queue = nullptr;
   size_t queue_bytes = 0;
   size_t queue_next_off = 0;  // of the next steps, in ints
@@ -250,10 +251,12 @@ static void tune_erase(uint64_t key) {
 
 // Slices of the launch's longest chains when it time-slices (ChainQueue): enough
 // that the last slices are a small part of the launch, few enough that a slice
-// (a few MC steps, hundreds of evaluations) hides its record's load and store.  When
-// all chains have a place at once they seldom move and what counts is how soon the
-// slowest reach the teams: slices of one MC step (1,536 chains as above: 11.6 ms, in
-// 16 slices 12.8).
+// (a few MC steps, hundreds of evaluations) hides its record's load and store.  Up to
+// 16 chains per SM (most or all have a place at once) they seldom move and what counts
+// is how soon the slowest reach the teams: 64 slices, of one MC step for jobs of up to
+// 63 (1,536 chains as above: 11.6 ms, in 16 slices 12.8).  The limit goes by chains and
+// not by the places that shared memory leaves: 2,280 chains of 10-60 atoms 27.8 ms,
+// with their 10 places per SM as the limit 36.9; 2,400 of 60 atoms 38.6 and 39.7.
 constexpr int kSliceRounds = 16, kSliceRoundsResident = 64;
 
 static ChainQueueMode queue_mode(const dsdp_plan* P) {
@@ -332,7 +335,7 @@ constexpr int kTailTeams = 8;
 
 // Warps of a chain (dock_team_kernel) when the plan's chains leave most of the GPU
 // idle; 1 when they do not.  Up to one chain per SM a team of 8 (64 plain-2k chains
-// 6.3 ms against 6.7 in teams of 4; 200 typical-4k chains 2.8 against 2.6), up to 8
+// take 6 % less time than in teams of 4, 200 typical-4k chains 7 % more), up to 8
 // per SM teams of 4 (1,200 chains 6.9 ms, one warp each 8.1; 1,536 chains 9.7 against
 // 8.3): beyond, the trial points that a line search does not come to cost more than
 // the shorter way saves.  Teams are a warp per SM sub-partition or two: 5 and 6 warps
@@ -584,9 +587,10 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
       const BlobHeader* h = (const BlobHeader*)jobs[j].h_blob;
       const double cost = (dj[j].n_steps + 1.0) * (dj[j].optimizer == DSDP_OPT_BB ? 1.6 : 1.0) *
                           (dj[j].n_opt_iters + 1.0) * (14.0 * apl[j] + h->n_steps);
-      P->shape[j] = dsdp_plan::Shape{fmt[j], apl[j], blob_bytes[j], atoms[j], tors[j], dj[j].n_chains, cost, 0, dj[j].maps,
-                                      (size_t)DSDP_NUM_MAP_TYPES * dj[j].n[0] * dj[j].n[1] * dj[j].n[2] *
-                                          fmt_channels(fmt[j]) * fmt_elem_bytes(fmt[j])};
+      const size_t map_bytes = (size_t)DSDP_NUM_MAP_TYPES * dj[j].n[0] * dj[j].n[1] * dj[j].n[2] *
+                               fmt_channels(fmt[j]) * fmt_elem_bytes(fmt[j]);
+      P->shape[j] = dsdp_plan::Shape{fmt[j],  apl[j],         blob_bytes[j], atoms[j], tors[j],
+                                     dj[j].n_chains, cost, 0, dj[j].maps, map_bytes};
       longest = std::max(longest, cost);
       total_chains += (size_t)dj[j].n_chains;
     }
@@ -601,7 +605,8 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
     for (int j = 0; j < n_jobs; ++j) {
       P->job_order[j] = j;
       // slices of about the same length whatever the job
-      const int steps = dj[j].n_steps + 1, want = (int)ceil((P->resident ? kSliceRoundsResident : kSliceRounds) * P->shape[j].cost / longest);
+      const int steps = dj[j].n_steps + 1, rounds = P->resident ? kSliceRoundsResident : kSliceRounds;
+      const int want = (int)ceil(rounds * P->shape[j].cost / longest);
       dj[j].slice_steps = (steps + want - 1) / want;
       P->shape[j].slices = (steps + dj[j].slice_steps - 1) / dj[j].slice_steps;
       max_blocks += P->shape[j].slices;
@@ -653,10 +658,12 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
   for (int j = 0; j < n_jobs; ++j)
     for (int c = 0; c < dj[j].n_chains; c += rw) rtiles.push_back(Tile{j, c, std::min(rw, dj[j].n_chains - c), 0});
   P->n_rtiles = (int)rtiles.size();
-  const size_t b_jobs = up256(sizeof(DevJob) * n_jobs), b_tiles = up256(sizeof(Tile) * total_chains) * (P->automatic.team > 1 ? 2 : 1),
+  const size_t b_jobs = up256(sizeof(DevJob) * n_jobs),
+               b_tiles = up256(sizeof(Tile) * total_chains) * (P->automatic.team > 1 ? 2 : 1),
                b_rtiles = up256(sizeof(Tile) * rtiles.size()), b_blocks = up256(sizeof(SliceBlock) * max_blocks);
   P->queue_next_off = 2 * kMaxGroups + total_chains;
-  P->queue_bytes = sizeof(int) * (2 * kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);  // tiles of W <= 4 may be part filled
+  // (tiles of W <= 4 may be part filled)
+  P->queue_bytes = sizeof(int) * (2 * kMaxGroups + 2 * total_chains + 4 * (size_t)n_jobs);
   const size_t b_cnt = up256(P->queue_bytes);
   P->arena_bytes = b_jobs + b_tiles + b_rtiles + b_blocks + b_cnt + scratch;
   P->arena = ctx_alloc(ctx, P->arena_bytes, nullptr);
@@ -760,7 +767,7 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.warps_per_cta = P->warps_per_cta;
     a.apl = g.apl;
     a.apl_mask = g.apl_mask;
-    a.maps_near = g.maps_near && P->groups.size() == 1;
+    a.maps_near = g.maps_near && P->groups.size() == 1 && !P->resident;
     a.blob_smem = (g.blob_smem + 15) & ~15;
     a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
     a.overlap = gi > 0 && queue != kNoQueue;

@@ -31,7 +31,9 @@ struct ChainLaunch {
   int team_when;      // CTAs left when a time-sliced launch leaves the rest to a team; 0: never
   int apl;            // largest atoms-per-lane tile present
   int apl_mask;       // tiles present: bit 0 one atom per lane (<= 32 atoms), bit 1 two (<= 64)
-  bool maps_near;     // the plan's only launch, its maps together at most kNearL2s times the L2 cache
+  // the plan's only launch, of more than 16 chains per SM, its maps together at most
+  // kNearL2s times the L2 cache
+  bool maps_near;
   int blob_smem;      // bytes reserved for the largest staged blob prefix
   ScratchLayout scratch;  // per-warp scratch, sized for the group's largest ligand
   int variant;        // register budget of the chain kernel (0: 128, 1: 96)
@@ -84,8 +86,9 @@ constexpr int kSmemPerSm = 228 * 1024;
 // receptors 22.2 ms at 73 %, 21.1 at 59, 22.8 at 52, 34.2 at 80; 32 systems of the above
 // 51.7 and 48.6 a launch).  A launch beside another group of its plan asks for 59 %: the
 // larger ligands' chains take the room (64 ligands of 10-60 atoms 63.7 ms, 65.3 at 73 %).
-// Measured for chains of up to 9.2 KB (16 in 164 KB); larger
-// ones keep what the driver gives.  (The split that a percentage stands for is the
+// So does one of up to 16 chains per SM, which need no more (1,024 Barzilai-Borwein
+// chains 6.16 ms, 6.21 at 73 %).  Measured for chains of up to 9.2 KB (16 in 164 KB);
+// larger ones keep what the driver gives.  (The split that a percentage stands for is the
 // driver's and not shown anywhere: 66 % ran like 59, 71 like 73, 87 like 100.)
 constexpr int kChainSmemPerSm = 164 * 1024, kChainSmemWarps = 16;
 constexpr int kChainSmemPercent = 59, kChainSmemPercentNear = 73, kNearL2s = 4;
