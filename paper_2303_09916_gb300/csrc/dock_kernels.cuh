@@ -261,7 +261,7 @@ cudaError_t launch_chains_var(const ChainLaunch& a, cudaStream_t st) {
   }
   if (carve) {
     attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[cfg.numAttrs++].val.sharedMemCarveout = a.maps_near ? kChainSmemPercentNear : kChainSmemPercent;
+    attr[cfg.numAttrs++].val.sharedMemCarveout = a.more_smem ? kChainSmemPercentMore : kChainSmemPercent;
   }
   return cudaLaunchKernelEx(&cfg, k, reinterpret_cast<const DevJob*>(a.jobs), reinterpret_cast<const Tile*>(a.tiles),
                             a.n_tiles, q, a.blob_smem, a.scratch);

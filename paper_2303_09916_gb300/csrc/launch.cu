@@ -27,7 +27,7 @@ struct dsdp_plan {
     int fmt, apl, first_tile, n_tiles, blob_smem, max_atoms, max_torsions, apl_mask;
     int first_block, n_blocks, n_items;  // time-sliced queue (SliceBlock)
     int first_chain, n_chains;           // tiles of one chain each (teams)
-    bool maps_near;                      // (ChainLaunch)
+    bool misses_less;                    // of near maps or Barzilai-Borwein alone (kChainSmemPercent)
   };
   std::vector<Group> groups;
   void* d_jobs = nullptr;
@@ -62,6 +62,7 @@ struct dsdp_plan {
     int slices;   // of each of its chains
     const void* maps;
     size_t map_bytes;
+    bool bfgs;
   };
   std::vector<Shape> shape;
   std::vector<int> job_order;  // jobs by chain length, longest first
@@ -291,6 +292,7 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
       g.first_tile = (int)tiles.size();
       items.clear();
       maps.clear();
+      bool bfgs = false;
       for (int j : P->job_order) {
         const dsdp_plan::Shape& s = P->shape[j];
         if (s.fmt != f || (apl && s.apl != apl)) continue;
@@ -300,6 +302,7 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
         g.max_atoms = std::max(g.max_atoms, s.atoms);
         g.max_torsions = std::max(g.max_torsions, s.torsions);
         maps.emplace_back(s.maps, s.map_bytes);
+        bfgs = bfgs || s.bfgs;
         const int first = (int)tiles.size() - g.first_tile;
         for (int c = 0; c < s.chains; c += W) tiles.push_back(Tile{j, c, std::min(W, s.chains - c), 0});
         const int n = (int)tiles.size() - g.first_tile - first;
@@ -313,7 +316,7 @@ static void plan_tiles(dsdp_plan* P, int W, std::vector<Tile>& tiles, std::vecto
       size_t map_bytes = 0;
       for (size_t k = 0; k < maps.size(); ++k)
         if (k + 1 == maps.size() || maps[k].first != maps[k + 1].first) map_bytes += maps[k].second;
-      g.maps_near = map_bytes <= kNearL2s * P->l2_bytes;
+      g.misses_less = map_bytes <= kNearL2s * P->l2_bytes || !bfgs;
       if (!g.n_tiles) continue;
       std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.left > b.left; });
       g.first_block = (int)blocks.size();
@@ -415,14 +418,16 @@ static size_t chains_in_flight(const dsdp_plan::Flight& own, cudaStream_t st) {
   return sum;
 }
 
-// Warps of a chain of a plan of `chains`, with `others` under way beside them (round of
-// launches of 10 steps, typical-4k, ms with one warp a chain / teams of 4 / of 8): streams
-// x chains 2 x 128 3.7 / 1.94 / 1.80, 4 x 128 4.4 / 2.5 / 2.9, 8 x 128 4.7 / 3.2 / 5.3;
+// Warps of a chain of a plan of `chains` that would take teams of `team` alone (1: it
+// would not), with `others` under way beside them (round of launches of 10 steps,
+// typical-4k, ms with one warp a chain / teams of 4 / of 8): streams x chains 2 x 128
+// 3.7 / 1.94 / 1.80, 4 x 128 4.4 / 2.5 / 2.9, 8 x 128 4.7 / 3.2 / 5.3;
 // 4 x 384 5.1 / 4.1 / 7.9, 5 x 5.0 / 4.8, 6 x 5.7 / 5.7, 7 x 5.6 / 6.8, 8 x 6.5 / 7.5.
 // Two atoms per lane (45): 4 x 128 9.3 / 4.3 / 4.1, 8 x 128 10.1 / 5.4 / 7.7; 8 x 384 10.7
 // in tiles of 4 chains / 12.4.  (One launch alone loses its teams' gain earlier,
 // team_warps: its chains keep step.)
-static int shared_team_warps(size_t chains, size_t others, int apl_max, int sms) {
+static int shared_team_warps(int team, size_t chains, size_t others, int apl_max, int sms) {
+  if (team == 1) return 1;
   const size_t all = chains + others;
   if (chains <= (size_t)sms && all <= (size_t)((apl_max == 2 ? 4 : 2) * sms)) return kMaxTeam;
   return all <= (size_t)((apl_max == 2 ? 18 : 16) * sms) ? 4 : 1;
@@ -589,8 +594,9 @@ dsdp_status dsdp::plan_create(dsdp_ctx* ctx, int n_jobs, const dsdp_job_device* 
                           (dj[j].n_opt_iters + 1.0) * (14.0 * apl[j] + h->n_steps);
       const size_t map_bytes = (size_t)DSDP_NUM_MAP_TYPES * dj[j].n[0] * dj[j].n[1] * dj[j].n[2] *
                                fmt_channels(fmt[j]) * fmt_elem_bytes(fmt[j]);
-      P->shape[j] = dsdp_plan::Shape{fmt[j],  apl[j],         blob_bytes[j], atoms[j], tors[j],
-                                     dj[j].n_chains, cost, 0, dj[j].maps, map_bytes};
+      const bool bfgs = dj[j].optimizer == DSDP_OPT_BFGS;
+      P->shape[j] = dsdp_plan::Shape{fmt[j], apl[j], blob_bytes[j], atoms[j], tors[j], dj[j].n_chains,
+                                     cost,   0,      dj[j].maps,    map_bytes, bfgs};
       longest = std::max(longest, cost);
       total_chains += (size_t)dj[j].n_chains;
     }
@@ -736,14 +742,17 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
   const cudaStream_t st = (cudaStream_t)stream;
   const ChainQueueMode queue = queue_mode(P);
   int team = P->team;
+  const bool lone = !P->ctx && P->groups.size() == 1 && !P->resident;
+  size_t others = 0;  // chains under way on other streams
   bool track = false;
   if (stages & DSDP_STAGE_CHAINS) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(st, &capture);
     if (e != cudaSuccess) cudaGetLastError();
     track = e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
-    if (team > 1 && track && P->flight.done)
-      team = shared_team_warps((size_t)P->flight.chains, chains_in_flight(P->flight, st), P->apl_max, P->sms);
+    if (track && P->flight.done && (team > 1 || (lone && P->groups[0].misses_less)))
+      others = chains_in_flight(P->flight, st);
+    if (others) team = shared_team_warps(team, (size_t)P->flight.chains, others, P->apl_max, P->sms);
     P->last_team = team;
   }
   if ((stages & DSDP_STAGE_CHAINS) && queue != kNoQueue) {
@@ -767,7 +776,7 @@ extern "C" dsdp_status dsdp_plan_launch_stage(dsdp_plan* P, uint32_t stages, voi
     a.warps_per_cta = P->warps_per_cta;
     a.apl = g.apl;
     a.apl_mask = g.apl_mask;
-    a.maps_near = g.maps_near && P->groups.size() == 1 && !P->resident;
+    a.more_smem = g.misses_less && lone && others == 0;
     a.blob_smem = (g.blob_smem + 15) & ~15;
     a.scratch = scratch_layout(g.max_atoms, g.max_torsions);
     a.overlap = gi > 0 && queue != kNoQueue;

@@ -31,9 +31,7 @@ struct ChainLaunch {
   int team_when;      // CTAs left when a time-sliced launch leaves the rest to a team; 0: never
   int apl;            // largest atoms-per-lane tile present
   int apl_mask;       // tiles present: bit 0 one atom per lane (<= 32 atoms), bit 1 two (<= 64)
-  // the plan's only launch, of more than 16 chains per SM, its maps together at most
-  // kNearL2s times the L2 cache
-  bool maps_near;
+  bool more_smem;     // kChainSmemPercentMore
   int blob_smem;      // bytes reserved for the largest staged blob prefix
   ScratchLayout scratch;  // per-warp scratch, sized for the group's largest ligand
   int variant;        // register budget of the chain kernel (0: 128, 1: 96)
@@ -79,19 +77,21 @@ constexpr int kSmemPerSm = 228 * 1024;
 // cells, which successive evaluations of a chain mostly share.  Unasked, the driver
 // leaves an SM that never drains with the split of whichever kernel it ran before: four
 // steps of 32 typical-4k systems in flight, grid builds and rescoring between them, ran
-// 418 systems/s, at 59 % 597 (one at a time 539 and 574).  More room for the corners is
-// the better the more of them come from beyond the L2 cache: of maps of up to 4 times
-// its size 73 % (32 ligands on one FP32 receptor, 20 steps, 25.0 ms, at 59 % 25.6 and at
-// 80 % 27.4; of 12 torsions 26.5, 28.3, 26.5; 6 receptors 20.2, 20.4), of more 59 % (24
-// receptors 22.2 ms at 73 %, 21.1 at 59, 22.8 at 52, 34.2 at 80; 32 systems of the above
-// 51.7 and 48.6 a launch).  A launch beside another group of its plan asks for 59 %: the
-// larger ligands' chains take the room (64 ligands of 10-60 atoms 63.7 ms, 65.3 at 73 %).
-// So does one of up to 16 chains per SM, which need no more (1,024 Barzilai-Borwein
-// chains 6.16 ms, 6.21 at 73 %).  Measured for chains of up to 9.2 KB (16 in 164 KB);
-// larger ones keep what the driver gives.  (The split that a percentage stands for is the
-// driver's and not shown anywhere: 66 % ran like 59, 71 like 73, 87 like 100.)
+// 418 systems/s, at 59 % 597 (one at a time 539 and 574).  59 % is the rule; 73 %
+// (more chains, less cache) for a launch that fills the GPU by itself and misses less:
+//   of maps of up to 4 times the L2 cache (32 ligands on one FP32 receptor, 20 steps,
+//     25.0 ms, at 59 % 25.6 and at 80 % 27.4; of 12 torsions 26.5, 28.3, 26.5; 6 receptors
+//     20.2, 20.4; but 24 receptors 22.2 ms at 73 %, 21.1 at 59, 22.8 at 52, 34.2 at 80);
+//   of Barzilai-Borwein chains alone (32 receptors, 10 steps, 24.1 ms, at 59 % 24.8).
+// Not beside another group of its plan or chains under way on other streams, with which
+// it shares the SMs (64 ligands of 10-60 atoms 63.7 ms, at 73 % 65.3), nor for a context's
+// jobs, whose next batch starts before an SM drains and finds the last one's split
+// (saturated serving 492 requests/s, 478), and not up to 16 chains per SM, which need
+// no more (1,024 Barzilai-Borwein chains 6.16 ms, 6.21).  Measured for chains of up to 9.2 KB (16 in
+// 164 KB); larger ones keep what the driver gives.  (The split that a percentage stands
+// for is the driver's and not shown anywhere: 66 % ran like 59, 71 like 73, 87 like 100.)
 constexpr int kChainSmemPerSm = 164 * 1024, kChainSmemWarps = 16;
-constexpr int kChainSmemPercent = 59, kChainSmemPercentNear = 73, kNearL2s = 4;
+constexpr int kChainSmemPercent = 59, kChainSmemPercentMore = 73, kNearL2s = 4;
 
 MapView map_view_of(const dsdp_grid_view* g);
 cudaError_t launch_rescore(const void* jobs, const void* tiles, int n_tiles, cudaStream_t st);

@@ -13,10 +13,11 @@ from paper_2303_09916_gb300 import dsdp  # noqa: E402
 from graph_nodes import CARVEOUT, captured_kernels  # noqa: E402
 
 
-@pytest.mark.parametrize("n_maps,atoms,percent", [(1, 30, 73), (2, 30, 59), (2, 40, None)])
-def test_split_by_the_size_of_the_maps(n_maps, atoms, percent):
+@pytest.mark.parametrize("n_maps,atoms,optimizer,percent", [(1, 30, 0, 73), (2, 30, 0, 59), (2, 30, 1, 73), (2, 40, 0, None)])
+def test_split_by_the_size_of_the_maps(n_maps, atoms, optimizer, percent):
     """Maps of 432 MB each (nothing is launched on them): one is below 4 times the L2 cache,
-    two are above; ligands of more than 32 atoms do not ask."""
+    two are above, which the optimiser without a line search does not mind; ligands of more
+    than 32 atoms do not ask."""
     l2 = torch.cuda.get_device_properties(0).L2_cache_size
     assert 432e6 <= 4 * l2 < 864e6
     buf = torch.zeros(64, device="cuda")
@@ -28,7 +29,7 @@ def test_split_by_the_size_of_the_maps(n_maps, atoms, percent):
         j = dsdp.dsdp_job_device()
         j.grid = dsdp.grid_view(buf.data_ptr() + 16 * (k % n_maps), [150] * 3, [0.0] * 3, 0.375)
         j.h_blob, j.d_blob = blob.ctypes.data, d_blob.data_ptr()
-        j.params = dsdp.make_params(n_chains=1000, n_mc_steps=4, seed=k)
+        j.params = dsdp.make_params(n_chains=1000, n_mc_steps=4, seed=k, optimizer=optimizer)
         for a in range(3):
             j.box_size[a] = 10.0
         jobs.append(j)
