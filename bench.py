@@ -1337,7 +1337,9 @@ def main():
     achieved_tflops = r["flops"] / per_launch_s / 1e12
     sm_mhz = peaks.get("sm_max_mhz", 2070.0)
     peak_tflops = fp32_peak_tflops(sm_mhz)
-    capture = chain_kernel_capture(args.batch, args.map_dtype, describe_tile_config(r["tile_config"]))
+    # the automatic arrangement of a plan of this size runs the 96-register kernel with the queue
+    # (14) and teams for its slowest chains
+    capture = chain_kernel_capture(args.batch, args.map_dtype, describe_tile_config(r["tile_config"] or 14))
     line = {
         "metric": "docked systems/s (typical-4k: 4k-atom receptor, 80^3 maps, 30-atom ligand, 384x40 MC+BFGS)",
         "value": value, "unit": "systems/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
